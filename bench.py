@@ -57,11 +57,10 @@ def kernels_per_step(global_index):
     """Kernels one route+commit launches.  Route: class parameters, prologue, leaders, hash,
     caps, the block-0 probe (one kernel with the global index; with per-instance tables three:
     claim of the distinct block-0 keys, their probes, the per-request expansion), probe search,
-    the four of the selection (records, initial envelopes, per-class selection, joint
-    selection: it returns at once unless the per-class path hands it the batch), finalize.
+    the two of the selection (records, deferred acceptance), finalize.
     Commit: insert dedup, insert work list, insert, the global-index pass (global layout only),
     sessions, and the five eviction kernels (estimate, collect, select, delete, shift)."""
-    return (12 + 9 + 1) if global_index else (14 + 9)
+    return (10 + 9 + 1) if global_index else (12 + 9)
 
 
 def max_over_ranks(ms, dist, device):
@@ -107,9 +106,8 @@ COMMIT_PHASES = ("insert", "gix_insert", "sessions", "evict")
 
 HASH_SOURCES = ("paper_2608_11152_gb300/csrc/hash.cu", "paper_2608_11152_gb300/csrc/common.cuh")
 HASH_PROFILE = os.path.join(ROOT, "profiles", "k1_block_hash_stress_n65536.md")
-SELECT_SOURCES = ("paper_2608_11152_gb300/csrc/select.cu", "paper_2608_11152_gb300/csrc/envelope.cuh",
-                  "paper_2608_11152_gb300/csrc/common.cuh")
-SELECT_PROFILE = os.path.join(ROOT, "profiles", "k4_select_class_stress_n65536.md")
+SELECT_SOURCES = ("paper_2608_11152_gb300/csrc/select.cu", "paper_2608_11152_gb300/csrc/common.cuh")
+SELECT_PROFILE = os.path.join(ROOT, "profiles", "k4_select_stress_n65536.md")
 
 
 def hash_sources_sha256(files=HASH_SOURCES):
@@ -150,7 +148,7 @@ def profiled_hash_fields():
 
 
 def profiled_select_traffic(n, instances):
-    """DRAM bytes per launch of the per-class selection from its committed ncu summary, when
+    """DRAM bytes per launch of the selection kernel from its committed ncu summary, when
     that capture's workload is this one (the stress batch at 128 instances), else None."""
     f = profiled_fields(SELECT_PROFILE, SELECT_SOURCES)
     if not f or int(f["batch_requests"]) != int(n) or int(f["instances"]) != int(instances):
@@ -364,8 +362,8 @@ def algorithmic_bytes(sc, st, mask_words=None, admitted_blocks=0, evict_buckets=
     ops = admitted_blocks if insert_ops is None else insert_ops
     return {
         "hash": hash_b, "probe_first": first_b, "probe_search": search_b, "n_blocks": n_blocks,
-        # K3b/K4a selection: one 32-byte record per request read, the decision fields written
-        "select": 32 * b.n + 10 * b.n,
+        # K3b/K4a selection: one 64-byte record per request read, the decision fields written
+        "select": 64 * b.n + 10 * b.n,
         # K4b insert: per key operation, its key read (8 B), its home key group (32 B) and the
         # read-modify-write of its meta (16 B); per new key its (key, instance) entry (16 B);
         # per block left to a later request, its key and the later request's key compared (16 B)
@@ -669,7 +667,7 @@ def run_gb300(args):
     # one kernel per phase below (the insert phase adds the small work-list kernel)
     KERNEL_NAMES = {"hash": "k1_block_hash",
                     "probe_first": "k2_probe_first_gix" if gidx else "k2_first_claim + k2_probe_distinct + k2_probe_first_gix",
-                    "probe_search": "k2_probe_search", "select": "k4_select_class", "insert": "k4_insert",
+                    "probe_search": "k2_probe_search", "select": "k4_select", "insert": "k4_insert",
                     "gix_insert": "k4_gix_insert", "evict_collect": "k4_evict_collect",
                     "evict_delete": "k4_evict_delete", "evict_shift": "k4_evict_shift"}
 
@@ -693,15 +691,15 @@ def run_gb300(args):
     if kernels["select"] is not None:
         if args.config == 5:
             kernels["select"]["traffic"] = profiled_select_traffic(sc.batch.n, sc.W)
-        kernels["select"]["limiter"] = ("one CTA per class walks its leaders in arrival order; bound by the "
-                                        "chain of headroom-exhaustion events (barrier-separated steps), not by memory")
+        kernels["select"]["limiter"] = ("deferred acceptance on one cluster of 16 CTAs; bound by the instruction "
+                                        "latency of its barrier-separated rounds, not by memory")
     # dominant kernel: the largest time per launch
     dom = max((k for k in kernels if kernels[k]), key=lambda k: kernels[k]["ms_per_launch"])
     dom_roof = dict(kernels[dom])
     if dom == "hash" and dom_roof.get("traffic") is not None:
         dom_roof["traffic_source"] = "profiles/k1_block_hash_stress_n65536.md (ncu dram__bytes_read.sum + dram__bytes_write.sum)"
     if dom == "select" and dom_roof.get("traffic") is not None:
-        dom_roof["traffic_source"] = "profiles/k4_select_class_stress_n65536.md (ncu dram__bytes_read.sum + dram__bytes_write.sum)"
+        dom_roof["traffic_source"] = "profiles/k4_select_stress_n65536.md (ncu dram__bytes_read.sum + dram__bytes_write.sum)"
 
     clocks = sampler.summary()
     line = {

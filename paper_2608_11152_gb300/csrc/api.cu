@@ -11,7 +11,6 @@
 #include <vector>
 
 #include "common.cuh"
-#include "envelope.cuh"
 #include "kernels.h"
 
 using namespace misat;
@@ -129,20 +128,15 @@ struct misat_ctx {
   int64_t hits_cap = 0;
   unsigned long long* d_bm_key = nullptr;
   int32_t* d_bm_val = nullptr;
-  int4* d_sel_rec = nullptr;     // per-request records of the selection
-  uint8_t* d_onhull = nullptr;   // initial envelopes of the selection [3W]
-  int32_t* d_rank = nullptr;     // slope order of the instances [W]
-  int32_t* d_rank_a = nullptr;   // (d_w, w) order of the instances [W]
-  int32_t* d_sel_list = nullptr; // [3 max_batch] each class's leaders per block of 256 requests
-  int32_t* d_sel_cnt = nullptr;  // [3 * blocks] leaders per class and block
-  int32_t* d_sel_x = nullptr;    // [W + 2] admissions per instance, ticket, coupled flag
+  int4* d_sel_rec = nullptr;     // leader records of the selection, compact per block of 256 requests
+  int32_t* d_sel_cnt = nullptr;  // [blocks] leaders per block
+  uint16_t* d_orders = nullptr;  // [kPriceCells][W] price orders
+  int select_cluster = 8;        // largest cluster of the selection kernel
   ulonglong2* d_grp = nullptr;   // (first key, instance) groups of a route's admitted requests
   GIndex fb{};                   // per-instance layout: batch-local index of the distinct block-0 keys
   int32_t* d_fb_list = nullptr;  // [max_batch] its claimed slots
   uint32_t grp_log2 = 1;
   int32_t* d_skip = nullptr;     // [max_batch] leading blocks a later request of the group inserts
-  // every d_w and every 1/mu_w below 2^25: the selection's envelope arithmetic fits in 64 bits
-  bool bk_small = true, tc_small = true;
   int32_t* d_chain_max = nullptr;  // per-chain insert limits of misat_load_chains
   // one small block of counters, mirrored to pinned host memory
   MetaLayout ml;
@@ -602,6 +596,9 @@ CapsArgs caps_args(misat_ctx* c) {
   ca.mode = c->mode;
   ca.contraction = c->d_contraction;
   ca.ia = c->ia;
+  ca.backlog = c->d_backlog;
+  ca.tokcost = c->d_tokcost;
+  ca.orders = c->d_orders;
   ca.err = c->err_ptr();
   return ca;
 }
@@ -690,67 +687,30 @@ void enqueue_route(misat_ctx* c, const misat_batch* b, misat_decisions* out, cud
   sp.W = c->W;
   sp.rq = c->rq;
   sp.H = c->d_H;
+  sp.backlog = c->d_backlog;
+  sp.tokcost = c->d_tokcost;
+  sp.gh = c->ia.gh;
+  sp.ch = c->ia.ch;
+  sp.hold_delay_q = c->hold_delay_q;
   sp.rec = c->d_sel_rec;
-  sp.adm = c->d_sel_x;
-  sp.ticket = reinterpret_cast<unsigned*>(c->d_sel_x + c->W);
-  sp.coupled = c->d_sel_x + c->W + 1;
-  sp.seg = c->d_sel_list;
   sp.segcnt = c->d_sel_cnt;
   sp.err = c->err_ptr();
   launch_select_prep(sp, st);
-  EnvInitArgs ei{};
-  ei.W = c->W;
-  ei.backlog = c->d_backlog;
-  ei.tokcost = c->d_tokcost;
-  ei.gh = c->ia.gh;
-  ei.ch = c->ia.ch;
-  ei.onhull = c->d_onhull;
-  ei.rank = c->d_rank;
-  ei.rank_a = c->d_rank_a;
-  ei.small = c->bk_small && c->tc_small;
-  ei.err = c->err_ptr();
-  launch_env_init(ei, st);
-  SelectClassArgs sc{};
-  sc.n = n;
-  sc.W = c->W;
-  sc.rec = c->d_sel_rec;
-  sc.rq = c->rq;
-  sc.gh = c->ia.gh;
-  sc.ch = c->ia.ch;
-  sc.backlog = c->d_backlog;
-  sc.tokcost = c->d_tokcost;
-  sc.onhull = c->d_onhull;
-  sc.rank = c->d_rank;
-  sc.rank_a = c->d_rank_a;
-  sc.H = c->d_H;
-  sc.hold_delay_q = c->hold_delay_q;
-  sc.small = c->bk_small && c->tc_small;
-  sc.seg = c->d_sel_list;
-  sc.segcnt = c->d_sel_cnt;
-  sc.adm = c->d_sel_x;
-  sc.ticket = reinterpret_cast<unsigned*>(c->d_sel_x + c->W);
-  sc.coupled = c->d_sel_x + c->W + 1;
-  sc.stats = c->stats_ptr();
-  sc.err = c->err_ptr();
-  launch_select_class(sc, st);
   SelectArgs sa{};
   sa.n = n;
   sa.W = c->W;
   sa.rec = c->d_sel_rec;
+  sa.segcnt = c->d_sel_cnt;
   sa.rq = c->rq;
   sa.gh = c->ia.gh;
   sa.ch = c->ia.ch;
   sa.backlog = c->d_backlog;
   sa.tokcost = c->d_tokcost;
-  sa.onhull = c->d_onhull;
-  sa.rank = c->d_rank;
-  sa.rank_a = c->d_rank_a;
-  sa.small = c->bk_small && c->tc_small;
+  sa.orders = c->d_orders;
   sa.H = c->d_H;
-  sa.hold_delay_q = c->hold_delay_q;
-  sa.coupled = c->d_sel_x + c->W + 1;
+  sa.stats = c->stats_ptr();
   sa.err = c->err_ptr();
-  launch_select(sa, st);
+  launch_select(sa, c->select_cluster, st);
   c->mark(6, st);
 
   FinalizeArgs fa{};
@@ -864,7 +824,7 @@ int misat_create(const misat_config* cfg, void* cuda_stream, misat_ctx** out) {
   if (cudaGetDevice(&c->device) != cudaSuccess) return fail(MISAT_ERR_CUDA);
   if (cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess)
     return fail(MISAT_ERR_CUDA);
-  if (select_configure() != cudaSuccess || select_class_configure() != cudaSuccess) return fail(MISAT_ERR_CUDA);
+  if (select_configure(&c->select_cluster) != cudaSuccess) return fail(MISAT_ERR_CUDA);
   c->stream = (cudaStream_t)cuda_stream;
   c->W = W;
   c->cap.assign(cfg->cap_blocks, cfg->cap_blocks + W);
@@ -903,13 +863,11 @@ int misat_create(const misat_config* cfg, void* cuda_stream, misat_ctx** out) {
   const int bm_log2 = std::max(1, ceil_log2(2 * NB));
   if ((rc = dalloc_n(c, &c->d_meta, c->ml.words)) || (rc = dalloc_n(c, &c->d_keys, (size_t)c->keys_cap)) ||
       (rc = dalloc_n(c, &c->d_units, 2 * (size_t)c->units_cap)) || (rc = dalloc_n(c, &c->d_units_n, 1)) ||
-      (rc = dalloc_n(c, &c->d_H, NB * Ws)) || (rc = dalloc_n(c, &c->d_hits, (size_t)c->hits_cap)) ||
+      (rc = dalloc_n(c, &c->d_H, NB * Ws + 8)) || (rc = dalloc_n(c, &c->d_hits, (size_t)c->hits_cap)) ||
       (rc = dalloc_n(c, &c->d_bm_key, (size_t)1 << bm_log2)) ||
-      (rc = dalloc_n(c, &c->d_bm_val, (size_t)1 << bm_log2)) || (rc = dalloc_n(c, &c->d_sel_rec, 2 * NB)) ||
-      (rc = dalloc_n(c, &c->d_onhull, 3 * Ws)) || (rc = dalloc_n(c, &c->d_rank, Ws)) ||
-      (rc = dalloc_n(c, &c->d_rank_a, Ws)) || (rc = dalloc_n(c, &c->d_sel_list, 3 * NB)) ||
-      (rc = dalloc_n(c, &c->d_sel_cnt, 3 * ((NB + 255) / 256))) ||
-      (rc = dalloc_n(c, &c->d_sel_x, Ws + 2)) || (rc = dalloc_n(c, &c->d_skip, NB)) ||
+      (rc = dalloc_n(c, &c->d_bm_val, (size_t)1 << bm_log2)) || (rc = dalloc_n(c, &c->d_sel_rec, kSelectRecInt4 * NB)) ||
+      (rc = dalloc_n(c, &c->d_sel_cnt, (NB + 255) / 256)) ||
+      (rc = dalloc_n(c, &c->d_orders, (size_t)kPriceCells * price_order_stride(W))) || (rc = dalloc_n(c, &c->d_skip, NB)) ||
       (rc = dalloc_n(c, &c->d_grp, (size_t)1 << bm_log2)) ||
       (rc = dalloc_n(c, &c->rq.nb, NB)) || (rc = dalloc_n(c, &c->rq.kbase, NB)) || (rc = dalloc_n(c, &c->rq.L, NB)) ||
       (rc = dalloc_n(c, &c->rq.cls, NB)) || (rc = dalloc_n(c, &c->rq.session, NB)) ||
@@ -997,13 +955,6 @@ int misat_set_instance_state(misat_ctx* c, const int64_t* backlog_q, const int64
     if (tokcost_q && (tokcost_q[w] < 0 || tokcost_q[w] > ((int64_t)1 << 32))) return MISAT_ERR_INVALID_ARG;
     if (cap_contraction && cap_contraction[w] < 0) return MISAT_ERR_INVALID_ARG;
   }
-  auto below = [&](const int64_t* v) {
-    for (int w = 0; w < c->W; ++w)
-      if (v[w] >= kEnvSmall) return false;
-    return true;
-  };
-  if (backlog_q) c->bk_small = below(backlog_q);
-  if (tokcost_q) c->tc_small = below(tokcost_q);
   if (backlog_q) CK(cudaMemcpyAsync(c->d_backlog, backlog_q, c->W * 8, cudaMemcpyHostToDevice, c->stream));
   if (tokcost_q) CK(cudaMemcpyAsync(c->d_tokcost, tokcost_q, c->W * 8, cudaMemcpyHostToDevice, c->stream));
   if (cap_contraction)
@@ -1060,8 +1011,7 @@ int misat_route(misat_ctx* c, const misat_batch* b, misat_decisions* out) {
                                   (uint64_t)c->sess.log2n,
                                   reinterpret_cast<uint64_t>(c->gix.keys),
                                   reinterpret_cast<uint64_t>(c->gix.masks),
-                                  (uint64_t)c->gix.log2nb,
-                                  (uint64_t)(c->bk_small && c->tc_small)};
+                                  (uint64_t)c->gix.log2nb};
   if (c->timing) {
     // phase events bracket the kernels directly (events recorded inside a graph do not time)
     enqueue_route(c, b, out, st);

@@ -114,9 +114,12 @@ struct CapsArgs {
   int32_t mode;
   const int32_t* contraction;  // [W]
   InstArrays ia;
+  const int64_t* backlog;      // [W] d_w
+  const int64_t* tokcost;      // [W] 1/mu_w
+  uint16_t* orders;            // [kPriceCells][stride] out: price orders of the selection
   const int32_t* err;
 };
-void launch_caps(const CapsArgs& a, cudaStream_t st);
+void launch_caps(const CapsArgs& a, cudaStream_t st);  // caps and price orders
 // Writes the host's per-route class parameters (footprints, residencies, mixture) to the
 // device (kernel arguments are taken at launch, so the host array may change right after).
 struct RouteParams {
@@ -125,88 +128,60 @@ struct RouteParams {
 void launch_route_params(const RouteParams& p, int64_t* dst, cudaStream_t st);
 
 // ---- serial selection (select.cu) ----
-constexpr int kSelectThreads = 512;        // leaders per window of the joint selection CTA
-constexpr int kSelectClassThreads = 512;   // leaders per window of a per-class selection CTA
+// Grid of prompt lengths whose price orders are kept: exact below 16 tokens, then 16 steps per
+// octave (prompts are below 2^20 tokens).
+constexpr int kPriceCells = 272;
+__host__ __device__ __forceinline__ int64_t price_cell_start(int cell) {
+  return cell < 16 ? cell : (int64_t)(16 + (cell & 15)) << ((cell >> 4) - 1);
+}
+__device__ __forceinline__ int price_cell(uint32_t x) {
+  if (x < 16) return (int)x;
+  const int e = 27 - __clz(x);  // x >> e is in [16, 32)
+  return ((e + 1) << 4) + (int)((x >> e) & 15);
+}
+// Entries of a price order's row: W rounded up to whole 16-byte pieces.
+__host__ __device__ __forceinline__ int price_order_stride(int W) { return (W + 7) & ~7; }
+// A price order's entry: the instance, and whether it is cheaper than every entry behind it
+// over the whole cell.
+constexpr uint32_t kPriceMask = 0x7fff, kPriceFast = 0x8000;
+constexpr int kSelectRecInt4 = 4;  // int4 per leader record
 
 struct SelectPrepArgs {
   int32_t n;
   int32_t W;
   ReqArrays rq;
-  const uint16_t* H;
-  int4* rec;                   // [2n] per-request records of the selection
-  int32_t* adm;                // [W] zeroed here: admissions per instance of the per-class path
-  unsigned* ticket;            // zeroed here
-  int32_t* coupled;            // zeroed here
-  int32_t* seg;                // [3n] out: per class and block of 256 requests, its leaders in order
-  int32_t* segcnt;             // [3 * blocks] out: leaders per class and block
+  const uint16_t* H;           // [n*W], readable 16 bytes past its end
+  const int64_t* backlog;      // [W] d_w
+  const int64_t* tokcost;      // [W] 1/mu_w
+  const int32_t* gh;           // [W] global headroom at batch start
+  const int32_t* ch;           // [W*3] class headroom at batch start
+  int64_t hold_delay_q;
+  int4* rec;                   // out: leader records, compact per block of 256 requests
+  int32_t* segcnt;             // [blocks] out: leaders per block
   const int32_t* err;
 };
 void launch_select_prep(const SelectPrepArgs& a, cudaStream_t st);
 
-struct EnvInitArgs {
-  int32_t W;
-  const int64_t* backlog;      // [W] d_w
-  const int64_t* tokcost;      // [W] 1/mu_w
-  const int32_t* gh;           // [W] global headroom at batch start
-  const int32_t* ch;           // [W*3] class headroom at batch start
-  uint8_t* onhull;             // [3*W] out: line w on the lower envelope of class b's instances
-  int32_t* rank;               // [W] out: position of line w in slope order
-  int32_t* rank_a;             // [W] out: position of line w in (d_w, w) order
-  bool small;                  // every d_w and 1/mu_w below 2^25: 64-bit envelope arithmetic
-  const int32_t* err;
-};
-void launch_env_init(const EnvInitArgs& a, cudaStream_t st);
-
 struct SelectArgs {
   int32_t n;
   int32_t W;
-  const int4* rec;             // [2n] from launch_select_prep
+  const int4* rec;             // from launch_select_prep
+  const int32_t* segcnt;       // [blocks] from launch_select_prep
   ReqArrays rq;                // out: status, inst, reason, last_reason of every leader
   const int32_t* gh;           // [W] global headroom at batch start
   const int32_t* ch;           // [W*3] class headroom at batch start
   const int64_t* backlog;      // [W] d_w
   const int64_t* tokcost;      // [W] 1/mu_w
-  const uint8_t* onhull;       // [3*W] initial envelopes (launch_env_init)
-  const int32_t* rank;         // [W] slope order (launch_env_init)
-  const int32_t* rank_a;       // [W] (d_w, w) order (launch_env_init)
-  const uint16_t* H;           // [n*W]
-  int64_t hold_delay_q;
-  bool small;                  // as EnvInitArgs::small
-  const int32_t* coupled;      // the joint selection runs only when the per-class path set this
+  const uint16_t* orders;      // [kPriceCells][stride] price orders (caps kernel)
+  const uint16_t* H;           // [n*W], readable 16 bytes past its end
+  unsigned long long* stats;   // route stats block: [25] = 1 when an instance runs out of global headroom
   int32_t* err;
 };
-size_t select_smem_bytes(int W);
-cudaError_t select_configure();  // per device, before the first launch: shared memory of the selection CTA
-void launch_select(const SelectArgs& a, cudaStream_t st);
-
-// Per-class selection (one CTA per class), valid while no instance runs out of global
-// headroom; otherwise it sets *coupled and launch_select decides the batch.
-struct SelectClassArgs {
-  int32_t n;
-  int32_t W;
-  const int4* rec;             // [2n] from launch_select_prep
-  ReqArrays rq;                // out: status, inst, reason, last_reason of every leader
-  const int32_t* gh;           // [W] global headroom at batch start
-  const int32_t* ch;           // [W*3] class headroom at batch start
-  const int64_t* backlog;      // [W] d_w
-  const int64_t* tokcost;      // [W] 1/mu_w
-  const uint8_t* onhull;       // [3*W] initial envelopes (launch_env_init)
-  const int32_t* rank;         // [W] slope order (launch_env_init)
-  const int32_t* rank_a;       // [W] (d_w, w) order (launch_env_init)
-  const uint16_t* H;           // [n*W]
-  int64_t hold_delay_q;
-  bool small;                  // as EnvInitArgs::small
-  const int32_t* seg;          // [3n] per class and block of 256 requests, its leaders (prep)
-  const int32_t* segcnt;       // [3 * blocks] leaders per class and block (prep)
-  int32_t* adm;                // [W] zeroed by launch_select_prep
-  unsigned* ticket;            // zeroed by launch_select_prep
-  int32_t* coupled;            // zeroed by launch_select_prep; set when the joint kernel must run
-  unsigned long long* stats;   // route stats block: [25] = 1 when the joint kernel runs
-  int32_t* err;
-};
-size_t select_class_smem_bytes(int W, int n);
-cudaError_t select_class_configure();
-void launch_select_class(const SelectClassArgs& a, cudaStream_t st);
+// per device, before the first launch; the largest cluster the selection may use
+cudaError_t select_configure(int* max_cluster);
+void launch_select(const SelectArgs& a, int max_cluster, cudaStream_t st);
+// CTAs that sort the price orders in the caps kernel's launch
+int price_order_blocks(int W);
 
 struct FinalizeArgs {
   int32_t n;

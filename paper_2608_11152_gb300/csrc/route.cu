@@ -116,9 +116,106 @@ void launch_prologue(const PrologueArgs& a, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------
-// K3a caps, one thread per instance (Sec. 4.1; Eqs. 9-10 MISA; Eqs. 11, 13 MISA-T).
+// Price orders.  Prompts of similar length rank the instances alike: for a grid of prompt
+// lengths x_g (16 steps per octave), the instances sorted by (d_w + x_g / mu_w, w).  A leader
+// of length x in [x_g, x_{g+1}) walks the order of x_g: the cost at x of everything behind
+// position k is at least cost_k(x_g) + (x - x_g) min 1/mu, so the walk ends a few entries after
+// the first instance with headroom; an entry that is cheaper than all behind it at both ends of
+// the cell is marked, and ends the walk.  Bitonic sort of 2048 / P grid cells per CTA (P = W rounded
+// up to a power of two), one compare-exchange per thread and stage: latency of 28 barrier
+// steps at W = 128 (2 us), run by extra CTAs of the caps kernel's launch, which takes longer.
+__device__ void sort_price_orders(const int64_t* backlog, const int64_t* tokcost, int W, int blk, uint16_t* orders) {
+  __shared__ int64_t s_c[2048];
+  __shared__ uint16_t s_w[2048];
+  const int tid = threadIdx.x;
+  int P = 2;
+  while (P < W) P <<= 1;
+  const int cell0 = blk * (2048 / P);
+  for (int e = tid; e < 2048; e += blockDim.x) {
+    const int w = e & (P - 1), cell = cell0 + e / P;
+    s_c[e] = w < W && cell < kPriceCells ? backlog[w] + (int64_t)price_cell_start(cell) * tokcost[w] : INT64_MAX;
+    s_w[e] = (uint16_t)w;
+  }
+  for (int k = 2; k <= P; k <<= 1)
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      __syncthreads();
+      const int lo = ((tid & ~(j - 1)) << 1) | (tid & (j - 1)), hi = lo | j;
+      const int64_t a = s_c[lo], b = s_c[hi];
+      const uint16_t u = s_w[lo], v = s_w[hi];
+      const bool after = a > b || (a == b && u > v);
+      const bool up = ((lo & (P - 1)) & k) == 0;
+      if (after == up) {
+        s_c[lo] = b;
+        s_c[hi] = a;
+        s_w[lo] = v;
+        s_w[hi] = u;
+      }
+    }
+  __syncthreads();
+  // fast entries: the cost at the cell's end is below that of every later entry (costs are
+  // linear in x); suffix minima of (cost at the end, w) by doubling
+  int64_t mine[2], sm[2];
+  uint16_t who[2], sw[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int e = tid + 1024 * u, cell = cell0 + e / P;
+    who[u] = s_w[e];
+    mine[u] = who[u] < W && cell < kPriceCells ? backlog[who[u]] + (price_cell_start(cell + 1) - 1) * tokcost[who[u]] : INT64_MAX;
+    sm[u] = mine[u];
+    sw[u] = who[u];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < 2; ++u) s_c[tid + 1024 * u] = mine[u];
+  for (int j = 1; j < P; j <<= 1) {
+    __syncthreads();
+    int64_t oc[2];
+    uint16_t ow[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int e = tid + 1024 * u;
+      const bool in = (e & (P - 1)) + j < P;
+      oc[u] = in ? s_c[e + j] : INT64_MAX;
+      ow[u] = in ? s_w[e + j] : (uint16_t)0xffff;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int e = tid + 1024 * u;
+      if (oc[u] < sm[u] || (oc[u] == sm[u] && ow[u] < sw[u])) {
+        sm[u] = oc[u];
+        sw[u] = ow[u];
+        s_c[e] = sm[u];
+        s_w[e] = sw[u];
+      }
+    }
+  }
+  const int stride = price_order_stride(W);
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int e = tid + 1024 * u;
+    const int k = e & (P - 1), cell = cell0 + e / P;
+    // its own (cost, w) is the minimum of its suffix
+    if (k < W && cell < kPriceCells)
+      orders[(size_t)cell * stride + k] = (uint16_t)(who[u] | (sw[u] == who[u] ? kPriceFast : 0));
+  }
+}
+
+int price_order_blocks(int W) {
+  int P = 2;
+  while (P < W) P <<= 1;
+  return (kPriceCells * P + 2047) / 2048;
+}
+
+// ---------------------------------------------------------------------------
+// K3a caps, one thread per instance (Sec. 4.1; Eqs. 9-10 MISA; Eqs. 11, 13 MISA-T) in the first
+// CTA; the other CTAs sort the selection's price orders.
 __global__ void __launch_bounds__(1024) k3_caps(CapsArgs a) {
   if (block_error(a.err)) return;
+  if (blockIdx.x > 0) {
+    sort_price_orders(a.backlog, a.tokcost, a.W, blockIdx.x - 1, a.orders);
+    return;
+  }
   int64_t kbar_b[3], T_b[3];
   uint32_t rho[3];
 #pragma unroll
@@ -185,7 +282,9 @@ __global__ void __launch_bounds__(1024) k3_caps(CapsArgs a) {
   }
 }
 
-void launch_caps(const CapsArgs& a, cudaStream_t st) { k3_caps<<<1, 1024, 0, st>>>(a); }
+void launch_caps(const CapsArgs& a, cudaStream_t st) {
+  k3_caps<<<1 + price_order_blocks(a.W), 1024, 0, st>>>(a);
+}
 
 __global__ void k_route_params(RouteParams p, int64_t* dst) {
   if (threadIdx.x < 9) dst[threadIdx.x] = p.v[threadIdx.x];

@@ -7,140 +7,128 @@
 // headroom), or is held when no instance has headroom for it; a released continuation may
 // prefer to wait for its cached instance (Eq. 7).
 //
-// The decisions form a serial chain, but the state that a leader's choice depends on
-// changes only when an instance runs out of headroom (at most 4 W times per batch).
-// Between such events every leader's choice is independent of the others', so one CTA
-// takes the batch in windows of kSelectThreads leaders (one per thread):
-//   1. every undecided leader of the window chooses against the state at the window's
-//      current start: for a cold prompt (nothing cached) the cheapest instance with
-//      headroom for its class is a query of the lower envelope of the lines
-//      d_w + L / mu_w (envelope.cuh), plus its few cached or protected instances;
-//   2. the admissions are counted per (instance, class); where an instance would be
-//      over-subscribed, arrival-order ranks (warp counts, one scan over the warps) find the
-//      first leader whose instance has no headroom left at its turn;
-//   3. the leaders before that one are final (their instance still had headroom, and every
-//      other instance only lost headroom, so the argmin stands); instances that ran out leave
-//      the envelopes of the classes they no longer admit, and the window continues from
-//      that leader.
-// Released continuations with a cached prefix (Eq. 7 compares two instances) are decided
-// only at the head of the window, where the state is exactly that of their turn.
+// This serial policy is a serial dictatorship with capacities, and its outcome is the unique
+// stable matching of the leaders (who rank instances by cost, ties to the lower index) and
+// the instances (which all rank leaders by arrival, under a class and a global quota).  It is
+// therefore found by deferred acceptance (Gale & Shapley 1962) instead of one leader after
+// the other: every undecided leader proposes to the cheapest instance that has not
+// refused it, every instance keeps the earliest proposers its quotas admit, and the refused
+// ones propose again until nobody is refused.  In terms of thresholds: te[b][w] is the
+// arrival position of the proposer that takes instance w's last headroom for class b (infinite
+// while some is left); a leader at position i may choose w exactly when i < te[b][w], and
+// thresholds only fall, so a choice stays right until its threshold passes it.  After r
+// rounds the r earliest events (an instance running out) are exact, so there are at most
+// 4 W + 1 rounds, and a round takes in every event whose proposers are already settled: 15
+// to 70 rounds for batches in which the serial chain has 100 to 500 events.
+//
+// Eq. (7) breaks the scheme in one way: a released continuation that proposes to w while
+// its cached instance w_hit has headroom may have to wait instead once w_hit is full, which
+// gives w's headroom back.  Everything before such a leader is unaffected, so when the
+// rounds have settled, the first one found so is fixed as held, the thresholds at or behind it
+// are lifted, and the leaders behind it propose again.  (A leader that waits and then sees
+// the instance it would have waited against fill up is not an exception: waiting takes
+// nothing, it simply proposes later.)
 #include "common.cuh"
-#include "envelope.cuh"
 #include "kernels.h"
 
 namespace misat {
 
 namespace {
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kNT = kSelectThreads;
-constexpr int kNW = kNT / 32;
-constexpr int kMaxGaps = 32;   // envelope gaps handled incrementally per update
-constexpr int kSlotInst = kNT / (4 * kNW);  // over-subscribed instances given exact ranks per pass
-static_assert(kNW == 16 && kSlotInst == 8, "one thread per (counter, warp) in the rank scan");
+constexpr int kNever = 0x7fff;       // threshold of an instance with headroom left (positions are below 2^14)
+constexpr int kRecInt4 = kSelectRecInt4;
+constexpr int kTop = 8;              // cached instances kept per leader, cheapest first
+
+// A choice that is not an instance.
+constexpr int kNone = -1;            // no instance has headroom
+constexpr int kWait = -2;            // Eq. (7): waiting for the cached instance is cheaper
+constexpr int kFixed = -3;           // the same, decided for good
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// Per-request records for the selection (32 bytes, one coalesced pair of loads):
-//   rec[2r]   = {L, cls | sst << 8 | leader << 16, protected / last instance, hbest}
-//   rec[2r+1] = {instances with H > 0, first two of them as (w << 16 | H), 0}
+// Per-leader records of the selection (64 bytes), compact per block of 256 requests:
+//   [0] = {L, class | state << 8, protected / last instance, hbest}
+//   [1] = {cached instances the leader may use, request, theta low, theta high}
+//   [2], [3] = the kTop cheapest of those, (w << 16 | H), by (cost, w)
+// theta is Eq. (7)'s bound: the released leader waits for a full w_hit when the chosen
+// instance's d_w is above theta.  H rows are read 16 bytes at a time, and only of leaders with
+// a cached prefix (one entry at a time took 0.13 ms at 3,001 requests of 1,000 instances).
 __global__ void __launch_bounds__(256) k3_select_prep(SelectPrepArgs a) {
-  __shared__ int s_wc[3][8];
-  if (blockIdx.x == 0) {
-    for (int w = threadIdx.x; w < a.W; w += blockDim.x) a.adm[w] = 0;
-    if (threadIdx.x == 0) {
-      *a.ticket = 0;
-      *a.coupled = 0;
-    }
-  }
+  __shared__ int s_wc[8];
   if (block_error(a.err)) return;
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  // this block's leaders of each class, in arrival order, for the per-class selection
-  {
-    const int c = r < a.n && a.rq.status[r] == kStUnresolved ? a.rq.cls[r] : 3;
-    unsigned mine = 0;
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const unsigned m = __ballot_sync(kFull, c == b);
-      if (lane == 0) s_wc[b][wid] = __popc(m);
-      if (c == b) mine = m;
-    }
-    __syncthreads();
-    if (c < 3) {
-      int off = __popc(mine & lanemask_lt());
-      for (int k = 0; k < wid; ++k) off += s_wc[c][k];
-      a.seg[(int64_t)c * a.n + blockIdx.x * 256 + off] = r;
-    }
-    if (threadIdx.x < 3) {
-      int t = 0;
-      for (int k = 0; k < 8; ++k) t += s_wc[threadIdx.x][k];
-      a.segcnt[threadIdx.x * gridDim.x + blockIdx.x] = t;
-    }
+  const bool lead = r < a.n && a.rq.status[r] == kStUnresolved;
+  const unsigned ml = __ballot_sync(kFull, lead);
+  if (lane == 0) s_wc[wid] = __popc(ml);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int t = 0;
+    for (int k = 0; k < 8; ++k) t += s_wc[k];
+    a.segcnt[blockIdx.x] = t;
   }
-  if (r >= a.n) return;
-  const int lead = a.rq.status[r] == kStUnresolved;
+  if (!lead) return;
+  int off = __popc(ml & lanemask_lt());
+  for (int k = 0; k < wid; ++k) off += s_wc[k];
+  const int64_t x = a.rq.L[r];
+  const int b = a.rq.cls[r], sst = a.rq.sst[r], sinst = a.rq.sinst[r];
+  const int pw = sst == (int)kSessProtected ? sinst : -1;
   const uint32_t hb = a.rq.hbest[r];
   int nh = 0;
-  uint32_t h0 = 0, h1 = 0;
-  if (lead && (hb >> 16) > 0) {
+  int64_t theta = INT64_MAX;
+  int64_t cost[kTop];
+  uint32_t ent[kTop];
+#pragma unroll
+  for (int i = 0; i < kTop; ++i) {
+    cost[i] = INT64_MAX;
+    ent[i] = 0;
+  }
+  if (hb >> 16) {
+    if (sst == (int)kSessReleased) {
+      const int hmax = (int)(hb >> 16), whit = 65535 - (int)(hb & 0xffffu);
+      theta = a.hold_delay_q + a.backlog[whit] - 16 * (int64_t)hmax * a.tokcost[whit];
+    }
+    // the row's entries in 16-byte pieces (its first and last piece may hold neighbours)
     const uint16_t* row = a.H + (int64_t)r * a.W;
-    for (int w = 0; w < a.W; ++w) {
-      const uint32_t h = row[w];
-      if (h) {
-        if (nh == 0) h0 = ((uint32_t)w << 16) | h;
-        else if (nh == 1) h1 = ((uint32_t)w << 16) | h;
+    const int lead_in = (int)((reinterpret_cast<uintptr_t>(row) & 15) >> 1);
+    const uint4* p = reinterpret_cast<const uint4*>(row - lead_in);
+    const int pieces = (lead_in + a.W + 7) >> 3;
+    for (int q = 0; q < pieces; ++q) {
+      const uint4 v = __ldg(p + q);
+      if ((v.x | v.y | v.z | v.w) == 0) continue;
+      const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const uint32_t h = (u[e >> 1] >> (16 * (e & 1))) & 0xffffu;
+        const int w = 8 * q + e - lead_in;
+        if (!h || w < 0 || w >= a.W) continue;
+        if (w != pw && (a.gh[w] <= 0 || a.ch[w * 3 + b] <= 0)) continue;
         ++nh;
+        const int64_t c = a.backlog[w] + (x - 16 * (int64_t)h) * a.tokcost[w];
+        if (c < cost[kTop - 1]) {  // instances come in index order: equal costs keep it
+          cost[kTop - 1] = c;
+          ent[kTop - 1] = ((uint32_t)w << 16) | h;
+#pragma unroll
+          for (int i = kTop - 1; i > 0; --i)
+            if (cost[i] < cost[i - 1]) {
+              const int64_t tcost = cost[i];
+              cost[i] = cost[i - 1];
+              cost[i - 1] = tcost;
+              const uint32_t te = ent[i];
+              ent[i] = ent[i - 1];
+              ent[i - 1] = te;
+            }
+        }
       }
     }
   }
-  a.rec[2 * r] = make_int4(a.rq.L[r], a.rq.cls[r] | (a.rq.sst[r] << 8) | (lead << 16), a.rq.sinst[r], (int)hb);
-  a.rec[2 * r + 1] = make_int4(nh, (int)h0, (int)h1, 0);
-}
-
-// ---------------------------------------------------------------------------
-// Initial envelopes and orders.  blockIdx.y = class b (0..2): is line i on the lower envelope
-// of the instances with headroom for class b?  blockIdx.y = 3: position of line i in slope
-// order; 4: its position in (d_w, w) order.  Eight lanes share line i, each taking every
-// eighth other line.
-__global__ void __launch_bounds__(1024) k3_env_init(EnvInitArgs a) {
-  if (block_error(a.err)) return;
-  const int i = blockIdx.x * 128 + (threadIdx.x >> 3);
-  const int sub = threadIdx.x & 7;
-  const int b = blockIdx.y;
-  const bool line = i < a.W;
-  const int64_t bki = line ? a.backlog[i] : 0, tci = line ? a.tokcost[i] : 0;
-  if (b >= 3) {  // 3: position in slope order; 4: position in (d_w, w) order
-    int cnt = 0;
-    if (line)
-      for (int j = sub; j < a.W; j += 8) {
-        const int64_t bkj = a.backlog[j];
-        if (j != i && (b == 3 ? env_slope_before(bkj, a.tokcost[j], j, bki, tci, i) : (bkj < bki || (bkj == bki && j < i))))
-          ++cnt;
-      }
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) cnt += __shfl_xor_sync(kFull, cnt, o);
-    if (line && sub == 0) (b == 3 ? a.rank : a.rank_a)[i] = cnt;
-    return;
+  int4* rec = a.rec + (int64_t)kRecInt4 * (blockIdx.x * 256 + off);
+  rec[0] = make_int4((int)x, b | (sst << 8), sinst, (int)hb);
+  rec[1] = make_int4(nh, r, (int)(uint32_t)theta, (int)(theta >> 32));
+  if (nh > 0) {
+    rec[2] = make_int4((int)ent[0], (int)ent[1], (int)ent[2], (int)ent[3]);
+    rec[3] = make_int4((int)ent[4], (int)ent[5], (int)ent[6], (int)ent[7]);
   }
-  auto avail = [&](int w) { return a.gh[w] > 0 && a.ch[w * 3 + b] > 0; };
-  const bool ai = line && avail(i);
-  EnvTest t;
-  env_test_init(t);
-  if (ai)
-    for (int j = sub; j < a.W; j += 8)
-      if (j != i && avail(j)) env_test_add(t, bki, tci, i, a.backlog[j], a.tokcost[j], j, a.small);
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) {
-    EnvTest u;
-    u.lo = EnvFrac{__shfl_xor_sync(kFull, t.lo.dbk, o), __shfl_xor_sync(kFull, t.lo.dw, o),
-                   __shfl_xor_sync(kFull, t.lo.dtc, o)};
-    u.hi = EnvFrac{__shfl_xor_sync(kFull, t.hi.dbk, o), __shfl_xor_sync(kFull, t.hi.dw, o),
-                   __shfl_xor_sync(kFull, t.hi.dtc, o)};
-    u.has_hi = __shfl_xor_sync(kFull, t.has_hi, o);
-    u.dominated = __shfl_xor_sync(kFull, t.dominated, o);
-    env_test_merge(t, u, a.small);
-  }
-  if (line && sub == 0) a.onhull[b * a.W + i] = ai && env_test_on(t, a.small) ? 1 : 0;
 }
 
 void launch_select_prep(const SelectPrepArgs& a, cudaStream_t st) {
@@ -148,1244 +136,745 @@ void launch_select_prep(const SelectPrepArgs& a, cudaStream_t st) {
   k3_select_prep<<<(a.n + 255) / 256, 256, 0, st>>>(a);
 }
 
-void launch_env_init(const EnvInitArgs& a, cudaStream_t st) {
-  dim3 grid((a.W + 127) / 128, 5);
-  k3_env_init<<<grid, 1024, 0, st>>>(a);
-}
-
 // ---------------------------------------------------------------------------
-// Shared state of the selection CTA.  Per class, the headroom flags are kept both by instance
-// (queries) and in slope order (envelope updates read them as contiguous bytes); the envelope
-// keeps its lines' d_w and 1/mu_w beside their indices, so a query step is one load level.
-struct SelSmem {
-  int64_t* bk;     // [W] d_w
-  int64_t* tc;     // [W] 1/mu_w
-  int64_t* hbk;    // [3][W] d_w of the envelope lines
-  int64_t* htc;    // [3][W] 1/mu_w of the envelope lines
-  int32_t* gh;     // [W] global headroom
-  int32_t* ch;     // [3][W] class headroom
-  int32_t* T;      // [W] admissions of the window's current choices
-  int32_t* Tb;     // [3][W]
-  int32_t* slot;   // [W] exact-rank slot of an over-subscribed instance, -1
-  int32_t* wc;     // [4 * kSlotInst counters][kNW warps]
-  int32_t* surv;   // [3][W] envelope candidates of each class's update
-  int16_t* ord;    // [W] instances in slope order
-  int16_t* pos;    // [W] position in slope order
-  int16_t* aord;   // [W] instances in (d_w, w) order
-  int16_t* hull;   // [3][W] envelope lines per class, slope order
-  uint8_t* av;     // [3][W] headroom for the class (gh > 0 and ch > 0), by instance
-  uint8_t* avp;    // [3][W] the same by slope position
-  uint8_t* onp;    // [3][W] on the envelope of the class, by slope position
-};
+// The selection kernel: one thread-block cluster takes the leaders in windows of one leader
+// per thread (up to 16 CTAs x 1024).  A leader's position in the window is its thread's rank
+// in the cluster.  Every CTA keeps a copy of the thresholds and the proposals of its own
+// leaders (one bit per instance and thread, and their number per class; a refused proposal's
+// bit stays, it lies behind its threshold for good).  A round:
+//   1. leaders without a standing proposal are packed into as few warps as hold them, choose
+//      and set their bits;                                                  cluster barrier
+//   2. the warp that owns instance w adds up w's proposals per class over the CTAs (distributed
+//      shared memory).  Where a quota is reached by new ones, a scan over the CTAs' numbers and
+//      one over the words of the CTA it ends in give the new threshold, which is written into
+//      every CTA;                                                           cluster barrier
+//   3. leaders whose proposal lies behind its threshold are refused.
+// What bounds it: the instruction latency of one warp through steps 1 and 2 (about 1,000 and
+// 1,500 cycles) and the barriers (500 to 700 cycles each); the SMs are mostly idle.
+namespace {
 
-// Per-class scratch of an envelope update (one warp per class).  headroom only shrinks, so
-// the first line with headroom in (d_w, w) order (the one that wins at x = 0) and the last in
-// slope order (the least 1/mu_w) are found by pointers that only move forward.
-struct EnvScratch {
-  int gp[kMaxGaps];
-  int gq[kMaxGaps];
-  int first_a;     // position in (d_w, w) order of the first line that may have headroom
-  int last_s;      // position in slope order of the last line that may have headroom
-};
-
-// Rebuild hull[b] from the on-envelope flags (compaction in slope order).  One warp.
-__device__ void env_compact_warp(const SelSmem& s, int W, int b, int* hm) {
-  const int lane = threadIdx.x & 31;
-  int base = 0;
-  for (int x0 = 0; x0 < W; x0 += 128) {
-    bool f[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int x = x0 + 32 * u + lane;
-      f[u] = x < W && s.onp[b * W + x];
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int x = x0 + 32 * u + lane;
-      const unsigned m = __ballot_sync(kFull, f[u]);
-      if (f[u]) {
-        const int k = base + __popc(m & lanemask_lt());
-        const int w = s.ord[x];
-        s.hull[b * W + k] = (int16_t)w;
-        s.hbk[b * W + k] = s.bk[w];
-        s.htc[b * W + k] = s.tc[w];
-      }
-      base += __popc(m);
-    }
-  }
-  if (lane == 0) *hm = base;
-  __syncwarp();
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
 }
-
-// The line of class b with headroom that wins at x = 0 (least (d_w, w)), -1 if none.  One warp
-// (warp-uniform result).
-__device__ __forceinline__ int env_first_line(const SelSmem& s, int W, int b, EnvScratch& sc) {
-  int k = sc.first_a;
-  while (k < W && !s.av[b * W + s.aord[k]]) ++k;
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0) sc.first_a = k;
-  __syncwarp();
-  return k < W ? s.aord[k] : -1;
+__device__ __forceinline__ uint32_t ld_cluster(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
 }
-
-// The line of class b with headroom that wins for large x: least 1/mu_w, then least d_w (the
-// first of the last run of equal slopes in slope order), -1 if none.  One warp.
-__device__ __forceinline__ int env_last_line(const SelSmem& s, int W, int b, EnvScratch& sc) {
-  int x = sc.last_s;
-  while (x >= 0 && !s.avp[b * W + x]) --x;
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0) sc.last_s = x;
-  __syncwarp();
-  if (x < 0) return -1;
-  const int64_t t = s.tc[s.ord[x]];
-  int y = x;
-  for (int z = x - 1; z >= 0 && s.tc[s.ord[z]] == t; --z)
-    if (s.avp[b * W + z]) y = z;
-  return s.ord[y];
+__device__ __forceinline__ void st_cluster(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-
-// Remove the lines of class b that lost their headroom from its envelope.  One warp.
-// Each maximal run of removed envelope lines leaves a gap between its surviving neighbours p
-// and q (slope order).  A gap at the start of the envelope is closed by the line that now
-// wins at x = 0 (least d_w: it is on the envelope), one at the end by the line that now wins
-// for large x (least 1/mu_w).  Between p and q the envelope is that of p, q and the lines of
-// slope strictly between them that lie below the chord p-q: a line above it cannot be on the
-// envelope there, and does not change the envelope of the ones below it.
-__device__ void env_update_warp(const SelSmem& s, int W, int b, int* hm, EnvScratch& sc, bool small) {
-  const int lane = threadIdx.x & 31;
-  const int m = *hm;
-  const int16_t* hull = s.hull + b * W;
-  int ng = 0;
-  // gaps, in hull order
-  for (int k0 = 0; k0 < m; k0 += 32) {
-    const int k = k0 + lane;
-    const int w = k < m ? hull[k] : 0;
-    const bool del = k < m && !s.av[b * W + w];
-    const unsigned md = __ballot_sync(kFull, del);
-    const bool prev_del = lane > 0 ? (md >> (lane - 1)) & 1 : (k > 0 && !s.av[b * W + hull[k - 1]]);
-    const bool start = del && !prev_del;
-    if (del) s.onp[b * W + s.pos[w]] = 0;
-    const unsigned ms = __ballot_sync(kFull, start);
-    if (start) {
-      int c = k + 1;
-      while (c < m && !s.av[b * W + hull[c]]) ++c;
-      const int g = ng + __popc(ms & lanemask_lt());
-      if (g < kMaxGaps) {
-        sc.gp[g] = k > 0 ? hull[k - 1] : -1;
-        sc.gq[g] = c < m ? hull[c] : -1;
-      }
-    }
-    ng += __popc(ms);
-  }
-  __syncwarp();
-  if (ng > kMaxGaps) {
-    // full rebuild: every line with headroom tested against all the others
-    for (int x = lane; x < W; x += 32) {
-      bool on = false;
-      if (s.avp[b * W + x]) {
-        const int i = s.ord[x];
-        EnvTest t;
-        env_test_init(t);
-        for (int j = 0; j < W; ++j)
-          if (j != i && s.av[b * W + j]) env_test_add(t, s.bk[i], s.tc[i], i, s.bk[j], s.tc[j], j, small);
-        on = env_test_on(t, small);
-      }
-      s.onp[b * W + x] = on;
-    }
-    __syncwarp();
+__device__ __forceinline__ void st_cluster_u16(uint32_t addr, int v) {
+  asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(addr), "h"((unsigned short)v) : "memory");
+}
+// Barrier over all threads of the cluster (a plain block barrier for one CTA).
+__device__ __forceinline__ void cluster_barrier(int cs) {
+  if (cs == 1) {
+    __syncthreads();
   } else {
-    int ns = 0;
-    int* surv = s.surv + b * W;
-    for (int g = 0; g < ng; ++g) {
-      int p = sc.gp[g], q = sc.gq[g];
-      if (p < 0) {  // the envelope's start was removed: the line that now wins at x = 0
-        p = env_first_line(s, W, b, sc);
-        if (p >= 0 && lane == 0) s.onp[b * W + s.pos[p]] = 1;
-      }
-      if (p >= 0 && q < 0) {  // the end was removed: the line that now wins for large x
-        q = env_last_line(s, W, b, sc);
-        if (lane == 0) s.onp[b * W + s.pos[q]] = 1;
-      }
-      if (p < 0 || q < 0 || p == q) continue;
-      const int g0 = ns;
-      const int xp = s.pos[p], xq = s.pos[q];
-      const int64_t bkp = s.bk[p], tcp = s.tc[p], bkq = s.bk[q], tcq = s.tc[q];
-      for (int x0 = xp + 1; x0 < xq; x0 += 128) {
-        bool c[4];
-        int iv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int x = x0 + 32 * u + lane;
-          c[u] = false;
-          iv[u] = 0;
-          if (x < xq && s.avp[b * W + x]) {
-            const int i = s.ord[x];
-            const int64_t tci = s.tc[i];
-            iv[u] = i;
-            c[u] = tci != tcp && env_below_chord(s.bk[i], tci, i, bkp, tcp, p, bkq, tcq, q, small);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const unsigned mc = __ballot_sync(kFull, c[u]);
-          if (c[u]) surv[ns + __popc(mc & lanemask_lt())] = iv[u];
-          ns += __popc(mc);
-        }
-      }
-      __syncwarp();
-      // each candidate against p, q and the other candidates of this gap
-      for (int e = g0 + lane; e < ns; e += 32) {
-        const int i = surv[e];
-        const int64_t bki = s.bk[i], tci = s.tc[i];
-        EnvTest t;
-        env_test_init(t);
-        env_test_add(t, bki, tci, i, bkp, tcp, p, small);
-        env_test_add(t, bki, tci, i, bkq, tcq, q, small);
-        for (int f = g0; f < ns; ++f) {
-          const int j = surv[f];
-          if (j != i) env_test_add(t, bki, tci, i, s.bk[j], s.tc[j], j, small);
-        }
-        if (env_test_on(t, small)) s.onp[b * W + s.pos[i]] = 1;
-      }
-      __syncwarp();
-    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
-  env_compact_warp(s, W, b, hm);
 }
 
-// Decision of one leader against the current state (see the file comment).  Returns the
-// instance (or -1) and sets *dec to MISAT_ADMIT_NEW, MISAT_ADMIT_CONT, MISAT_HOLD_PREFER_CACHE,
-// MISAT_HOLD_CLASS_CAP or MISAT_HOLD_GLOBAL_CAP.
-__device__ __forceinline__ int sel_choose(const SelSmem& s, const int* s_hm, int W, int nglobal, int L, int b,
-                                          int sst, int pw, uint32_t hb, int nh, uint32_t h0, uint32_t h1,
-                                          const uint16_t* Hrow, int64_t hold, uint8_t* dec) {
-  int64_t best_c = INT64_MAX;
-  int best_w = INT32_MAX;
-  const int m = s_hm[b];
-  const int16_t* hull = s.hull + b * W;
-  const int64_t* hbk = s.hbk + b * W;
-  const int64_t* htc = s.htc + b * W;
-  const int64_t x = L;
-  if (m > 0) {
-    int lo = 0, hi = m - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      const int64_t cu = hbk[mid] + x * htc[mid], cv = hbk[mid + 1] + x * htc[mid + 1];
-      // line mid + 1 beats line mid at x (ties to the lower index)
-      if (cv < cu || (cv == cu && hull[mid + 1] < hull[mid])) lo = mid + 1;
-      else hi = mid;
-    }
-    best_w = hull[lo];
-    best_c = hbk[lo] + x * htc[lo];
+// Bits of word q (positions 32q .. 32q + 31) at or before position t.
+__device__ __forceinline__ unsigned upto_mask(int q, int t) {
+  const int k = t - 32 * q;
+  return k >= 31 ? ~0u : (k < 0 ? 0u : (2u << k) - 1u);
+}
+
+__device__ __forceinline__ int warp_scan(int v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(kFull, v, o);
+    if (lane >= o) v += u;
   }
-  auto consider = [&](int w, int64_t h) {
-    const int64_t c = s.bk[w] + (x - 16 * h) * s.tc[w];
+  return v;
+}
+
+// Inclusive scans of two registers over the warp, side by side.
+__device__ __forceinline__ void warp_scan_pair(unsigned* a, unsigned* b) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned u = __shfl_up_sync(kFull, *a, o), v = __shfl_up_sync(kFull, *b, o);
+    if (lane >= o) {
+      *a += u;
+      *b += v;
+    }
+  }
+}
+
+struct SelSmem {
+  longlong2* ln;   // [W] {d_w, 1/mu_w}
+  unsigned* prop;  // [W][warps] proposals of this CTA's leaders, one bit per thread
+  unsigned* n01;   // [W] their number: class 0 | class 1 << 16
+  unsigned* n2;    // [W] class 2
+  int16_t* te;     // [3][W] position of the proposer that takes the class's last headroom, kNever
+  int16_t* tg;     // [W] position of the proposer that takes the last global headroom, kNever
+  // of the instances this CTA owns (w mod CTAs = its rank), by w / CTAs:
+  int4* hr;        // headroom left: classes 0..2, global
+  unsigned* seen;  // proposals when its thresholds were last computed
+  unsigned* cm;    // [3][words] the window's leaders of each class, one bit per position
+  int* pre;        // [blocks] leaders before each block of 256 requests
+  // per leader of the CTA's part of the window
+  uint32_t* lx;    // prompt tokens | class << 20 | (Eq. 7 may apply) << 22
+  uint32_t* lpos;  // price cell | (its order before this position has no headroom for the leader) << 16
+  uint32_t* lcp;   // protected instance + 1 | cached instances passed over << 16
+  int32_t* lrec;   // record
+  int16_t* lch;    // choice: an instance, kNone, kWait or kFixed
+  uint16_t* queue; // leaders that choose in this round
+  // copies that spare the rounds their global loads (the barriers' acquire drops L1); NULL
+  // when they do not fit, and the originals are read
+  uint4* ord;      // [kPriceCells][stride] price orders
+  uint32_t* list;  // [kTop][threads] the leaders' cached instances
+  int4* eq7;       // [threads] Eq. (7): {w_hit, -, theta low, theta high}
+};
+constexpr size_t kSelSmemMax = 226 * 1024;
+
+__host__ __device__ inline size_t sel_smem_layout(int W, int cs, int warps, int nblk, SelSmem* s, unsigned char* p) {
+  size_t o = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = o;
+    o += (bytes + 15) & ~(size_t)15;
+    return at;
+  };
+  const size_t own = (size_t)((W + cs - 1) / cs) * 16;
+  const size_t ln = take((size_t)W * 16), prop = take((size_t)W * warps * 4), n01 = take((size_t)W * 4),
+               n2 = take((size_t)W * 4), te = take((size_t)W * 6), tg = take((size_t)W * 2), hr = take(own),
+               seen = take(own / 4), cm = take((size_t)cs * warps * 12), pre = take((size_t)nblk * 4),
+               lx = take((size_t)warps * 128), lpos = take((size_t)warps * 128), lcp = take((size_t)warps * 128),
+               lrec = take((size_t)warps * 128), lch = take((size_t)warps * 64), queue = take((size_t)warps * 64);
+  const size_t base = o;
+  const size_t ord = take((size_t)kPriceCells * price_order_stride(W) * 2), list = take((size_t)kTop * warps * 128),
+               eq7 = take((size_t)warps * 512);
+  const bool copies = o <= kSelSmemMax;
+  if (s) {
+    s->ln = reinterpret_cast<longlong2*>(p + ln);
+    s->prop = reinterpret_cast<unsigned*>(p + prop);
+    s->n01 = reinterpret_cast<unsigned*>(p + n01);
+    s->n2 = reinterpret_cast<unsigned*>(p + n2);
+    s->te = reinterpret_cast<int16_t*>(p + te);
+    s->tg = reinterpret_cast<int16_t*>(p + tg);
+    s->hr = reinterpret_cast<int4*>(p + hr);
+    s->seen = reinterpret_cast<unsigned*>(p + seen);
+    s->cm = reinterpret_cast<unsigned*>(p + cm);
+    s->pre = reinterpret_cast<int*>(p + pre);
+    s->lx = reinterpret_cast<uint32_t*>(p + lx);
+    s->lpos = reinterpret_cast<uint32_t*>(p + lpos);
+    s->lcp = reinterpret_cast<uint32_t*>(p + lcp);
+    s->lrec = reinterpret_cast<int32_t*>(p + lrec);
+    s->lch = reinterpret_cast<int16_t*>(p + lch);
+    s->queue = reinterpret_cast<uint16_t*>(p + queue);
+    s->ord = copies ? reinterpret_cast<uint4*>(p + ord) : nullptr;
+    s->list = copies ? reinterpret_cast<uint32_t*>(p + list) : nullptr;
+    s->eq7 = copies ? reinterpret_cast<int4*>(p + eq7) : nullptr;
+  }
+  return copies ? o : base;
+}
+
+// The choice of the CTA's leader t at window position pos given the thresholds: an instance,
+// kNone or kWait.
+__device__ __forceinline__ int sel_choose(const SelSmem& s, const SelectArgs& a, int64_t tc_min, int T, int t, int pos) {
+  const int W = a.W;
+  const uint32_t lx = s.lx[t], lcell = s.lpos[t], lcp = s.lcp[t];
+  const int64_t x = lx & 0xfffffu;
+  const int16_t* te = s.te + ((lx >> 20) & 3) * W;
+  const int pw = (int)(lcp & 0xffffu) - 1;
+  const int cell = (int)(lcell & 0xffffu);
+  int p0 = (int)(lcell >> 16), cp = (int)(lcp >> 16);
+  int64_t best_c = INT64_MAX;
+  int best_w = kNone;
+  auto consider = [&](int w, int64_t c) {
     if (c < best_c || (c == best_c && w < best_w)) {
       best_c = c;
       best_w = w;
     }
   };
-  // cached instances with headroom (or the protected one): below their line of the envelope
-  if (nh > 0 && nh <= 2) {
-    const int w0 = (int)(h0 >> 16);
-    if (s.av[b * W + w0] || w0 == pw) consider(w0, h0 & 0xffff);
-    if (nh == 2) {
-      const int w1 = (int)(h1 >> 16);
-      if (s.av[b * W + w1] || w1 == pw) consider(w1, h1 & 0xffff);
+  // cached instances, cheapest first (an empty entry ends the list, cp is kTop + 1 from then on);
+  // beyond the kept ones the whole row
+  if (cp <= kTop) {
+    const int cp0 = cp;
+    while (cp < kTop) {
+      const uint32_t e = s.list ? s.list[cp * T + t] : reinterpret_cast<const uint32_t*>(a.rec + s.lrec[t] + 2)[cp];
+      if (e == 0) {
+        cp = kTop + 1;
+        break;
+      }
+      const int w = (int)(e >> 16);
+      if (te[w] > pos || w == pw) {
+        const longlong2 q = s.ln[w];
+        consider(w, q.x + (x - 16 * (int64_t)(e & 0xffffu)) * q.y);
+        break;
+      }
+      ++cp;
     }
-  } else if (nh > 2) {
-    for (int w = 0; w < W; ++w) {
-      const int h = Hrow[w];
-      if (h && (s.av[b * W + w] || w == pw)) consider(w, h);
+    if (cp == kTop && a.rec[s.lrec[t] + 1].x <= kTop) cp = kTop + 1;
+    if (cp != cp0) s.lcp[t] = (lcp & 0xffffu) | ((uint32_t)cp << 16);
+    if (cp == kTop) {
+      const uint16_t* row = a.H + (int64_t)a.rec[s.lrec[t] + 1].y * W;
+      const int lead_in = (int)((reinterpret_cast<uintptr_t>(row) & 15) >> 1);
+      const uint4* p = reinterpret_cast<const uint4*>(row - lead_in);
+      const int pieces = (lead_in + W + 7) >> 3;
+      for (int q = 0; q < pieces; ++q) {
+        const uint4 v = __ldg(p + q);
+        if ((v.x | v.y | v.z | v.w) == 0) continue;
+        for (int e = 0; e < 8; ++e) {
+          const uint32_t u = e < 2 ? v.x : (e < 4 ? v.y : (e < 6 ? v.z : v.w));
+          const uint32_t h = (u >> (16 * (e & 1))) & 0xffffu;
+          const int w = 8 * q + e - lead_in;
+          if (!h || w < 0 || w >= W || !(te[w] > pos || w == pw)) continue;
+          const longlong2 y = s.ln[w];
+          consider(w, y.x + (x - 16 * (int64_t)h) * y.y);
+        }
+      }
     }
   }
   // the protected instance is eligible without headroom (its cached cost was considered above)
-  if (pw >= 0) consider(pw, 0);
-  if (best_w == INT32_MAX) {
-    *dec = nglobal > 0 ? MISAT_HOLD_CLASS_CAP : MISAT_HOLD_GLOBAL_CAP;
-    return -1;
+  if (pw >= 0) {
+    const longlong2 y = s.ln[pw];
+    consider(pw, y.x + x * y.y);
   }
-  const int hmax = (int)(hb >> 16), whit = 65535 - (int)(hb & 0xffffu);
-  if (sst == kSessReleased && hmax > 0 && !s.av[b * W + whit]) {
-    const int64_t lhs = hold + s.bk[whit] - s.bk[best_w];
-    const int64_t rhs = 16 * (int64_t)hmax * s.tc[whit];
-    if (lhs < rhs) {
-      *dec = MISAT_HOLD_PREFER_CACHE;
-      return -1;
+  // without a cached prefix: the price order of the cell, eight entries at a time (one load,
+  // then eight independent threshold reads): first the piece with headroom, then its entries
+  const int Wp = price_order_stride(W);
+  const uint4* ord = (s.ord ? s.ord : reinterpret_cast<const uint4*>(a.orders)) + cell * (Wp >> 3);
+  uint4 v = make_uint4(0, 0, 0, 0);
+  auto open_of = [&](int k) -> unsigned {
+    v = ord[k >> 3];
+    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+    unsigned av = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (te[(u[e >> 1] >> (16 * (e & 1))) & kPriceMask] > pos) av |= 1u << e;
+    // (the row's padding names instance 0)
+    return k + 8 > W ? av & ((1u << (W - k)) - 1u) : av;
+  };
+  const int p_in = p0;
+  unsigned av = 0;
+  while (p0 < Wp && !(av = open_of(p0))) p0 += 8;
+  if (p0 != p_in) s.lpos[t] = (uint32_t)cell | ((uint32_t)p0 << 16);
+  const int64_t xg = price_cell_start(cell), dx = x - xg;
+  const int64_t slack = dx * tc_min;
+  int k = p0;
+  while (k < Wp) {
+    if (!av) {
+      k += 8;
+      if (k < Wp) av = open_of(k);
+      continue;
     }
+    const int e = __ffs(av) - 1;
+    av &= av - 1;
+    const uint32_t pair = e < 4 ? (e < 2 ? v.x : v.y) : (e < 6 ? v.z : v.w);
+    const uint32_t ent = pair >> (16 * (e & 1));
+    const int w = (int)(ent & kPriceMask);
+    const longlong2 y = s.ln[w];
+    const int64_t cg = y.x + xg * y.y;
+    const int64_t bound = cg + slack;  // of this and every later entry
+    if (bound > best_c) break;
+    // equal bound: this entry may still win by its index; one behind it could only tie with it by
+    // having the same cost at x_g, and then it has the larger index.  A fast entry is
+    // cheaper than all behind it over the whole cell.
+    const bool last = bound == best_c || (ent & kPriceFast);
+    consider(w, cg + dx * y.y);
+    if (last) break;
   }
-  *dec = best_w == pw ? MISAT_ADMIT_CONT : MISAT_ADMIT_NEW;
+  if (best_w >= 0 && ((lx >> 22) & 1u)) {
+    int4 q;
+    if (s.eq7) {
+      q = s.eq7[t];
+    } else {
+      q = a.rec[s.lrec[t] + 1];
+      q.x = 65535 - (a.rec[s.lrec[t]].w & 0xffff);
+    }
+    const int64_t theta = ((int64_t)q.w << 32) | (uint32_t)q.z;
+    if (te[q.x] <= pos && s.ln[best_w].x > theta) return kWait;
+  }
   return best_w;
 }
 
-// First set position >= from in the window's kNW-word bitmask held by lanes 0 .. kNW-1 of
-// every warp (kNT if none).  Warp-uniform.
-__device__ __forceinline__ int first_set_from(unsigned word, int lane, int from) {
-  const int fw = from >> 5;
-  unsigned m = lane < fw ? 0u : word;
-  if (lane == fw) m &= ~0u << (from & 31);
-  const unsigned nz = __ballot_sync(kFull, m != 0);
-  if (!nz) return kNT;
-  const int w = __ffs(nz) - 1;
-  return w * 32 + __ffs(__shfl_sync(kFull, m, w)) - 1;
+// The two halves of finding the position of the (rank + 1)-th proposal in a set whose number per
+// CTA lane c holds in n (c < cs): the CTA and the rank in it, ...
+__device__ __forceinline__ int find_cta(int n, int* rank) {
+  const int incl = warp_scan(n);
+  const int src = __ffs(__ballot_sync(kFull, incl > *rank)) - 1;
+  *rank -= __shfl_sync(kFull, incl - n, src);
+  return src;
+}
+// ... and the position from that CTA's words of the set, word i in lane i.
+__device__ __forceinline__ int find_pos(unsigned x, int rank, int first_word) {
+  const int lane = threadIdx.x & 31;
+  const int n = __popc(x);
+  const int incl = warp_scan(n);
+  const int i = __ffs(__ballot_sync(kFull, incl > rank)) - 1;
+  const int k = rank - __shfl_sync(kFull, incl - n, i);
+  const unsigned y = __shfl_sync(kFull, x, i);
+  const unsigned bit = __ballot_sync(kFull, ((y >> lane) & 1u) && __popc(y & lanemask_lt()) == k);
+  return 32 * (first_word + i) + __ffs(bit) - 1;
 }
 
-// An instance's headroom dropped to `g` (global) or its class b headroom to `c`: clear its
-// flags for the classes it no longer admits.
-__device__ __forceinline__ void sel_flags(const SelSmem& s, int W, int w, int b, bool gone_g, bool gone_c,
-                                          int* s_dirty) {
-  const int x = s.pos[w];
-#pragma unroll
-  for (int c = 0; c < 3; ++c)
-    if ((gone_g || (gone_c && c == b)) && s.av[c * W + w]) {
-      s.av[c * W + w] = 0;
-      s.avp[c * W + x] = 0;
-      if (s.onp[c * W + x]) s_dirty[c] = 1;
-    }
-}
-
-__global__ void __launch_bounds__(kNT, 1) k4_select(SelectArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int s_hm[3], s_q, s_nslot, s_nglobal, s_f, s_dirty[3];
-  __shared__ unsigned s_lead[kNW], s_sens[kNW];
-  __shared__ EnvScratch s_env[3];
-  if (block_error(a.err)) return;
-  // the per-class path decided the batch unless it raised the flag (no flag: always run)
-  if (a.coupled != nullptr && *(volatile const int32_t*)a.coupled == 0) return;
-  const int W = a.W;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  SelSmem s;
-  {
-    unsigned char* p = smem;
-    s.bk = reinterpret_cast<int64_t*>(p);
-    p += (size_t)W * 8;
-    s.tc = reinterpret_cast<int64_t*>(p);
-    p += (size_t)W * 8;
-    s.hbk = reinterpret_cast<int64_t*>(p);
-    p += (size_t)W * 24;
-    s.htc = reinterpret_cast<int64_t*>(p);
-    p += (size_t)W * 24;
-    s.gh = reinterpret_cast<int32_t*>(p);
-    p += (size_t)W * 4;
-    s.ch = reinterpret_cast<int32_t*>(p);
-    p += (size_t)W * 12;
-    s.T = reinterpret_cast<int32_t*>(p);
-    p += (size_t)W * 4;
-    s.Tb = reinterpret_cast<int32_t*>(p);
-    p += (size_t)W * 12;
-    s.slot = reinterpret_cast<int32_t*>(p);
-    p += (size_t)W * 4;
-    s.wc = reinterpret_cast<int32_t*>(p);
-    p += (size_t)kNT * 4;
-    s.surv = reinterpret_cast<int32_t*>(p);
-    p += (size_t)W * 12;
-    s.ord = reinterpret_cast<int16_t*>(p);
-    p += (size_t)W * 2;
-    s.pos = reinterpret_cast<int16_t*>(p);
-    p += (size_t)W * 2;
-    s.aord = reinterpret_cast<int16_t*>(p);
-    p += (size_t)W * 2;
-    s.hull = reinterpret_cast<int16_t*>(p);
-    p += (size_t)W * 6;
-    s.av = p;
-    p += (size_t)W * 3;
-    s.avp = p;
-    p += (size_t)W * 3;
-    s.onp = p;
-  }
-  if (tid == 0) {
-    s_nglobal = 0;
-    s_q = kNT;
-    s_nslot = 0;
-    s_f = -1;
-    s_dirty[0] = s_dirty[1] = s_dirty[2] = 0;
-  }
-  __syncthreads();
-  for (int w = tid; w < W; w += kNT) {
-    const int r = a.rank[w];
-    s.ord[r] = (int16_t)w;
-    s.pos[w] = (int16_t)r;
-    s.aord[a.rank_a[w]] = (int16_t)w;
-    s.bk[w] = a.backlog[w];
-    s.tc[w] = a.tokcost[w];
-    const int32_t g = a.gh[w];
-    s.gh[w] = g;
-    if (g > 0) atomicAdd(&s_nglobal, 1);
-    s.T[w] = 0;
-    s.slot[w] = -1;
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const int32_t c = a.ch[w * 3 + b];
-      const uint8_t v = g > 0 && c > 0;
-      s.ch[b * W + w] = c;
-      s.Tb[b * W + w] = 0;
-      s.av[b * W + w] = v;
-      s.avp[b * W + r] = v;
-      s.onp[b * W + r] = a.onhull[b * W + w];
-    }
-  }
-  s.wc[tid] = 0;
-  if (tid < 3) {
-    s_env[tid].first_a = 0;
-    s_env[tid].last_s = W - 1;
-  }
-  __syncthreads();
-  if (wid < 3) env_compact_warp(s, W, wid, &s_hm[wid]);
-  __syncthreads();
-
-  // records of the first window
-  int4 n0 = make_int4(0, 0, 0, 0), n1 = make_int4(0, 0, 0, 0);
-  if (tid < a.n) {
-    n0 = a.rec[2 * tid];
-    n1 = a.rec[2 * tid + 1];
-  }
-#pragma unroll 1
-  for (int base = 0; base < a.n; base += kNT) {
-    const int i = base + tid;
-    const int4 r0 = n0, r1 = n1;
-    if (i + kNT < a.n) {  // next window's records, in flight during this one
-      n0 = a.rec[2 * (i + kNT)];
-      n1 = a.rec[2 * (i + kNT) + 1];
-    }
-    const int L = r0.x;
-    const int b = r0.y & 0xff;
-    const int sst = (r0.y >> 8) & 0xff;
-    const int pw = sst == (int)kSessProtected ? r0.z : -1;
-    const uint32_t hb = (uint32_t)r0.w;
-    const int nh = r1.x;
-    const uint32_t h0 = (uint32_t)r1.y, h1 = (uint32_t)r1.z;
-    const bool lead = i < a.n && ((r0.y >> 16) & 1);
-    const bool sens = sst == (int)kSessReleased && (hb >> 16) > 0;
-    {
-      const unsigned ml = __ballot_sync(kFull, lead), ms = __ballot_sync(kFull, lead && sens);
-      if (lane == 0) {
-        s_lead[wid] = ml;
-        s_sens[wid] = ms;
-      }
-    }
-    __syncthreads();
-    const unsigned lead_word = lane < kNW ? s_lead[lane] : 0u;
-    const unsigned sens_word = lane < kNW ? s_sens[lane] : 0u;
-    // the window's leaders before `done` are decided; a leader's tentative decision is kept
-    // over the iterations while it stays right: an admission stays the argmin as long as its
-    // instance keeps headroom for the class (the other instances only lose headroom), and a
-    // hold stays a hold
-    int done = 0;
-    bool have = false;
-    uint8_t dec = 0;
-    int dw = -1;
-    // every iteration finalises at least the window's first undecided leader (its choice is
-    // taken against the exact state of its turn), so a window needs at most kNT iterations
-    int guard = 0;
-#pragma unroll 1
-    while (true) {
-      const int head = first_set_from(lead_word, lane, done);
-      if (head == kNT) break;
-      if (++guard > kNT) {
-        if (tid == 0) set_error(a.err, MISAT_ERR_INTERNAL);
-        return;
-      }
-      // the first undecided Eq. (7) leader: the leaders before it are decided now, and an
-      // Eq. (7) leader at the head is decided alone
-      const int qcut = max(first_set_from(sens_word, lane, head), head + 1);
-      const int ng0 = s_nglobal;
-      const bool act = lead && tid >= head && tid < qcut;
-      // 1. choices against the state at the window's current start
-      if (act && !have) {
-        dw = sel_choose(s, s_hm, W, ng0, L, b, sst, pw, hb, nh, h0, h1, a.H + (int64_t)i * W, a.hold_delay_q, &dec);
-        have = true;
-      }
-      const bool cons = act && dec == MISAT_ADMIT_NEW;
-      // 2. admissions per (instance, class)
-      const unsigned pm = __match_any_sync(kFull, cons ? dw : -1 - lane);
-      const unsigned pc = __match_any_sync(kFull, cons ? dw * 3 + b : -1 - lane);
-      const bool gl = cons && lane == __ffs(pm) - 1;  // first lane of its instance in the warp
-      const bool cl = cons && lane == __ffs(pc) - 1;
-      if (gl) atomicAdd(&s.T[dw], __popc(pm));
-      if (cl) atomicAdd(&s.Tb[b * W + dw], __popc(pc));
-      __syncthreads();
-      bool any;
-      {
-        const bool over = gl && s.T[dw] > s.gh[dw];
-        const bool overc = cl && s.Tb[b * W + dw] > s.ch[b * W + dw];
-        if ((over || overc) && atomicCAS(&s.slot[dw], -1, -2) == -1) s.slot[dw] = atomicAdd(&s_nslot, 1);
-        any = __syncthreads_or(over || overc);
-      }
-      int qv = kNT;
-      if (any) {
-        // exact arrival-order ranks at the over-subscribed instances, kSlotInst at a time: a
-        // consumer is invalid when the consumers before it fill its instance or its class
-        const int nslot = s_nslot;
-        for (int p0 = 0; p0 < nslot; p0 += kSlotInst) {
-          const int sl = cons ? s.slot[dw] - p0 : -1;
-          const bool mine = sl >= 0 && sl < kSlotInst;
-          if (mine && gl) s.wc[(sl * 4) * kNW + wid] = __popc(pm);
-          if (mine && cl) s.wc[(sl * 4 + 1 + b) * kNW + wid] = __popc(pc);
-          __syncthreads();
-          {  // exclusive scan over the warps of each counter: thread = (counter, warp)
-            const int v = s.wc[tid];
-            int incl = v;
-#pragma unroll
-            for (int o = 1; o < kNW; o <<= 1) {
-              const int t = __shfl_up_sync(kFull, incl, o, kNW);
-              if ((lane & (kNW - 1)) >= o) incl += t;
-            }
-            s.wc[tid] = incl - v;
-          }
-          __syncthreads();
-          bool bad = false;
-          if (mine) {
-            const unsigned lt = lanemask_lt();
-            const int ag = __popc(pm & lt) + s.wc[(sl * 4) * kNW + wid];
-            const int ac = __popc(pc & lt) + s.wc[(sl * 4 + 1 + b) * kNW + wid];
-            bad = ag >= s.gh[dw] || ac >= s.ch[b * W + dw];
-          }
-          const unsigned mb = __ballot_sync(kFull, bad);
-          if (lane == 0 && mb) atomicMin(&s_q, wid * 32 + __ffs(mb) - 1);
-          __syncthreads();
-          s.wc[tid] = 0;
-          __syncthreads();
-        }
-        qv = s_q;
-      }
-      const int q = min(qv, qcut);
-      // 3. the leaders before q are final: take their admissions out of the headroom (per
-      //    warp, atomically; the one that empties an instance or class clears its flags)
-      {
-        const bool cc = cons && tid < q;
-        const int qw = q - wid * 32;  // lanes of this warp before q
-        const unsigned below = qw >= 32 ? kFull : (qw <= 0 ? 0u : ((1u << qw) - 1));
-        const unsigned qm = pm & below, qc = pc & below;
-        if (cc && lane == __ffs(qm) - 1) {
-          const int k = __popc(qm);
-          const int g = atomicSub(&s.gh[dw], k);
-          if (g > 0 && g - k <= 0) {
-            atomicSub(&s_nglobal, 1);
-            sel_flags(s, W, dw, b, true, false, s_dirty);
-          }
-        }
-        if (cc && lane == __ffs(qc) - 1) {
-          const int k = __popc(qc);
-          const int c = atomicSub(&s.ch[b * W + dw], k);
-          if (c > 0 && c - k <= 0) sel_flags(s, W, dw, b, false, true, s_dirty);
-        }
-      }
-      __syncthreads();
-      if (gl) {
-        s.T[dw] = 0;
-        s.slot[dw] = -1;
-      }
-      if (cl) s.Tb[b * W + dw] = 0;
-      // the last instance with global headroom filled in this prefix: the holds after the
-      // admission that filled it found no global headroom at their turn
-      const bool exhausted = ng0 > 0 && s_nglobal == 0;
-      if (exhausted) {  // uniform
-        const unsigned mf = __ballot_sync(kFull, cons && tid < q);
-        if (lane == 0 && mf) atomicMax(&s_f, wid * 32 + 31 - __clz(mf));
-        __syncthreads();
-      }
-      if (act && tid < q) {
-        if (dec == MISAT_HOLD_CLASS_CAP && (ng0 == 0 || (exhausted && tid > s_f))) dec = MISAT_HOLD_GLOBAL_CAP;
-        if (dec == MISAT_ADMIT_NEW || dec == MISAT_ADMIT_CONT) {
-          a.rq.status[i] = kStResolved;
-          a.rq.inst[i] = dw;
-          a.rq.reason[i] = dec;
-        } else {  // (inst may hold an admission of the per-class path, which this replaces)
-          a.rq.status[i] = kStHeld;
-          a.rq.inst[i] = -1;
-          a.rq.last_reason[i] = dec;
-        }
-      } else if (have && dec == MISAT_ADMIT_NEW && !s.av[b * W + dw]) {
-        have = false;  // its instance has no headroom for the class any more: choose again
-      }
-      done = q;
-      // envelopes of the classes that lost an envelope line: one warp per class
-      if (wid < 3 && s_dirty[wid]) env_update_warp(s, W, wid, &s_hm[wid], s_env[wid], a.small);
-      __syncthreads();
-      // nobody reads these again before the next iteration's first barrier
-      if (tid == 0) {
-        s_q = kNT;
-        s_nslot = 0;
-        s_f = -1;
-        s_dirty[0] = s_dirty[1] = s_dirty[2] = 0;
-      }
-    }
-    __syncthreads();  // the window's bitmasks are read until here
-  }
-}
-
-size_t select_smem_bytes(int W) {
-  return (size_t)W * 8 * 2 + (size_t)W * 48 + (size_t)W * 4 * 4 + (size_t)W * 4 * 4 + (size_t)W * 4 +
-         (size_t)kNT * 4 + (size_t)W * 12 + (size_t)W * 2 * 6 + (size_t)W * 9 + 16;
-}
-
-cudaError_t select_configure() {
-  // sized for the largest instance count, so that contexts of any size share the setting
-  return cudaFuncSetAttribute(k4_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)select_smem_bytes(kMaxW));
-}
-
-void launch_select(const SelectArgs& a, cudaStream_t st) {
-  if (a.n <= 0) return;
-  k4_select<<<1, kNT, select_smem_bytes(a.W), st>>>(a);
-}
-
-// ---------------------------------------------------------------------------
-// Per-class selection: the path taken when no instance runs out of global headroom.
-//
-// A leader of class b is eligible on w when w has global headroom and class-b headroom
-// (Eq. 6 with the class cap of Sec. 4.2).  As long as every instance keeps global headroom,
-// eligibility depends only on the admissions of the leader's own class, so the leaders of the
-// three classes form three independent chains.  One CTA per class decides its class's leaders
-// in arrival order with the window scheme of k4_select, on one envelope and per-instance
-// counters.  At the end the CTAs add up their admissions per instance: if every instance that
-// had global headroom at batch start keeps some, no decision could have depended on the global
-// cap, and the result is exactly that of the joint arrival order (by induction over the arrival
-// order: each instance's global headroom stays positive at every leader's turn, so the joint
-// eligibility equals the per-class one, and a hold's reason -- class cap while some instance
-// has global headroom -- is the class cap exactly when some instance had it at batch start).
-// Otherwise the last CTA sets `coupled` and k4_select decides the whole batch again.
-//
-// Within a window a tentative admission is final once the registered choosers of its
-// instance before it leave it headroom; the first leader that finds none cuts the window.
-// Registrations stay in place for the whole window (decided ones included), so the slot where
-// an instance runs out (the ch-th registered chooser, ch its headroom at the window's start)
-// and the slot of its first chooser that finds none only move earlier as leaders register,
-// and are recomputed (one warp per instance) only for the instances that received
-// registrations since their last scan.  An instance that runs out leaves the envelope by a
-// local repair (the lines between its neighbours that lie below their chord, envelope.cuh),
-// and only the undecided leaders that had chosen it choose again.
-namespace {
-constexpr int kCT = kSelectClassThreads;
-constexpr int kMaxBatchBlocks = 4096;  // blocks of 256 requests: batches of up to 2^20 requests
-constexpr int kCW = kCT / 32;
-static_assert(kCW <= 32 && (kCW & (kCW - 1)) == 0, "the window bitmask is at most one word per lane of a warp");
 }  // namespace
 
-struct ClsSmem {
-  unsigned* regm;  // [W][kCW] registered choosers of each instance in the window: one bit per slot
-  longlong2* ln;   // [W] {d_w, 1/mu_w}
-  longlong2* hl;   // [W] {d_w, 1/mu_w} of the envelope lines, slope order
-  longlong2* tl;   // [W] scratch of the envelope repair
-  int32_t* ch;     // [W] class headroom at the window's start (0 without global headroom)
-  int32_t* T;      // [W] registered choosers in the window
-  int32_t* fpos;   // [W] window slot of the chooser that takes an instance's last headroom, kCT
-  int32_t* pp;     // [W] window slot of its first chooser that finds no headroom, kCT
-  int32_t* cand;   // [W] envelope repair candidates
-  int32_t* rem;    // [W] instances that ran out in this iteration
-  int16_t* hull;   // [W] envelope lines, slope order
-  int16_t* th;     // [W] scratch of the envelope repair
-  int16_t* hp;     // [W] position of an instance on the envelope, -1 if it is not on it
-  int16_t* ord;    // [W] instances in slope order
-  int16_t* pos;    // [W] position in slope order
-  int16_t* aord;   // [W] instances in (d_w, w) order
-  uint8_t* av;     // [W] class headroom left
-  unsigned* tm;    // [32] "tight" instances: registered choosers >= class headroom > 0
-  unsigned* dm;    // [32] tight instances with registrations since their last scan
-};
-
-size_t select_class_smem_bytes(int W, int n) {
-  const size_t nblk = ((size_t)n + 255) >> 8;
-  return (size_t)256 + (size_t)W * (4 * kCW + 16 * 3 + 4 * 6 + 2 * 6) + (((size_t)W + 15) & ~(size_t)15) +
-         nblk * 4 + 64;
-}
-
-// First set position >= from in a kCT-bit mask held one word per lane (kCT if none).  Warp-uniform.
-__device__ __forceinline__ int cls_first_set(unsigned word, int lane, int from) {
-  if (from >= kCT) return kCT;
-  const int fw = from >> 5;
-  unsigned m = lane < fw ? 0u : word;
-  if (lane == fw) m &= ~0u << (from & 31);
-  const unsigned nz = __ballot_sync(kFull, m != 0);
-  if (!nz) return kCT;
-  const int w = __ffs(nz) - 1;
-  return w * 32 + __ffs(__shfl_sync(kFull, m, w)) - 1;
-}
-
-// Position of the (k+1)-th set bit of x (0 <= k < popc(x)): a binary search on bit counts.
-__device__ __forceinline__ int nth_set(unsigned x, int k) {
-  int pos = 0;
-  int c = __popc(x & 0xffffu);
-  if (k >= c) { k -= c; x >>= 16; pos += 16; }
-  c = __popc(x & 0xffu);
-  if (k >= c) { k -= c; x >>= 8; pos += 8; }
-  c = __popc(x & 0xfu);
-  if (k >= c) { k -= c; x >>= 4; pos += 4; }
-  c = __popc(x & 0x3u);
-  if (k >= c) { k -= c; x >>= 2; pos += 2; }
-  if (k >= (int)(x & 1u)) pos += 1;
-  return pos;
-}
-
-// Decision of one leader of the CTA's class against the current state; see sel_choose.
-__device__ __forceinline__ int cls_choose(const ClsSmem& s, int m, int nglobal, int64_t x, int sst, int pw,
-                                          uint32_t hb, int nh, uint32_t h0, uint32_t h1, const uint16_t* Hrow,
-                                          int W, int64_t hold, uint8_t* dec) {
-  int64_t best_c = INT64_MAX;
-  int best_w = INT32_MAX;
-  if (m > 0) {
-    int lo = 0, hi = m - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      const longlong2 u = s.hl[mid], v = s.hl[mid + 1];
-      const int64_t cu = u.x + x * u.y, cv = v.x + x * v.y;
-      // line mid + 1 beats line mid at x (ties to the lower index)
-      if (cv < cu || (cv == cu && s.hull[mid + 1] < s.hull[mid])) lo = mid + 1;
-      else hi = mid;
-    }
-    const longlong2 t = s.hl[lo];
-    best_w = s.hull[lo];
-    best_c = t.x + x * t.y;
-  }
-  auto consider = [&](int w, int64_t h) {
-    const longlong2 t = s.ln[w];
-    const int64_t c = t.x + (x - 16 * h) * t.y;
-    if (c < best_c || (c == best_c && w < best_w)) {
-      best_c = c;
-      best_w = w;
-    }
-  };
-  if (nh > 0 && nh <= 2) {
-    const int w0 = (int)(h0 >> 16);
-    if (s.av[w0] || w0 == pw) consider(w0, h0 & 0xffff);
-    if (nh == 2) {
-      const int w1 = (int)(h1 >> 16);
-      if (s.av[w1] || w1 == pw) consider(w1, h1 & 0xffff);
-    }
-  } else if (nh > 2) {
-    for (int w = 0; w < W; ++w) {
-      const int h = Hrow[w];
-      if (h && (s.av[w] || w == pw)) consider(w, h);
-    }
-  }
-  if (pw >= 0) consider(pw, 0);
-  if (best_w == INT32_MAX) {
-    *dec = nglobal > 0 ? MISAT_HOLD_CLASS_CAP : MISAT_HOLD_GLOBAL_CAP;
-    return -1;
-  }
-  const int hmax = (int)(hb >> 16), whit = 65535 - (int)(hb & 0xffffu);
-  if (sst == kSessReleased && hmax > 0 && !s.av[whit]) {
-    const int64_t lhs = hold + s.ln[whit].x - s.ln[best_w].x;
-    const int64_t rhs = 16 * (int64_t)hmax * s.ln[whit].y;
-    if (lhs < rhs) {
-      *dec = MISAT_HOLD_PREFER_CACHE;
-      return -1;
-    }
-  }
-  *dec = best_w == pw ? MISAT_ADMIT_CONT : MISAT_ADMIT_NEW;
-  return best_w;
-}
-
-__device__ __forceinline__ bool cls_present(const ClsSmem& s, int i) { return s.av[i] || s.hp[i] >= 0; }
-
-// Envelope repair after instance w ran out of headroom (one warp).  The lines p and q that bound
-// the repaired stretch are w's neighbours on the envelope, or, where w was the first (last)
-// line, the line that now wins at x = 0 (for large x).  The lines strictly between p and q in
-// slope order that lie below the chord p-q are the candidates; each is tested against p, q and
-// the other candidates (EnvTest over the domain x >= 0), and the ones on the envelope replace
-// w.  A line that ran out in the same iteration but is still on the envelope counts as present
-// until its own repair, so that every repair computes the envelope of a well-defined set; the
-// order of the repairs does not change the final envelope.  first_a / last_s: forward-only
-// pointers to the lines that may win at x = 0 ((d_w, w) order) and for large x (slope order).
-__device__ __forceinline__ void cls_repair(const ClsSmem& s, int W, int w, int* hm, int* first_a, int* last_s,
-                                           bool small) {
-  const int lane = threadIdx.x & 31;
-  const int k = s.hp[w];
-  __syncwarp();
-  if (k < 0) return;
-  if (lane == 0) s.hp[w] = -1;
-  __syncwarp();
-  const int m = *hm;
-  const int P = k > 0 ? s.hull[k - 1] : -1, Q = k + 1 < m ? s.hull[k + 1] : -1;
-  int p = P, q = Q;
-  if (p < 0) {  // the line that now wins at x = 0
-    int a = *first_a;
-    while (a < W && !cls_present(s, s.aord[a])) ++a;
-    p = a < W ? s.aord[a] : -1;
-    __syncwarp();
-    if (lane == 0) *first_a = a;
-  }
-  if (q < 0 && p >= 0) {  // the line that now wins for large x: least 1/mu_w, then least d_w
-    int x = *last_s;
-    while (x >= 0 && !cls_present(s, s.ord[x])) --x;
-    __syncwarp();
-    if (lane == 0) *last_s = x;
-    const int64_t t = s.ln[s.ord[x]].y;
-    int y = x;
-    for (int z = x - 1; z >= 0 && s.ln[s.ord[z]].y == t; --z)
-      if (cls_present(s, s.ord[z])) y = z;
-    q = s.ord[y];
-  }
-  int nnew = 0;
-  if (P < 0 && p >= 0 && p != Q) {
-    if (lane == 0) s.th[0] = (int16_t)p;
-    nnew = 1;
-  }
-  if (p >= 0 && q != p) {
-    const int xp = s.pos[p], xq = s.pos[q];
-    const longlong2 lp = s.ln[p], lq = s.ln[q];
-    int nc = 0;
-    for (int x0 = xp + 1; x0 < xq; x0 += 32) {
-      const int x = x0 + lane;
-      bool c = false;
-      int i = 0;
-      if (x < xq) {
-        i = s.ord[x];
-        if (s.av[i]) {
-          const longlong2 li = s.ln[i];
-          c = li.y != lp.y && env_below_chord(li.x, li.y, i, lp.x, lp.y, p, lq.x, lq.y, q, small);
-        }
-      }
-      const unsigned mc = __ballot_sync(kFull, c);
-      if (c) s.cand[nc + __popc(mc & lanemask_lt())] = i;
-      nc += __popc(mc);
-    }
-    __syncwarp();
-    if (nc == 1) {
-      // a single line below the chord beats p and q around their crossing (x >= 0): it is on
-      // the envelope, and nothing else enters between p and q
-      if (lane == 0) s.th[nnew] = (int16_t)s.cand[0];
-      nnew += 1;
-    }
-    for (int e0 = 0; nc > 1 && e0 < nc; e0 += 32) {
-      const int e = e0 + lane;
-      bool on = false;
-      int i = 0;
-      if (e < nc) {
-        i = s.cand[e];
-        const longlong2 li = s.ln[i];
-        EnvTest t;
-        env_test_init(t);
-        env_test_add(t, li.x, li.y, i, lp.x, lp.y, p, small);
-        env_test_add(t, li.x, li.y, i, lq.x, lq.y, q, small);
-        for (int f = 0; f < nc; ++f) {
-          const int j = s.cand[f];
-          if (j != i) {
-            const longlong2 lj = s.ln[j];
-            env_test_add(t, li.x, li.y, i, lj.x, lj.y, j, small);
-          }
-        }
-        on = env_test_on(t, small);
-      }
-      const unsigned mo = __ballot_sync(kFull, on);
-      if (on) s.th[nnew + __popc(mo & lanemask_lt())] = (int16_t)i;
-      nnew += __popc(mo);
-    }
-    if (Q < 0 && q != P) {
-      if (lane == 0) s.th[nnew] = (int16_t)q;
-      nnew += 1;
-    }
-  }
-  __syncwarp();
-  // splice: hull[0..k-1] ++ th[0..nnew-1] ++ hull[k+1..m-1]
-  const int tail = m - k - 1;
-  for (int t = lane; t < tail; t += 32) {
-    s.th[nnew + t] = s.hull[k + 1 + t];
-    s.tl[nnew + t] = s.hl[k + 1 + t];
-  }
-  for (int t = lane; t < nnew; t += 32) s.tl[t] = s.ln[s.th[t]];
-  __syncwarp();
-  const int total = nnew + tail;
-  for (int t = lane; t < total; t += 32) {
-    const int v = s.th[t];
-    s.hull[k + t] = (int16_t)v;
-    s.hl[k + t] = s.tl[t];
-    s.hp[v] = (int16_t)(k + t);
-  }
-  if (lane == 0) *hm = k + total;
-  __syncwarp();
-}
-
-__global__ void __launch_bounds__(kCT, 1) k4_select_class(SelectClassArgs a) {
+__global__ void __launch_bounds__(1024, 1) k4_select(SelectArgs a, int cs) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int s_nc, s_hm, s_first_a, s_last_s, s_nglobal, s_last, s_navail;
-  __shared__ int s_qb[2];  // cut bound of the current and the next iteration
-  __shared__ int s_ws[kCW];
-  __shared__ unsigned s_lead[kCW], s_sens[kCW];
+  __shared__ int s_ws[32];
+  __shared__ int s_total;
+  __shared__ int s_queued;          // leaders in the queue
+  __shared__ int s_changed[2];      // some threshold moved in this round (written by any CTA)
+  __shared__ int s_fix[16];         // per CTA: first leader of the window to fix as held
+  __shared__ int s_fixmin;
+  __shared__ int s_tgmax;
+  __shared__ unsigned long long s_tcmin;
   if (block_error(a.err)) return;
-  const int W = a.W, b = blockIdx.x;
+  const int W = a.W;
+  const int T = blockDim.x, NW = T >> 5;
+  const int words = cs * NW;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  ClsSmem s;
-  {
-    unsigned char* p = smem;
-    s.tm = reinterpret_cast<unsigned*>(p);
-    s.dm = s.tm + 32;
-    p += 256;
-    s.regm = reinterpret_cast<unsigned*>(p);
-    p += (size_t)W * kCW * 4;
-    s.ln = reinterpret_cast<longlong2*>(p);
-    p += (size_t)W * 16;
-    s.hl = reinterpret_cast<longlong2*>(p);
-    p += (size_t)W * 16;
-    s.tl = reinterpret_cast<longlong2*>(p);
-    p += (size_t)W * 16;
-    s.ch = reinterpret_cast<int32_t*>(p);
-    p += (size_t)W * 4;
-    s.T = reinterpret_cast<int32_t*>(p);
-    p += (size_t)W * 4;
-    s.fpos = reinterpret_cast<int32_t*>(p);
-    p += (size_t)W * 4;
-    s.pp = reinterpret_cast<int32_t*>(p);
-    p += (size_t)W * 4;
-    s.cand = reinterpret_cast<int32_t*>(p);
-    p += (size_t)W * 4;
-    s.rem = reinterpret_cast<int32_t*>(p);
-    p += (size_t)W * 4;
-    s.hull = reinterpret_cast<int16_t*>(p);
-    p += (size_t)W * 2;
-    s.th = reinterpret_cast<int16_t*>(p);
-    p += (size_t)W * 2;
-    s.hp = reinterpret_cast<int16_t*>(p);
-    p += (size_t)W * 2;
-    s.ord = reinterpret_cast<int16_t*>(p);
-    p += (size_t)W * 2;
-    s.pos = reinterpret_cast<int16_t*>(p);
-    p += (size_t)W * 2;
-    s.aord = reinterpret_cast<int16_t*>(p);
-    p += (size_t)W * 2;
-    s.av = p;
-  }
-  if (tid == 0) {
-    s_nglobal = 0;
-    s_qb[0] = kCT;
-    s_first_a = 0;
-    s_last_s = W - 1;
-    s_navail = 0;
-  }
-  __syncthreads();
-  for (int w = tid; w < W; w += kCT) {
-    const int r = a.rank[w];
-    s.ord[r] = (int16_t)w;
-    s.pos[w] = (int16_t)r;
-    s.aord[a.rank_a[w]] = (int16_t)w;
-    s.ln[w] = make_longlong2(a.backlog[w], a.tokcost[w]);
-    const int g = a.gh[w];
-    if (g > 0) atomicAdd(&s_nglobal, 1);
-    const int c = g > 0 ? a.ch[w * 3 + b] : 0;
-    s.ch[w] = c;
-    s.av[w] = c > 0;
-    if (c > 0) atomicAdd(&s_navail, 1);
-    s.T[w] = 0;
-    s.fpos[w] = kCT;
-    s.pp[w] = kCT;
-    s.hp[w] = -1;
-  }
-  for (int i = tid; i < W * kCW; i += kCT) s.regm[i] = 0;
-  if (tid < 64) s.tm[tid] = 0;  // tm and dm
-  __syncthreads();
-  // initial envelope of the class (launch_env_init), compacted in slope order
-  if (wid == 0) {
-    int base = 0;
-    for (int x0 = 0; x0 < W; x0 += 32) {
-      const int x = x0 + lane;
-      const int w = x < W ? s.ord[x] : 0;
-      const bool f = x < W && a.onhull[b * W + w];
-      const unsigned mf = __ballot_sync(kFull, f);
-      if (f) {
-        const int k = base + __popc(mf & lanemask_lt());
-        s.hull[k] = (int16_t)w;
-        s.hl[k] = s.ln[w];
-        s.hp[w] = (int16_t)k;
-      }
-      base += __popc(mf);
-    }
-    if (lane == 0) s_hm = base;
-  }
-  // The class's leaders in arrival order: the prep kernel listed them per block of 256
-  // requests; the block offsets are an exclusive scan of its counts (s_pre), and the class
-  // index g of a leader maps to its block by binary search.
+  const int cta = cs == 1 ? 0 : (int)blockIdx.x;
+  const int pos = cta * T + tid;    // position of this thread's leader in the window
   const int nblk = (a.n + 255) >> 8;
-  const int32_t* seg = a.seg + (int64_t)b * a.n;
-  int* s_pre = reinterpret_cast<int*>(s.av + ((W + 15) & ~15));
+  SelSmem s;
+  sel_smem_layout(W, cs, NW, nblk, &s, smem);
+  const uint32_t sm_te = smem_addr(s.te), sm_tg = smem_addr(s.tg), sm_cm = smem_addr(s.cm),
+                 sm_prop = smem_addr(s.prop), sm_n01 = smem_addr(s.n01), sm_n2 = smem_addr(s.n2),
+                 sm_changed = smem_addr(s_changed), sm_fix = smem_addr(s_fix);
+
+  // ---- state at batch start
+  if (tid == 0) {
+    s_changed[0] = s_changed[1] = 0;
+    s_queued = 0;
+    s_tcmin = ~0ull;
+  }
+  __syncthreads();
+  for (int w = tid; w < W; w += T) {
+    const longlong2 t = make_longlong2(a.backlog[w], a.tokcost[w]);
+    s.ln[w] = t;
+    atomicMin(&s_tcmin, (unsigned long long)t.y);
+    const int g = a.gh[w], c0 = a.ch[w * 3], c1 = a.ch[w * 3 + 1], c2 = a.ch[w * 3 + 2];
+    s.tg[w] = g > 0 ? kNever : -1;
+    s.te[w] = g > 0 && c0 > 0 ? kNever : -1;
+    s.te[W + w] = g > 0 && c1 > 0 ? kNever : -1;
+    s.te[2 * W + w] = g > 0 && c2 > 0 ? kNever : -1;
+    s.n01[w] = 0;
+    s.n2[w] = 0;
+    if (w % cs == cta) {
+      s.hr[w / cs] = make_int4(c0, c1, c2, g);
+      s.seen[w / cs] = 0;
+    }
+  }
+  for (int i = tid; i < W * NW; i += T) s.prop[i] = 0;
+  if (s.ord) {
+    const uint4* src = reinterpret_cast<const uint4*>(a.orders);
+    const int pieces = kPriceCells * (price_order_stride(W) >> 3);
+#pragma unroll 4
+    for (int i = tid; i < pieces; i += T) s.ord[i] = __ldg(src + i);
+  }
+  // leaders before each block of 256 requests (exclusive scan of the prep kernel's counts)
   {
-    constexpr int kPer = (kMaxBatchBlocks + kCT - 1) / kCT;
-    int v[kPer], t = 0;
-#pragma unroll
-    for (int u = 0; u < kPer; ++u) {
-      const int j = tid * kPer + u;
-      v[u] = j < nblk ? a.segcnt[b * nblk + j] : 0;
-      t += v[u];
+    const int per = (nblk + T - 1) / T;
+    int t = 0;
+    for (int u = 0; u < per; ++u) {
+      const int j = tid * per + u;
+      if (j < nblk) t += a.segcnt[j];
     }
-    int incl = t;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int x = __shfl_up_sync(kFull, incl, o);
-      if (lane >= o) incl += x;
-    }
+    const int incl = warp_scan(t);
     if (lane == 31) s_ws[wid] = incl;
     __syncthreads();
     if (wid == 0) {
-      const int x = lane < kCW ? s_ws[lane] : 0;
-      int wi = x;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(kFull, wi, o);
-        if (lane >= o) wi += y;
-      }
-      if (lane < kCW) s_ws[lane] = wi - x;
-      if (lane == 31) s_nc = wi;
+      const int v = lane < NW ? s_ws[lane] : 0;
+      const int sc = warp_scan(v);
+      s_ws[lane] = sc - v;
+      if (lane == 31) s_total = sc;
     }
     __syncthreads();
     int off = s_ws[wid] + incl - t;
-#pragma unroll
-    for (int u = 0; u < kPer; ++u) {
-      const int j = tid * kPer + u;
-      if (j < nblk) s_pre[j] = off;
-      off += v[u];
+    for (int u = 0; u < per; ++u) {
+      const int j = tid * per + u;
+      if (j < nblk) {
+        s.pre[j] = off;
+        off += a.segcnt[j];
+      }
     }
     __syncthreads();
   }
-  const int nc = s_nc;
-  // request of class index g (< nc): the last block whose offset is <= g
-  auto leader_at = [&](int g) -> int {
+  const int nl = s_total;
+  const int64_t tc_min = (int64_t)s_tcmin;
+  // record of the g-th leader: its block is the last one whose offset is <= g
+  auto leader_rec = [&](int g) -> int {
     int lo = 0, hi = nblk - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (s_pre[mid] <= g) lo = mid;
+      if (s.pre[mid] <= g) lo = mid;
       else hi = mid - 1;
     }
-    return seg[(int64_t)lo * 256 + (g - s_pre[lo])];
+    return kRecInt4 * (lo * 256 + (g - s.pre[lo]));
   };
-  const int nglobal = s_nglobal;
+  auto decide = [&](int r, int choice, int pw, bool global_left) {
+    if (choice >= 0) {
+      a.rq.status[r] = kStResolved;
+      a.rq.inst[r] = choice;
+      a.rq.reason[r] = choice == pw ? MISAT_ADMIT_CONT : MISAT_ADMIT_NEW;
+    } else {
+      a.rq.status[r] = kStHeld;
+      a.rq.inst[r] = -1;
+      a.rq.last_reason[r] = choice == kWait || choice == kFixed
+                                ? MISAT_HOLD_PREFER_CACHE
+                                : (global_left ? MISAT_HOLD_CLASS_CAP : MISAT_HOLD_GLOBAL_CAP);
+    }
+  };
+  // the other CTAs' shared memory is written from here on
+  cluster_barrier(cs);
 
-  // records of the first window
-  int rn = tid < nc ? leader_at(tid) : 0;
-  int4 n0 = make_int4(0, 0, 0, 0), n1 = make_int4(0, 0, 0, 0);
-  if (tid < nc) {
-    n0 = a.rec[2 * rn];
-    n1 = a.rec[2 * rn + 1];
-  }
+  int par = 0;  // parity of the round's changed flag
 #pragma unroll 1
-  for (int base = 0; base < nc; base += kCT) {
-    if (s_navail == 0) {
-      // no instance has headroom for the class any more: every remaining leader is decided
-      // on its own (a protected session continues on its instance, anyone else is held)
-      for (int i = base + tid; i < nc; i += kCT) {
-        const int r = leader_at(i);
-        const int4 r0 = a.rec[2 * r];
-        if (((r0.y >> 8) & 0xff) == (int)kSessProtected) {
-          a.rq.status[r] = kStResolved;
-          a.rq.inst[r] = r0.z;
-          a.rq.reason[r] = MISAT_ADMIT_CONT;
-        } else {
-          a.rq.status[r] = kStHeld;
-          a.rq.inst[r] = -1;
-          a.rq.last_reason[r] = nglobal > 0 ? MISAT_HOLD_CLASS_CAP : MISAT_HOLD_GLOBAL_CAP;
-        }
-      }
-      break;
-    }
-    const int i = base + tid;
-    const bool valid = i < nc;
-    const int r = rn;
-    const int4 r0 = n0, r1 = n1;
-    if (i + kCT < nc) {  // the next window's records, in flight during this one
-      rn = leader_at(i + kCT);
-      n0 = a.rec[2 * rn];
-      n1 = a.rec[2 * rn + 1];
-    }
-    const int64_t L = r0.x;
-    const int sst = (r0.y >> 8) & 0xff;
-    const int pw = sst == (int)kSessProtected ? r0.z : -1;
-    const uint32_t hb = (uint32_t)r0.w;
-    const int nh = r1.x;
-    const uint32_t h0 = (uint32_t)r1.y, h1 = (uint32_t)r1.z;
-    const bool sens = valid && sst == (int)kSessReleased && (hb >> 16) > 0;
+  for (int base = 0; base < nl; base += cs * T) {
+    // no headroom left for any class: the leaders that remain are decided on their own (a
+    // protected session continues on its instance, anyone else is held)
     {
-      const unsigned ml = __ballot_sync(kFull, valid), ms = __ballot_sync(kFull, sens);
-      if (lane == 0) {
-        s_lead[wid] = ml;
-        s_sens[wid] = ms;
+      bool any = false, anyg = false;
+      for (int w = tid; w < W; w += T) {
+        any |= s.te[w] >= 0 || s.te[W + w] >= 0 || s.te[2 * W + w] >= 0;
+        anyg |= s.tg[w] >= 0;
+      }
+      any = __syncthreads_or(any);
+      if (!any) {
+        anyg = __syncthreads_or(anyg);
+        for (int g = base + pos; g < nl; g += cs * T) {
+          const int4* rec = a.rec + leader_rec(g);
+          const int4 q0 = rec[0];
+          const int pw = ((q0.y >> 8) & 0xff) == (int)kSessProtected ? q0.z : -1;
+          decide(rec[1].y, pw >= 0 ? pw : kNone, pw, anyg);
+        }
+        break;
       }
     }
-    __syncthreads();
-    const unsigned lead_word = lane < kCW ? s_lead[lane] : 0u;
-    const unsigned sens_word = lane < kCW ? s_sens[lane] : 0u;
-    int done = 0, par = 0;
-    bool have = false, reg = false;
-    uint8_t dec = 0;
-    int dw = -1;
+    const bool valid = base + pos < nl;
+    int b = 3;
+    bool eq7 = false;
+    if (valid) {
+      const int at = leader_rec(base + pos);
+      const int4 q0 = a.rec[at], q1 = a.rec[at + 1];
+      b = q0.y & 0xff;
+      eq7 = q1.w != (int)(INT64_MAX >> 32);
+      s.lx[tid] = (uint32_t)q0.x | ((uint32_t)b << 20) | ((uint32_t)eq7 << 22);
+      s.lpos[tid] = (uint32_t)price_cell((uint32_t)q0.x);
+      s.lcp[tid] = (uint32_t)((((q0.y >> 8) & 0xff) == (int)kSessProtected ? q0.z : -1) + 1) |
+                   ((q1.x > 0 ? 0u : kTop + 1u) << 16);
+      s.lrec[tid] = at;
+      if (eq7 && s.eq7) s.eq7[tid] = make_int4(65535 - (q0.w & 0xffff), 0, q1.z, q1.w);
+      if (q1.x > 0 && s.list) {
+        const int4 q2 = a.rec[at + 2], q3 = a.rec[at + 3];
+        const int e[kTop] = {q2.x, q2.y, q2.z, q2.w, q3.x, q3.y, q3.z, q3.w};
+#pragma unroll
+        for (int k = 0; k < kTop; ++k) s.list[k * T + tid] = (uint32_t)e[k];
+      }
+    }
+    s.lch[tid] = kNone;
+    {
+      const unsigned m0 = __ballot_sync(kFull, b == 0), m1 = __ballot_sync(kFull, b == 1),
+                     m2 = __ballot_sync(kFull, b == 2);
+      for (int i = lane; i < 3 * cs; i += 32) {
+        const int c = i / cs, rank = i - c * cs;
+        st_cluster(map_rank(sm_cm + 4 * (c * words + cta * NW + wid), rank), c == 0 ? m0 : (c == 1 ? m1 : m2));
+      }
+    }
+    const int pw = valid ? (int)(s.lcp[tid] & 0xffffu) - 1 : -1;
+    bool need = valid;
     int guard = 0;
 #pragma unroll 1
     while (true) {
-      const int head = cls_first_set(lead_word, lane, done);
-      if (head == kCT) break;
-      if (++guard > 2 * kCT) {  // every iteration decides at least the leader at `head`
-        if (tid == 0) set_error(a.err, MISAT_ERR_INTERNAL);
-        return;
-      }
-      // an Eq. (7) leader is decided alone, at the head, against the exact state of its turn
-      const int qcut = max(cls_first_set(sens_word, lane, head), head + 1);
-      const bool act = valid && tid >= head && tid < qcut;
-      // 1. an undecided leader whose instance ran out chooses again (its stale registration
-      //    stays with that instance, which is never scanned again); choices and registration,
-      //    one shared-memory update per (warp, instance)
-      if (tid >= done && reg && !s.av[dw]) {
-        reg = false;
-        have = false;
-      }
-      bool nreg = false;
-      if (act && !have) {
-        dw = cls_choose(s, s_hm, nglobal, L, sst, pw, hb, nh, h0, h1, a.H + (int64_t)r * W, W, a.hold_delay_q, &dec);
-        have = true;
-        nreg = dec == MISAT_ADMIT_NEW;
-        reg = nreg;
-      }
-      if (__any_sync(kFull, nreg)) {
-        const unsigned grp = __match_any_sync(kFull, nreg ? dw : -1 - lane);
-        if (nreg && lane == __ffs(grp) - 1) {
-          s.regm[dw * kCW + wid] |= grp;  // word (dw, wid) is written by this warp only
-          const int t1 = atomicAdd(&s.T[dw], __popc(grp)) + __popc(grp);
-          if (t1 >= s.ch[dw]) {
-            const unsigned bit = 1u << (dw & 31);
-            if (!(s.tm[dw >> 5] & bit)) atomicOr(&s.tm[dw >> 5], bit);
-            if (!(s.dm[dw >> 5] & bit)) atomicOr(&s.dm[dw >> 5], bit);
-          }
-        }
-      }
-      __syncthreads();
-      // 2. tight instances with new registrations: the slot of the chooser that takes the last
-      //    headroom (fpos) and of the first one that finds none (pp); the k-th such instance
-      //    goes to warp k mod kCW.  Both slots only move earlier while the instance is tight,
-      //    so the cut bound starts from the others' pp (set by step 3 of the last iteration).
+      // ---- 1. proposals, the leaders that choose packed into as few warps as hold them
       {
-        const unsigned word = s.tm[lane] & s.dm[lane];
-        const unsigned nzw = __ballot_sync(kFull, word != 0);
-        int seen = 0;
-        for (unsigned zz = nzw; zz; zz &= zz - 1) {
-          const int wi = __ffs(zz) - 1;
-          const unsigned bits = __shfl_sync(kFull, word, wi);
-          unsigned mine = 0;
-          for (unsigned t = bits; t; t &= t - 1) {
-            if ((seen & (kCW - 1)) == wid) mine |= t & (0u - t);
-            ++seen;
-          }
-          while (mine) {
-            const int w = 32 * wi + __ffs(mine) - 1;
-            mine &= mine - 1;
-            const int need = s.ch[w];
-            // lane j holds the registered choosers of w among slots [32 j, 32 j + 32)
-            const unsigned word = lane < kCW ? s.regm[w * kCW + lane] : 0u;
-            const int c = __popc(word);
-            int incl = c;
-#pragma unroll
-            for (int o = 1; o < kCW; o <<= 1) {
-              const int t = __shfl_up_sync(kFull, incl, o);
-              if (lane >= o) incl += t;
-            }
-            // slots of the need-th and (need + 1)-th registered choosers of w (kCT if fewer)
-            const unsigned mx1 = __ballot_sync(kFull, lane < kCW && incl >= need);
-            const unsigned mx2 = __ballot_sync(kFull, lane < kCW && incl > need);
-            const int l1 = mx1 ? __ffs(mx1) - 1 : 0, l2 = mx2 ? __ffs(mx2) - 1 : 0;
-            const unsigned w1 = __shfl_sync(kFull, word, l1), w2 = __shfl_sync(kFull, word, l2);
-            const int before1 = __shfl_sync(kFull, incl - c, l1), before2 = __shfl_sync(kFull, incl - c, l2);
-            const int f = mx1 ? 32 * l1 + nth_set(w1, need - 1 - before1) : kCT;
-            const int p = mx2 ? 32 * l2 + nth_set(w2, need - before2) : kCT;
-            if (lane == 0) {
-              s.fpos[w] = f;
-              s.pp[w] = p;
-              if (p < kCT) atomicMin(&s_qb[par], p);
-            }
-          }
-        }
+        const unsigned m = __ballot_sync(kFull, need);
+        int at = 0;
+        if (lane == 0 && m) at = atomicAdd(&s_queued, __popc(m));
+        at = __shfl_sync(kFull, at, 0);
+        if (need) s.queue[at + __popc(m & lanemask_lt())] = (uint16_t)tid;
       }
       __syncthreads();
-      const int q = min(s_qb[par], qcut);
-      // 3. the leaders before q are decided; warp 0 takes the instances whose last headroom
-      //    went to one of them out of the envelope, and sets the next iteration's cut bound
-      if (act && tid < q) {
-        if (dec == MISAT_ADMIT_NEW || dec == MISAT_ADMIT_CONT) {
-          a.rq.status[r] = kStResolved;
-          a.rq.inst[r] = dw;
-          a.rq.reason[r] = dec;
-        } else {
-          a.rq.status[r] = kStHeld;
-          a.rq.inst[r] = -1;
-          a.rq.last_reason[r] = dec;
+      if (tid < s_queued) {
+        const int t = s.queue[tid];
+        const int c = sel_choose(s, a, tc_min, T, t, cta * T + t);
+        s.lch[t] = (int16_t)c;
+        if (c >= 0 && c != (int)(s.lcp[t] & 0xffffu) - 1) {
+          atomicOr(&s.prop[c * NW + (t >> 5)], 1u << (t & 31));
+          const int cb = (int)((s.lx[t] >> 20) & 3);
+          atomicAdd(cb == 2 ? &s.n2[c] : &s.n01[c], cb == 1 ? 1u << 16 : 1u);
         }
       }
-      if (wid == 0) {
-        const unsigned word = s.tm[lane];
-        unsigned out = 0;
-        int mn = kCT;
-        for (unsigned t = word; t; t &= t - 1) {  // lane-local: the tight instances of word `lane`
-          const int w = 32 * lane + __ffs(t) - 1;
-          if (s.fpos[w] < q) {
-            out |= t & (0u - t);
-            s.fpos[w] = kCT;
-            s.pp[w] = kCT;
-          } else {
-            mn = min(mn, s.pp[w]);
+      cluster_barrier(cs);
+      // ---- 2. thresholds of the instances this warp owns
+      if (tid == 0) {
+        s_changed[par ^ 1] = 0;
+        s_queued = 0;
+      }
+      bool moved = false;
+      for (int o = wid; o * cs + cta < W; o += NW) {
+        const int w = o * cs + cta;
+        const int4 h4 = s.hr[o];
+        const unsigned seen = s.seen[o];
+        if (h4.w <= 0) continue;
+        // lane c: CTA c's proposals per class; totals
+        unsigned p01 = 0, p2 = 0;
+        if (lane < cs) {
+          p01 = ld_cluster(map_rank(sm_n01 + 4 * w, lane));
+          p2 = ld_cluster(map_rank(sm_n2 + 4 * w, lane));
+        }
+        const unsigned t01 = __reduce_add_sync(kFull, p01), t2 = __reduce_add_sync(kFull, p2);
+        const int n[3] = {(int)(t01 & 0xffffu), (int)(t01 >> 16), (int)t2};
+        const int h[3] = {h4.x, h4.y, h4.z};
+        const unsigned all = (unsigned)(n[0] + n[1] + n[2]);
+        // proposals are only added: the same number is the same set
+        if (all == seen || !((h[0] > 0 && n[0] >= h[0]) || (h[1] > 0 && n[1] >= h[1]) ||
+                             (h[2] > 0 && n[2] >= h[2]) || (int)all >= h4.w))
+          continue;
+        // per class: the position of its h-th proposal, through a scan over the CTAs and one over
+        // the words of the CTA it is in; the three classes go through the same instructions
+        // side by side (two share a register in the scans)
+        unsigned i01 = p01, i2 = p2;
+        warp_scan_pair(&i01, &i2);
+        const int own[3] = {(int)(p01 & 0xffffu), (int)(p01 >> 16), (int)p2};
+        const int inc[3] = {(int)(i01 & 0xffffu), (int)(i01 >> 16), (int)i2};
+        int src[3], rank[3];
+        unsigned x[3];
+#pragma unroll
+        for (int bb = 0; bb < 3; ++bb) {
+          const unsigned hit = __ballot_sync(kFull, inc[bb] >= h[bb]);
+          src[bb] = hit ? __ffs(hit) - 1 : 0;
+          rank[bb] = h[bb] - 1 - __shfl_sync(kFull, inc[bb] - own[bb], src[bb]);
+        }
+#pragma unroll
+        for (int bb = 0; bb < 3; ++bb)
+          x[bb] = lane < NW && h[bb] > 0 && n[bb] >= h[bb]
+                      ? ld_cluster(map_rank(sm_prop + 4 * (w * NW + lane), src[bb])) & s.cm[bb * words + src[bb] * NW + lane]
+                      : 0u;
+        const int pc[3] = {__popc(x[0]), __popc(x[1]), __popc(x[2])};
+        unsigned q01 = (unsigned)pc[0] | ((unsigned)pc[1] << 16), q2 = (unsigned)pc[2];
+        warp_scan_pair(&q01, &q2);
+        const int win[3] = {(int)(q01 & 0xffffu), (int)(q01 >> 16), (int)q2};
+        int t[3], kept = 0;  // kept: lane c's proposals that pass the class quotas
+#pragma unroll
+        for (int bb = 0; bb < 3; ++bb) {
+          const unsigned hit = __ballot_sync(kFull, win[bb] > rank[bb]);
+          const int i = hit ? __ffs(hit) - 1 : 0;
+          const int k = rank[bb] - __shfl_sync(kFull, win[bb] - pc[bb], i);
+          const unsigned y = __shfl_sync(kFull, x[bb], i);
+          const unsigned bit = __ballot_sync(kFull, ((y >> lane) & 1u) && __popc(y & lanemask_lt()) == k);
+          const bool full = n[bb] >= h[bb];
+          t[bb] = h[bb] <= 0 ? -1 : (full ? 32 * (src[bb] * NW + i) + __ffs(bit) - 1 : kNever);
+          kept += h[bb] <= 0 ? 0 : (!full || lane < src[bb] ? own[bb] : (lane == src[bb] ? rank[bb] + 1 : 0));
+        }
+        int tgw = kNever;
+        // the proposals that pass the class quotas count against the global one
+        if ((int)all >= h4.w && (int)__reduce_add_sync(kFull, (unsigned)kept) >= h4.w) {
+          int r = h4.w - 1;
+          const int c = find_cta(kept, &r);
+          unsigned y = 0;
+          if (lane < NW) {
+            const int q = c * NW + lane;
+            y = ld_cluster(map_rank(sm_prop + 4 * (w * NW + lane), c)) &
+                ((s.cm[q] & upto_mask(q, t[0])) | (s.cm[words + q] & upto_mask(q, t[1])) |
+                 (s.cm[2 * words + q] & upto_mask(q, t[2])));
           }
-        }
-        s.tm[lane] = word & ~out;
-        s.dm[lane] = 0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mn = min(mn, __shfl_xor_sync(kFull, mn, o));
-        if (lane == 0) s_qb[par ^ 1] = mn;  // last read before the barrier above
-        // instances that ran out, in index order
-        int cnt = __popc(out), excl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int v = __shfl_up_sync(kFull, excl, o);
-          if (lane >= o) excl += v;
-        }
-        const int nrem = __shfl_sync(kFull, excl, 31);
-        excl -= cnt;
-        if (lane == 0) s_navail -= nrem;
-        for (unsigned t = out; t; t &= t - 1) {
-          const int w = 32 * lane + __ffs(t) - 1;
-          s.av[w] = 0;
-          s.rem[excl++] = w;
+          tgw = find_pos(y, r, c * NW);
         }
         __syncwarp();
-        for (int e = 0; e < nrem; ++e) cls_repair(s, W, s.rem[e], &s_hm, &s_first_a, &s_last_s, a.small);
+        if (lane == 0) s.seen[o] = all;
+#pragma unroll
+        for (int bb = 0; bb < 3; ++bb) t[bb] = min(t[bb], tgw);
+        if (t[0] != s.te[w] || t[1] != s.te[W + w] || t[2] != s.te[2 * W + w] || tgw != s.tg[w]) {
+          moved = true;
+          __syncwarp();
+          for (int i = lane; i < 4 * cs; i += 32) {
+            const int bb = i / cs, rank = i - bb * cs;
+            st_cluster_u16(map_rank(bb < 3 ? sm_te + 2 * (bb * W + w) : sm_tg + 2 * w, rank),
+                           bb == 0 ? t[0] : (bb == 1 ? t[1] : (bb == 2 ? t[2] : tgw)));
+          }
+        }
       }
-      __syncthreads();
-      done = q;
+      if (moved && lane < cs) st_cluster(map_rank(sm_changed + 4 * par, lane), 1u);
+      cluster_barrier(cs);
+      // ---- 3. refusals
+      const bool changed = *(volatile int*)&s_changed[par] != 0;
       par ^= 1;
+      if (changed) {
+        if (++guard > 4 * W + 4) {  // at least one event becomes exact per round (uniform over the cluster)
+          if (tid == 0) set_error(a.err, MISAT_ERR_INTERNAL);
+          return;
+        }
+        const int c = s.lch[tid];
+        need = valid && (c == kWait || (c >= 0 && c != pw && s.te[b * W + c] < pos));
+        continue;
+      }
+      // settled: the first Eq. (7) leader whose cached instance filled up after it had
+      // proposed elsewhere, where waiting is cheaper
+      if (!__syncthreads_or(eq7) && cs == 1) break;
+      {
+        if (tid == 0) s_fixmin = kNever;
+        __syncthreads();
+        const int c = s.lch[tid];
+        if (eq7 && c >= 0) {
+          const int4 q0 = a.rec[s.lrec[tid]], q1 = a.rec[s.lrec[tid] + 1];
+          const int whit = 65535 - (q0.w & 0xffff);
+          const int64_t theta = ((int64_t)q1.w << 32) | (uint32_t)q1.z;
+          if (c != whit && s.te[b * W + whit] <= pos && s.ln[c].x > theta) atomicMin(&s_fixmin, pos);
+        }
+        __syncthreads();
+        if (tid < cs) st_cluster(map_rank(sm_fix + 4 * cta, tid), (uint32_t)s_fixmin);
+        cluster_barrier(cs);
+      }
+      int fix = kNever;
+      for (int i = 0; i < cs; ++i) fix = min(fix, *(volatile int*)&s_fix[i]);
+      if (fix == kNever) break;
+      // that leader waits; thresholds at or behind it are lifted (every CTA its own copy), its
+      // proposal and those behind it withdrawn, and the leaders behind it start over
+      for (int w = tid; w < W; w += T) {
+        unsigned k01 = 0, k2 = 0;
+        for (int i = 0; i < NW; ++i) {
+          const int q = cta * NW + i;
+          const unsigned x = s.prop[w * NW + i] & upto_mask(q, fix - 1);
+          s.prop[w * NW + i] = x;
+          k01 += __popc(x & s.cm[q]) + (__popc(x & s.cm[words + q]) << 16);
+          k2 += __popc(x & s.cm[2 * words + q]);
+        }
+        s.n01[w] = k01;
+        s.n2[w] = k2;
+        if (w % cs == cta) s.seen[w / cs] = 0;
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+          if (s.te[i * W + w] >= fix) s.te[i * W + w] = kNever;
+        if (s.tg[w] >= fix) s.tg[w] = kNever;
+      }
+      if (pos == fix) s.lch[tid] = kFixed;
+      need = valid && pos > fix;
+      if (need) {
+        s.lch[tid] = kNone;
+        s.lpos[tid] &= 0xffffu;
+        s.lcp[tid] = (s.lcp[tid] & 0xffffu) | ((a.rec[s.lrec[tid] + 1].x > 0 ? 0u : kTop + 1u) << 16);
+      }
+      guard = 0;
+      cluster_barrier(cs);  // every CTA has read s_fix and lifted its copies
     }
-    // end of the window: every tight instance ran out (its last headroom went to a decided
-    // leader); the others lose the window's admissions
-    for (int w = tid; w < W; w += kCT) {
-      s.ch[w] = s.av[w] ? s.ch[w] - s.T[w] : 0;
-      s.T[w] = 0;
+    // ---- the window's decisions; behind position s_tgmax no instance has global headroom
+    if (tid == 0) s_tgmax = -1;
+    __syncthreads();
+    for (int w = tid; w < W; w += T)
+      if (s.tg[w] >= 0) atomicMax(&s_tgmax, (int)s.tg[w]);
+    __syncthreads();
+    if (valid) decide(a.rec[s.lrec[tid] + 1].y, s.lch[tid], pw, s_tgmax > pos);
+    const bool more = base + cs * T < nl;
+    // headroom left after the window (accepted proposals lie at or before their threshold)
+    for (int o = wid; o * cs + cta < W; o += NW) {
+      const int w = o * cs + cta;
+      unsigned used01 = 0, used2 = 0;
+      for (int q = lane; q < words; q += 32) {
+        const unsigned v = ld_cluster(map_rank(sm_prop + 4 * (w * NW + q % NW), q / NW));
+        used01 += __popc(v & s.cm[q] & upto_mask(q, s.te[w])) +
+                  (__popc(v & s.cm[words + q] & upto_mask(q, s.te[W + w])) << 16);
+        used2 += __popc(v & s.cm[2 * words + q] & upto_mask(q, s.te[2 * W + w]));
+      }
+      used01 = __reduce_add_sync(kFull, used01);
+      used2 = __reduce_add_sync(kFull, used2);
+      if (lane == 0) {
+        int4 h = s.hr[o];
+        h.x -= (int)(used01 & 0xffffu);
+        h.y -= (int)(used01 >> 16);
+        h.z -= (int)used2;
+        const int all = (int)(used01 & 0xffffu) + (int)(used01 >> 16) + (int)used2;
+        h.w -= all;
+        s.hr[o] = h;
+        // an instance that had global headroom ran out of it
+        if (all && h.w <= 0) a.stats[25] = 1;
+      }
     }
-    for (int i = tid; i < W * kCW; i += kCT) s.regm[i] = 0;
-    if (tid == 0) s_qb[0] = kCT;
-    __syncthreads();  // s_lead / s_sens are rewritten by the next window
+    cluster_barrier(cs);
+    if (!more) break;
+    for (int o = wid; o * cs + cta < W; o += NW) {
+      const int w = o * cs + cta;
+      const int4 h = s.hr[o];
+      for (int i = lane; i < 4 * cs; i += 32) {
+        const int bb = i / cs, rank = i - bb * cs;
+        const bool left = h.w > 0 && (bb == 0 ? h.x : (bb == 1 ? h.y : (bb == 2 ? h.z : 1))) > 0;
+        st_cluster_u16(map_rank(bb < 3 ? sm_te + 2 * (bb * W + w) : sm_tg + 2 * w, rank), left ? kNever : -1);
+      }
+      if (lane == 0) s.seen[o] = 0;
+    }
+    for (int i = tid; i < W * NW; i += T) s.prop[i] = 0;
+    for (int w = tid; w < W; w += T) {
+      s.n01[w] = 0;
+      s.n2[w] = 0;
+    }
+    cluster_barrier(cs);
   }
-  // admissions per instance, and the check that no instance ran out of global headroom
-  for (int w = tid; w < W; w += kCT) {
-    const int c0 = a.gh[w] > 0 ? a.ch[w * 3 + b] : 0;
-    const int used = c0 - s.ch[w];
-    if (used) atomicAdd(&a.adm[w], used);
-  }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) s_last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (s_last) {
-    __threadfence();
-    bool bad = false;
-    for (int w = tid; w < W; w += kCT) {
-      const int g = a.gh[w];
-      if (g > 0 && __ldcg(&a.adm[w]) >= g) bad = true;
-    }
-    if (__syncthreads_or(bad) && tid == 0) {
-      *a.coupled = 1;
-      a.stats[25] = 1;
-    }
-  }
+  // no CTA leaves while another may still read its shared memory: the last access to another
+  // CTA's is before the barrier that ends the last window (or before the loop)
 }
 
-cudaError_t select_class_configure() {
-  return cudaFuncSetAttribute(k4_select_class, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)select_class_smem_bytes(kMaxW, 256 * kMaxBatchBlocks));
+namespace {
+
+// CTAs and threads of the selection cluster for a batch of n requests: one CTA while the
+// leaders fit it (its barriers are block barriers), then as many CTAs as a cluster takes with
+// as few threads as hold the batch (a round's choices share an SM's issue slots), then windows
+// of 16 x 1024.
+void select_shape(int n, int max_cs, int* cs, int* threads) {
+  *cs = 1;
+  if (n <= 1024) {
+    *threads = n <= 256 ? 256 : (n <= 512 ? 512 : 1024);
+    return;
+  }
+  *cs = max_cs;
+  *threads = 256;
+  while (*threads < 1024 && *cs * *threads < n) *threads <<= 1;
 }
 
-void launch_select_class(const SelectClassArgs& a, cudaStream_t st) {
+}  // namespace
+
+cudaError_t select_configure(int* max_cluster) {
+  // sized for the largest instance count and batch, so that contexts of any size share the setting
+  cudaError_t e = cudaFuncSetAttribute(k4_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelSmemMax);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k4_select, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  // 16 CTAs per cluster where the device can hold one, else the portable 8
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 16;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3(16);
+  lc.blockDim = dim3(1024);
+  lc.dynamicSmemBytes = kSelSmemMax;
+  lc.attrs = &at;
+  lc.numAttrs = 1;
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, k4_select, &lc) != cudaSuccess) {
+    cudaGetLastError();
+    clusters = 0;
+  }
+  *max_cluster = clusters > 0 ? 16 : 8;
+  return cudaSuccess;
+}
+
+void launch_select(const SelectArgs& a, int max_cluster, cudaStream_t st) {
   if (a.n <= 0) return;
-  k4_select_class<<<3, kCT, select_class_smem_bytes(a.W, a.n), st>>>(a);
+  int cs, threads;
+  select_shape(a.n, max_cluster, &cs, &threads);
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = cs;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3(cs);
+  lc.blockDim = dim3(threads);
+  lc.dynamicSmemBytes = sel_smem_layout(a.W, cs, threads / 32, (a.n + 255) / 256, nullptr, nullptr);
+  lc.stream = st;
+  lc.attrs = &at;
+  lc.numAttrs = 1;
+  cudaLaunchKernelEx(&lc, k4_select, a, cs);
 }
 
 }  // namespace misat
