@@ -19,7 +19,8 @@ namespace {
 
 
 // Small device block copied to the host in one transfer after each route / commit.
-// Layout (8-byte words): stats[32] | U[W] | size[W] | sess_used | err | cand[3] | work | n_hits
+// Layout (8-byte words): stats[32] | U[W] | size[W] | sess_used | err | cand[3] | work (counters of the
+// block hash) | n_hits | g_used
 struct MetaLayout {
   size_t stats = 0, U = 0, size = 0, sess_used = 0, err = 0, cand = 0, work = 0, n_hits = 0, g_used = 0, words = 0;
   void init(int W) {
@@ -30,7 +31,7 @@ struct MetaLayout {
     err = sess_used + 1;
     cand = err + 1;
     work = cand + 3;
-    n_hits = work + 1;
+    n_hits = work + (kHashCtrs + 1) / 2;
     g_used = n_hits + 1;
     words = g_used + 1;
   }
@@ -129,6 +130,7 @@ struct misat_ctx {
   unsigned long long* d_bm_key = nullptr;
   int32_t* d_bm_val = nullptr;
   int4* d_sel_rec = nullptr;     // leader records of the selection, compact per block of 256 requests
+  int32_t* d_hash_list = nullptr;  // [max_batch] longer prompts, for the block hash
   int32_t* d_sel_cnt = nullptr;  // [blocks] leaders per block
   uint16_t* d_orders = nullptr;  // [kPriceCells][W] price orders
   int select_cluster = 8;        // largest cluster of the selection kernel
@@ -611,7 +613,7 @@ void enqueue_route(misat_ctx* c, const misat_batch* b, misat_decisions* out, cud
   // reset the per-batch counters: stats, U, cand, work, n_hits (size and sess_used persist)
   cudaMemsetAsync(c->d_meta + c->ml.stats, 0, 32 * 8, st);
   cudaMemsetAsync(c->d_meta + c->ml.U, 0, c->W * 8, st);
-  cudaMemsetAsync(c->d_meta + c->ml.cand, 0, 5 * 8, st);
+  cudaMemsetAsync(c->d_meta + c->ml.cand, 0, (c->ml.g_used - c->ml.cand) * 8, st);
   const int bm_log2 = std::max(1, ceil_log2(2 * (uint64_t)n));
   cudaMemsetAsync(c->d_bm_key, 0, ((size_t)1 << bm_log2) * 8, st);
   cudaMemsetAsync(c->d_bm_val, 0x7f, ((size_t)1 << bm_log2) * 4, st);
@@ -636,6 +638,9 @@ void enqueue_route(misat_ctx* c, const misat_batch* b, misat_decisions* out, cud
   pa.bm_val = c->d_bm_val;
   pa.bm_log2 = (uint32_t)bm_log2;
   pa.cand = c->cand_ptr();
+  pa.hash_ctr = c->work_ptr();
+  pa.hash_list = c->d_hash_list;
+  pa.hash_long = hash_long_blocks(b->n_tokens, c->num_sms);
   pa.err = c->err_ptr();
   launch_prologue(pa, st);
   c->mark(1, st);
@@ -648,7 +653,8 @@ void enqueue_route(misat_ctx* c, const misat_batch* b, misat_decisions* out, cud
   ha.seed = c->seed;
   ha.keys = c->d_keys;
   ha.keys_cap = c->keys_cap;
-  ha.work = c->work_ptr();
+  ha.ctr = c->work_ptr();
+  ha.list = c->d_hash_list;
   ha.err = c->err_ptr();
   launch_block_hash(ha, c->num_sms, st);
   c->mark(2, st);
@@ -868,7 +874,7 @@ int misat_create(const misat_config* cfg, void* cuda_stream, misat_ctx** out) {
       (rc = dalloc_n(c, &c->d_bm_val, (size_t)1 << bm_log2)) || (rc = dalloc_n(c, &c->d_sel_rec, kSelectRecInt4 * NB)) ||
       (rc = dalloc_n(c, &c->d_sel_cnt, (NB + 255) / 256)) ||
       (rc = dalloc_n(c, &c->d_orders, (size_t)kPriceCells * price_order_stride(W))) || (rc = dalloc_n(c, &c->d_skip, NB)) ||
-      (rc = dalloc_n(c, &c->d_grp, (size_t)1 << bm_log2)) ||
+      (rc = dalloc_n(c, &c->d_hash_list, NB)) || (rc = dalloc_n(c, &c->d_grp, (size_t)1 << bm_log2)) ||
       (rc = dalloc_n(c, &c->rq.nb, NB)) || (rc = dalloc_n(c, &c->rq.kbase, NB)) || (rc = dalloc_n(c, &c->rq.L, NB)) ||
       (rc = dalloc_n(c, &c->rq.cls, NB)) || (rc = dalloc_n(c, &c->rq.session, NB)) ||
       (rc = dalloc_n(c, &c->rq.sst, NB)) || (rc = dalloc_n(c, &c->rq.sinst, NB)) ||
@@ -988,7 +994,7 @@ int misat_route(misat_ctx* c, const misat_batch* b, misat_decisions* out) {
     // the caps of an empty batch are still defined (no candidate sessions)
     CK(cudaMemsetAsync(c->d_meta + c->ml.stats, 0, 32 * 8, st));
     CK(cudaMemsetAsync(c->d_meta + c->ml.U, 0, c->W * 8, st));
-    CK(cudaMemsetAsync(c->d_meta + c->ml.cand, 0, 5 * 8, st));
+    CK(cudaMemsetAsync(c->d_meta + c->ml.cand, 0, (c->ml.g_used - c->ml.cand) * 8, st));
     launch_caps(caps_args(c), st);
     CK(cudaGetLastError());
     CK(enqueue_meta(c));
@@ -1478,7 +1484,6 @@ int misat_load_chains(misat_ctx* c, int32_t n_chains, const int64_t* tok_off, co
   CK(cudaMemcpyAsync(c->rq.session, seq, (size_t)n_chains * 8, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(c->d_chain_max, max_blocks, (size_t)n_chains * 4, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(c->d_out_hit, arr, (size_t)n_chains * 4, cudaMemcpyHostToDevice, st));
-  CK(cudaMemsetAsync(c->work_ptr(), 0, 4, st));
   HashArgs ha{};
   ha.tok_off = c->d_stage_off;
   ha.tokens = c->d_stage_tok;
@@ -1487,8 +1492,11 @@ int misat_load_chains(misat_ctx* c, int32_t n_chains, const int64_t* tok_off, co
   ha.seed = c->seed;
   ha.keys = c->d_keys;
   ha.keys_cap = c->keys_cap;
-  ha.work = c->work_ptr();
+  ha.ctr = c->work_ptr();
+  ha.list = c->d_hash_list;
+  ha.long_blocks = hash_long_blocks(ntok, c->num_sms);
   ha.err = c->err_ptr();
+  launch_hash_lists(ha, st);
   launch_block_hash(ha, c->num_sms, st);
   InsertArgs ia{};
   ia.desc = c->d_desc;

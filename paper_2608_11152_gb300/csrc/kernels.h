@@ -10,18 +10,45 @@
 namespace misat {
 
 // ---- K1 ----
+// Counters of the block hash: prompts on the list, and those handed out.
+enum { kHashNLong, kHashNMid, kHashWLong, kHashWMid, kHashWGroup, kHashCtrs };
+constexpr int kHashShort = 31;  // blocks up to which a prompt is hashed with its neighbours
 struct HashArgs {
   const int64_t* tok_off;
   const int32_t* tokens;
   int64_t n_tokens;
   int32_t n;
   uint64_t seed;
-  uint64_t* keys;       // key of (r, j) at floor(tok_off[r]/16) + j
+  uint64_t* keys;       // key of (r, j) at floor(tok_off[r]/16) + j, or compact
   int64_t keys_cap;
-  unsigned* work;       // zeroed before the launch
+  uint32_t* off;        // NULL, or compact key positions within a tile of requests,
+  uint32_t* tile;       //   and those of the tiles
+  unsigned* ctr;        // [kHashCtrs], zeroed before the prompts are listed
+  int32_t* list;        // [n] long prompts from the front, middle ones from the back (hash_list)
+  int32_t long_blocks;  // prompts of at least as many blocks are long (hash_long_blocks)
+  int32_t group;        // requests per group of short prompts (set by the launcher)
   const int32_t* err;
 };
-void launch_block_hash(const HashArgs& a, int num_sms, cudaStream_t st);
+int32_t hash_long_blocks(int64_t n_tokens, int num_sms);
+void launch_hash_lists(const HashArgs& a, cudaStream_t st);  // where the prologue does not list them
+void launch_block_hash(HashArgs a, int num_sms, cudaStream_t st);
+
+// Puts a prompt of nb blocks on the hash's lists (every lane of the warp calls; positions by
+// ballot, one atomic per warp and list).
+__device__ __forceinline__ void hash_list(unsigned* ctr, int32_t* list, int32_t n, int r, int32_t nb,
+                                          int32_t long_blocks) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const bool mine = nb > kHashShort && (nb >= long_blocks) == (c == 0);
+    const unsigned m = __ballot_sync(0xffffffffu, mine);
+    if (!m) continue;
+    unsigned at = 0;
+    if (lane == 0) at = atomicAdd(ctr + (c == 0 ? kHashNLong : kHashNMid), (unsigned)__popc(m));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & lanemask_lt());
+    if (mine) list[c == 0 ? at : n - 1 - at] = r;
+  }
+}
 
 // ---- per-request derived data shared by the route and commit kernels ----
 struct ReqArrays {
@@ -100,6 +127,9 @@ struct PrologueArgs {
   int32_t* bm_val;
   uint32_t bm_log2;
   long long* cand;             // [3]
+  unsigned* hash_ctr;          // lists of the block hash (hash_list)
+  int32_t* hash_list;
+  int32_t hash_long;
   int32_t* err;
 };
 void launch_prologue(const PrologueArgs& a, cudaStream_t st);

@@ -11,17 +11,22 @@ namespace misat {
 // insert them into a batch-local map that keeps each session's first arrival.
 __global__ void __launch_bounds__(256) k0_prologue(PrologueArgs a) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= a.n) return;
-  const uint8_t c = a.cls[r];
-  const uint64_t s = a.session[r];
-  const int64_t t0 = a.tok_off[r], t1 = a.tok_off[r + 1];
-  bool ok = c < 3 && s != 0 && t0 >= 0 && t1 >= t0 && t1 <= a.n_tokens && (t1 - t0) < (1 << 20);
-  if (r == 0 && t0 != 0) ok = false;
-  if (r == a.n - 1 && t1 != a.n_tokens) ok = false;
-  if (!ok) {
-    set_error(a.err, MISAT_ERR_INVALID_ARG);
-    return;
+  bool ok = r < a.n;
+  uint8_t c = 0;
+  uint64_t s = 0;
+  int64_t t0 = 0, t1 = 0;
+  if (ok) {
+    c = a.cls[r];
+    s = a.session[r];
+    t0 = a.tok_off[r];
+    t1 = a.tok_off[r + 1];
+    ok = c < 3 && s != 0 && t0 >= 0 && t1 >= t0 && t1 <= a.n_tokens && (t1 - t0) < (1 << 20);
+    if (r == 0 && t0 != 0) ok = false;
+    if (r == a.n - 1 && t1 != a.n_tokens) ok = false;
+    if (!ok) set_error(a.err, MISAT_ERR_INVALID_ARG);
   }
+  hash_list(a.hash_ctr, a.hash_list, a.n, r, ok ? (int32_t)((t1 - t0) >> 4) : 0, a.hash_long);
+  if (!ok) return;
   const int32_t L = (int32_t)(t1 - t0);
   a.rq.nb[r] = L >> 4;
   a.rq.kbase[r] = t0 >> 4;
