@@ -205,7 +205,7 @@ struct misat_ctx {
       entries.clear();
       pending.clear();
     }
-  } g_evict, g_evict_apply, g_route;
+  } g_route;
   int64_t* d_params = nullptr;  // [9] per-route class parameters (caps)
   // the commit's global-index pass runs on a side stream, beside the session update and
   // the read-only half of the eviction, and joins before the deletions
@@ -568,24 +568,20 @@ EvictArgs evict_args(misat_ctx* c, unsigned long long* evicted_counter) {
   return ev;
 }
 
-// Eviction of every instance above capacity; `join` (may be NULL) is waited for between the
-// read-only half and the deletions.
+// Eviction of every instance above capacity (d_nact zeroed before); `join` (may be NULL) is waited
+// for between the read-only half and the deletions.
 int evict_all(misat_ctx* c, unsigned long long* evicted_counter, cudaEvent_t join = nullptr) {
   const EvictArgs ev = evict_args(c, evicted_counter);
   // streaming CTAs per instance: about 4 buckets per thread, at most 256 CTAs of 256
   uint32_t maxlg = 1;
   for (auto& d : c->h_desc) maxlg = std::max(maxlg, d.log2nb);
   const int chunks = (int)std::min<uint64_t>(256, std::max<uint64_t>(1, ((uint64_t)1 << maxlg) / (4 * 256)));
-  const std::vector<uint64_t> key{(uint64_t)chunks, reinterpret_cast<uint64_t>(ev.gix.keys),
-                                  (uint64_t)ev.gix.log2nb, reinterpret_cast<uint64_t>(evicted_counter)};
-  // with phase timing the kernels are launched directly with an event after each
+  // with phase timing there is an event after each kernel
   const cudaEvent_t* marks = c->timing ? c->ev + 12 : nullptr;
-  int rc = run_graph(c, c->g_evict, key,
-                     [&](cudaStream_t s) { launch_evict_select(ev, chunks, c->num_sms, s, marks); });
-  if (rc) return rc;
+  launch_evict_select(ev, chunks, c->num_sms, c->stream, marks);
   if (join) CK(cudaStreamWaitEvent(c->stream, join, 0));
-  return run_graph(c, c->g_evict_apply, key,
-                   [&](cudaStream_t s) { launch_evict_apply(ev, c->num_sms, s, marks ? marks + 3 : nullptr); });
+  launch_evict_apply(ev, c->num_sms, c->stream, marks ? marks + 3 : nullptr);
+  return cudaGetLastError() == cudaSuccess ? MISAT_OK : MISAT_ERR_CUDA;
 }
 
 CapsArgs caps_args(misat_ctx* c) {
@@ -606,24 +602,50 @@ CapsArgs caps_args(misat_ctx* c) {
   return ca;
 }
 
-// The device work of one route (n > 0), enqueued on stream st: counters reset, prologue,
+// Slots of the batch-local tables of n requests (log2, at least four).
+int batch_log2(int32_t n) { return std::max(2, ceil_log2(2 * (uint64_t)n)); }
+
+// Class parameters and cleared scratch of a route: the counters of a batch (size and sess_used
+// persist) and, for n > 0, its tables.
+void enqueue_clear(misat_ctx* c, int32_t n, cudaStream_t st) {
+  ClearArgs a{};
+  for (int i = 0; i < 3; ++i) {
+    a.v[i] = c->kbar_b[i];
+    a.v[3 + i] = c->T_b[i];
+    a.v[6 + i] = (int64_t)c->rho[i];
+  }
+  a.params = c->d_params;
+  a.words[0] = c->d_meta + c->ml.stats;
+  a.n_words[0] = (int32_t)(c->ml.size - c->ml.stats);
+  a.words[1] = c->d_meta + c->ml.cand;
+  a.n_words[1] = (int32_t)(c->ml.g_used - c->ml.cand);
+  if (n > 0) {
+    const uint32_t slots = 1u << batch_log2(n);
+    a.run[0] = reinterpret_cast<uint4*>(c->d_bm_key);
+    a.n_run[0] = slots / 2;
+    a.run[1] = reinterpret_cast<uint4*>(c->d_bm_val);
+    a.n_run[1] = slots / 4;
+    a.fill[1] = 0x7f7f7f7fu;
+    a.run[2] = reinterpret_cast<uint4*>(c->d_grp);
+    a.n_run[2] = slots;
+    if (c->fb.keys) {
+      a.run[3] = reinterpret_cast<uint4*>(c->fb.keys);
+      a.n_run[3] = slots / 2;
+    }
+  }
+  launch_clear(a, c->num_sms, st);
+}
+
+// The device work of one route (n > 0) behind enqueue_clear, enqueued on stream st: prologue,
 // block hash, caps, probes, serial selection, finalize.  Captured into the route graph, or
 // launched directly while the caller captures the context's stream.
 void enqueue_route(misat_ctx* c, const misat_batch* b, misat_decisions* out, cudaStream_t st) {
   const int32_t n = b->n;
-  // reset the per-batch counters: stats, U, cand, work, n_hits (size and sess_used persist)
-  cudaMemsetAsync(c->d_meta + c->ml.stats, 0, 32 * 8, st);
-  cudaMemsetAsync(c->d_meta + c->ml.U, 0, c->W * 8, st);
-  cudaMemsetAsync(c->d_meta + c->ml.cand, 0, (c->ml.g_used - c->ml.cand) * 8, st);
-  const int bm_log2 = std::max(1, ceil_log2(2 * (uint64_t)n));
-  cudaMemsetAsync(c->d_bm_key, 0, ((size_t)1 << bm_log2) * 8, st);
-  cudaMemsetAsync(c->d_bm_val, 0x7f, ((size_t)1 << bm_log2) * 4, st);
-  cudaMemsetAsync(c->d_grp, 0, ((size_t)1 << bm_log2) * sizeof(ulonglong2), st);
+  const int bm_log2 = batch_log2(n);
   GIndex fb{};
   if (c->fb.keys) {
     fb = c->fb;
-    fb.log2nb = (uint32_t)std::max(0, bm_log2 - 2);
-    cudaMemsetAsync(fb.keys, 0, ((size_t)4 << fb.log2nb) * 8, st);
+    fb.log2nb = (uint32_t)(bm_log2 - 2);
   }
 
   c->mark(0, st);
@@ -686,14 +708,13 @@ void enqueue_route(misat_ctx* c, const misat_batch* b, misat_decisions* out, cud
   c->mark(4, st);
   launch_probe_search(pr, c->num_sms, st);
   c->mark(5, st);
-  if (b->out_H)
-    cudaMemcpyAsync(b->out_H, c->d_H, (size_t)n * c->W * sizeof(uint16_t), cudaMemcpyDeviceToDevice, st);
 
   SelectPrepArgs sp{};
   sp.n = n;
   sp.W = c->W;
   sp.rq = c->rq;
   sp.H = c->d_H;
+  sp.out_H = reinterpret_cast<uint16_t*>(b->out_H);
   sp.backlog = c->d_backlog;
   sp.tokcost = c->d_tokcost;
   sp.gh = c->ia.gh;
@@ -702,7 +723,7 @@ void enqueue_route(misat_ctx* c, const misat_batch* b, misat_decisions* out, cud
   sp.rec = c->d_sel_rec;
   sp.segcnt = c->d_sel_cnt;
   sp.err = c->err_ptr();
-  launch_select_prep(sp, st);
+  launch_select_prep(sp, c->num_sms, st);
   SelectArgs sa{};
   sa.n = n;
   sa.W = c->W;
@@ -760,8 +781,6 @@ const char* misat_strerror(int code) {
 int misat_destroy(misat_ctx* c) {
   if (!c) return MISAT_ERR_INVALID_ARG;
   cudaStreamSynchronize(c->stream);
-  c->g_evict.clear();
-  c->g_evict_apply.clear();
   c->g_route.clear();
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->side_stream) {
@@ -867,7 +886,7 @@ int misat_create(const misat_config* cfg, void* cuda_stream, misat_ctx** out) {
   c->keys_cap = c->max_tokens / 16 + 1;
   c->units_cap = (int64_t)NB + c->keys_cap / 128 + 1;  // one unit per 128 blocks of a request
   c->hits_cap = (int64_t)std::min<size_t>(NB * Ws, (size_t)1 << 27);
-  const int bm_log2 = std::max(1, ceil_log2(2 * NB));
+  const int bm_log2 = batch_log2((int32_t)NB);
   if ((rc = dalloc_n(c, &c->d_meta, c->ml.words)) || (rc = dalloc_n(c, &c->d_keys, (size_t)c->keys_cap)) ||
       (rc = dalloc_n(c, &c->d_units, 2 * (size_t)c->units_cap)) || (rc = dalloc_n(c, &c->d_units_n, 1)) ||
       (rc = dalloc_n(c, &c->d_H, NB * Ws + 8)) || (rc = dalloc_n(c, &c->d_hits, (size_t)c->hits_cap)) ||
@@ -982,20 +1001,11 @@ int misat_route(misat_ctx* c, const misat_batch* b, misat_decisions* out) {
   estimate_classes(c);
   c->last_n = n;
   c->last_ntok = b->n_tokens;
-  c->grp_log2 = (uint32_t)std::max(1, ceil_log2(2 * (uint64_t)std::max(n, 1)));  // as enqueue_route
-  RouteParams prm{};
-  for (int i = 0; i < 3; ++i) {
-    prm.v[i] = c->kbar_b[i];
-    prm.v[3 + i] = c->T_b[i];
-    prm.v[6 + i] = (int64_t)c->rho[i];
-  }
-  launch_route_params(prm, c->d_params, st);
+  c->grp_log2 = (uint32_t)batch_log2(std::max(n, 1));  // as enqueue_route
+  enqueue_clear(c, n, st);
   CK(cudaGetLastError());
   if (n == 0) {
     // the caps of an empty batch are still defined (no candidate sessions)
-    CK(cudaMemsetAsync(c->d_meta + c->ml.stats, 0, 32 * 8, st));
-    CK(cudaMemsetAsync(c->d_meta + c->ml.U, 0, c->W * 8, st));
-    CK(cudaMemsetAsync(c->d_meta + c->ml.cand, 0, (c->ml.g_used - c->ml.cand) * 8, st));
     launch_caps(caps_args(c), st);
     CK(cudaGetLastError());
     CK(enqueue_meta(c));
@@ -1247,8 +1257,6 @@ int misat_commit(misat_ctx* c) {
     rc = maybe_rebuild_sessions(c, n);
     if (rc) return rc;
   }
-  CK(cudaMemsetAsync(c->stats_ptr() + 18, 0, 2 * 8, st));
-  CK(cudaMemsetAsync(c->stats_ptr() + 24, 0, 8, st));
   c->mark(8);
   if (n > 0) {
     InsertArgs ia{};
@@ -1274,6 +1282,8 @@ int misat_commit(misat_ctx* c) {
     ia.grp_log2 = c->grp_log2;
     ia.skip = c->d_skip;
     ia.ops = c->stats_ptr() + 24;
+    ia.n_act = c->d_nact;
+    ia.sess = SessUpdateArgs{c->rq, c->sess, c->d_prot};
     launch_insert_tables(ia, c->num_sms, st);
     c->mark(9);
     cudaEvent_t join = nullptr;
@@ -1289,8 +1299,6 @@ int misat_commit(misat_ctx* c) {
       }
     }
     c->mark(10);
-    SessUpdateArgs sa{n, c->rq, c->sess, c->d_prot, c->err_ptr()};
-    launch_session_update(sa, st);
     c->mark(11);
     int rc = evict_all(c, c->stats_ptr() + 19, join);
     if (rc) return rc;
@@ -1473,6 +1481,7 @@ int misat_evict(misat_ctx* c, int32_t w, const uint64_t* keys, int64_t n) {
 }
 
 static int load_common_evict(misat_ctx* c) {
+  CK(cudaMemsetAsync(c->d_nact, 0, sizeof(unsigned), c->stream));
   int rc = evict_all(c, c->stats_ptr() + 20);
   if (rc) return rc;
   CK(cudaStreamSynchronize(c->stream));

@@ -89,7 +89,7 @@ struct UnitRec {
 };
 
 __device__ __forceinline__ UnitRec load_unit(const int4* units, int64_t u) {
-  const int4 x = __ldg(units + 2 * u), y = __ldg(units + 2 * u + 1);
+  const int4 x = __ldcg(units + 2 * u), y = __ldcg(units + 2 * u + 1);
   UnitRec r;
   r.keys = reinterpret_cast<const unsigned long long*>(((uint64_t)(uint32_t)x.y << 32) | (uint32_t)x.x);
   r.tab = reinterpret_cast<Bucket*>(((uint64_t)(uint32_t)x.w << 32) | (uint32_t)x.z);
@@ -106,9 +106,48 @@ __device__ __forceinline__ void load_unit_keys(const UnitRec& u, int lane, uint6
   for (int k = 0; k < kIns; ++k) key[k] = lane + 32 * k < u.cnt ? __ldg(u.keys + lane + 32 * k) : 0;
 }
 
+// Session table update at commit (Sec. 4.1: an admitted new session becomes pending /
+// protected on its instance; a rebound one leaves its previous instance's count).
+// Only leaders with ADMIT_NEW change anything; each session has one leader per batch.
+__device__ __forceinline__ void update_session(const SessUpdateArgs& a, int r, int32_t* err) {
+  if (a.rq.leader[r] != r || a.rq.reason[r] != MISAT_ADMIT_NEW) return;
+  const uint64_t s = a.rq.session[r];
+  const int w = a.rq.inst[r];
+  const int b = a.rq.cls[r];
+  const uint64_t nv = sess_val(kSessProtected, (uint32_t)b, (uint32_t)w);
+  const uint32_t mask = (1u << a.st.log2n) - 1;
+  uint32_t h = sess_home(s, a.st.log2n);
+  for (uint32_t it = 0; it <= mask; ++it) {
+    SessSlot* sl = a.st.slots + h;
+    unsigned long long k = __ldcg(&sl->key);
+    if (k == 0) {
+      k = atomicCAS(&sl->key, 0ull, (unsigned long long)s);
+      if (k == 0) {
+        sl->val = nv;
+        atomicAdd(a.st.used, 1ull);
+        atomicAdd(&a.prot[w * 3 + b], 1);
+        return;
+      }
+    }
+    if (k == s) {
+      const uint64_t ov = sl->val;
+      if (sess_state(ov) == kSessProtected) atomicSub(&a.prot[sess_inst(ov) * 3 + sess_cls(ov)], 1);
+      sl->val = nv;
+      atomicAdd(&a.prot[w * 3 + b], 1);
+      return;
+    }
+    h = (h + 1) & mask;
+  }
+  set_error(err, MISAT_ERR_TABLE_FULL);
+}
+
+// The batch's units, and its session table update beside them (both a thread per request).
 __global__ void __launch_bounds__(256) k4_units(InsertArgs a) {
+  chain_wait();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
+  if (a.sess.rq.leader && r < a.n && *a.err == 0) update_session(a.sess, r, a.err);
+  __syncwarp();
   int u = 0, c = 0, w = 0, s0 = 0;
   if (r < a.n && *a.err == 0 && a.inst[r] >= 0) {
     w = a.inst[r];
@@ -165,6 +204,12 @@ __global__ void __launch_bounds__(256) k4_units(InsertArgs a) {
 // the common prefix, compared key by key (one warp per request, 32 keys per step).  An agentic
 // turn and the next turn of its session, or two samples of one prompt, share their prefix.
 __global__ void __launch_bounds__(256) k4_dedup(InsertArgs a) {
+  chain_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {  // list lengths of the kernels behind this one
+    *a.n_units = 0;
+    if (a.gix.keys) *a.n_gnew = 0;
+    if (a.n_act) *a.n_act = 0;
+  }
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= a.n) return;
@@ -208,6 +253,7 @@ __global__ void __launch_bounds__(256) k4_dedup(InsertArgs a) {
 
 __global__ void __launch_bounds__(kInsThreads, 3) k4_insert(InsertArgs a) {
   __shared__ unsigned s_new[kMaxW];  // new keys per instance, flushed once per CTA
+  chain_wait();
   if (block_error(a.err)) return;
   for (int i = threadIdx.x; i < a.n_inst; i += blockDim.x) s_new[i] = 0;
   __syncthreads();
@@ -290,6 +336,7 @@ __global__ void __launch_bounds__(kInsThreads, 3) k4_insert(InsertArgs a) {
 
 // Global index pass: bit w for every key new to instance w, one thread per listed key.
 __global__ void __launch_bounds__(256) k4_gix_insert(InsertArgs a) {
+  chain_wait();
   if (block_error(a.err)) return;
   const int64_t n = min((int64_t)__ldcg(a.n_gnew), a.gnew_cap);
   long long claimed = 0;
@@ -307,16 +354,21 @@ __global__ void __launch_bounds__(256) k4_gix_insert(InsertArgs a) {
 
 void launch_insert_tables(const InsertArgs& a, int num_sms, cudaStream_t st) {
   if (a.n <= 0) return;
-  cudaMemsetAsync(a.n_units, 0, sizeof(unsigned), st);
-  if (a.gix.keys) cudaMemsetAsync(a.n_gnew, 0, sizeof(unsigned), st);
-  if (a.grp && a.skip) k4_dedup<<<(a.n + 7) / 8, 256, 0, st>>>(a);
-  k4_units<<<(a.n + 255) / 256, 256, 0, st>>>(a);
-  k4_insert<<<num_sms * 3, kInsThreads, 0, st>>>(a);  // resident CTAs: 3 per SM
+  if (a.grp && a.skip) {
+    // launched without overlap: the route's keys are complete (they are read through the
+    // read-only path)
+    k4_dedup<<<(a.n + 7) / 8, 256, 0, st>>>(a);
+  } else {
+    cudaMemsetAsync(a.n_units, 0, sizeof(unsigned), st);
+    if (a.gix.keys) cudaMemsetAsync(a.n_gnew, 0, sizeof(unsigned), st);
+  }
+  launch_chained(k4_units, (a.n + 255) / 256, 256, 0, st, a);
+  launch_chained(k4_insert, num_sms * 3, kInsThreads, 0, st, a);  // resident CTAs: 3 per SM
 }
 
 void launch_insert_gix(const InsertArgs& a, int ctas, cudaStream_t st) {
   if (a.n <= 0 || !a.gix.keys) return;
-  k4_gix_insert<<<ctas, 256, 0, st>>>(a);
+  launch_chained(k4_gix_insert, ctas, 256, 0, st, a);
 }
 
 void launch_insert(const InsertArgs& a, int num_sms, cudaStream_t st) {
@@ -357,52 +409,10 @@ void launch_insert_entries(const EntryInsertArgs& a, cudaStream_t st) {
   k4_insert_entries<<<(int)(blocks < 4096 ? blocks : 4096), 256, 0, st>>>(a);
 }
 
-// ---------------------------------------------------------------------------
-// Session table update at commit (Sec. 4.1: an admitted new session becomes pending /
-// protected on its instance; a rebound one leaves its previous instance's count).
-// Only leaders with ADMIT_NEW change anything; each session has one leader per batch.
-__global__ void __launch_bounds__(256) k4_sessions(SessUpdateArgs a) {
-  if (block_error(a.err)) return;
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= a.n || a.rq.leader[r] != r || a.rq.reason[r] != MISAT_ADMIT_NEW) return;
-  const uint64_t s = a.rq.session[r];
-  const int w = a.rq.inst[r];
-  const int b = a.rq.cls[r];
-  const uint64_t nv = sess_val(kSessProtected, (uint32_t)b, (uint32_t)w);
-  const uint32_t mask = (1u << a.st.log2n) - 1;
-  uint32_t h = sess_home(s, a.st.log2n);
-  for (uint32_t it = 0; it <= mask; ++it) {
-    SessSlot* sl = a.st.slots + h;
-    unsigned long long k = __ldcg(&sl->key);
-    if (k == 0) {
-      k = atomicCAS(&sl->key, 0ull, (unsigned long long)s);
-      if (k == 0) {
-        sl->val = nv;
-        atomicAdd(a.st.used, 1ull);
-        atomicAdd(&a.prot[w * 3 + b], 1);
-        return;
-      }
-    }
-    if (k == s) {
-      const uint64_t ov = sl->val;
-      if (sess_state(ov) == kSessProtected) atomicSub(&a.prot[sess_inst(ov) * 3 + sess_cls(ov)], 1);
-      sl->val = nv;
-      atomicAdd(&a.prot[w * 3 + b], 1);
-      return;
-    }
-    h = (h + 1) & mask;
-  }
-  set_error(a.err, MISAT_ERR_TABLE_FULL);
-}
-
-void launch_session_update(const SessUpdateArgs& a, cudaStream_t st) {
-  if (a.n <= 0) return;
-  k4_sessions<<<(a.n + 255) / 256, 256, 0, st>>>(a);
-}
-
 // Completion events (distinct sessions): leave the protected set; done -> dead slot,
 // otherwise released (a later request must be admitted again, Eq. 7).
 __global__ void __launch_bounds__(256) k_complete(CompleteArgs a) {
+  chain_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= a.n) return;
   const uint64_t s = a.session[i];
@@ -426,7 +436,7 @@ __global__ void __launch_bounds__(256) k_complete(CompleteArgs a) {
 
 void launch_complete(const CompleteArgs& a, cudaStream_t st) {
   if (a.n <= 0) return;
-  k_complete<<<(a.n + 255) / 256, 256, 0, st>>>(a);
+  launch_chained(k_complete, (a.n + 255) / 256, 256, 0, st, a);
 }
 
 // External removal (Sec. 4.4 engine events): mark listed keys (meta = 0), rebuild the

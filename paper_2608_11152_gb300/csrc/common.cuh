@@ -30,6 +30,32 @@ inline int resident_grid(int block, size_t smem, int num_sms) {
   return per_sm * num_sms;
 }
 
+// Kernels of one stream whose launches overlap (programmatic dependent launch): a kernel lets the
+// next one's blocks be placed as soon as its own are, and touches no memory before every kernel
+// before it has finished and its writes are visible.  A pass of 64 requests is 20 kernels of 2 to 20
+// us each, one after the other, and the launch of each costs 1 to 2 us when it waits for
+// the end of the last.  Data that an earlier kernel of the chain writes is not read through the
+// read-only path (the compiler may move such loads up).
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Launches a kernel that begins with chain_wait() behind the stream's last operation.
+template <class... P, class... A>
+inline void launch_chained(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3(grid);
+  lc.blockDim = dim3(block);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = st;
+  lc.attrs = &at;
+  lc.numAttrs = 1;
+  cudaLaunchKernelEx(&lc, kernel, static_cast<P>(args)...);
+}
+
 constexpr int kBlockTokens = 16;
 constexpr uint64_t kGold = 0x9e3779b97f4a7c15ull;  // SplitMix64 increment, chain multiplier
 constexpr uint64_t kEmpty = 0;                     // empty slot key (block keys are >= 2)

@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(kSelThreads) k4_evict_estimate(EvictArgs a) {
   __shared__ long long s_tmp[32];
   __shared__ unsigned long long s_min, s_max;
   __shared__ unsigned s_m;
+  chain_wait();
   const int w = a.only_w ? *a.only_w : blockIdx.x;
   if (block_error(a.err)) return;
   const long long size = a.size[w];
@@ -294,6 +295,7 @@ __device__ __forceinline__ void collect_chunk(const EvictArgs& a, int w, uint32_
 // Work items (active instance, chunk), taken by a grid of resident CTAs: instances within
 // capacity cost nothing (their list entries are never made).
 __global__ void __launch_bounds__(256) k4_evict_collect(EvictArgs a, uint32_t chunks) {
+  chain_wait();
   if (block_error(a.err)) return;
   const uint32_t items = *(volatile const unsigned*)a.n_act * chunks;
   for (uint32_t it = blockIdx.x; it < items; it += gridDim.x) collect_chunk(a, a.act[it / chunks], it % chunks, chunks);
@@ -304,6 +306,7 @@ __global__ void __launch_bounds__(kSelThreads) k4_evict_select(EvictArgs a) {
   __shared__ long long s_tmp[32];
   __shared__ unsigned s_cnt;
   __shared__ unsigned long long s_or_hi, s_or_lo, s_v0_hi, s_v0_lo;
+  chain_wait();
   const int w = a.only_w ? *a.only_w : blockIdx.x;
   if (block_error(a.err)) return;
   if (a.active[w] != 1) return;
@@ -472,6 +475,7 @@ __device__ __forceinline__ void delete_slot(const GIndex& g, int w, Bucket* tab,
 __global__ void __launch_bounds__(256) k4_evict_delete(EvictArgs a) {
   __shared__ unsigned long long s_pre[kMaxW + 1];
   __shared__ unsigned s_del[kMaxW];
+  chain_wait();
   if (block_error(a.err)) return;
   const int nact = (int)*(volatile const unsigned*)a.n_act;
   for (int k = threadIdx.x; k < nact; k += blockDim.x) s_del[k] = 0;
@@ -509,6 +513,7 @@ __global__ void __launch_bounds__(256) k4_evict_delete(EvictArgs a) {
 // run's first deleted slot (lowest bucket, then lowest slot) owns the run.
 __global__ void __launch_bounds__(256) k4_evict_shift(EvictArgs a) {
   __shared__ unsigned long long s_pre[kMaxW + 1];
+  chain_wait();
   if (block_error(a.err)) return;
   const int nact = (int)*(volatile const unsigned*)a.n_act;
   const unsigned long long total = list_prefix(a, s_pre, nact);
@@ -624,27 +629,21 @@ int stream_grid(const EvictArgs& a, int chunks_per_inst, int resident) {
 void launch_evict_select(const EvictArgs& a, int chunks_per_inst, int num_sms, cudaStream_t st,
                          const cudaEvent_t* marks) {
   const int W = a.only_w ? 1 : a.W;
-  cudaMemsetAsync(a.n_act, 0, sizeof(unsigned), st);
-  k4_evict_estimate<<<W, kSelThreads, 0, st>>>(a);
+  launch_chained(k4_evict_estimate, W, kSelThreads, 0, st, a);
   if (marks) cudaEventRecord(marks[0], st);
-  k4_evict_collect<<<stream_grid(a, chunks_per_inst, resident_grid<k4_evict_collect>(256, 0, num_sms)), 256, 0, st>>>(
-      a, (uint32_t)chunks_per_inst);
+  launch_chained(k4_evict_collect, stream_grid(a, chunks_per_inst, resident_grid<k4_evict_collect>(256, 0, num_sms)), 256,
+                 0, st, a, (uint32_t)chunks_per_inst);
   if (marks) cudaEventRecord(marks[1], st);
-  k4_evict_select<<<W, kSelThreads, 0, st>>>(a);
+  launch_chained(k4_evict_select, W, kSelThreads, 0, st, a);
   if (marks) cudaEventRecord(marks[2], st);
 }
 
 void launch_evict_apply(const EvictArgs& a, int num_sms, cudaStream_t st, const cudaEvent_t* marks) {
   // one grid-stride pass over the list entries of every instance over capacity, one wave each
-  k4_evict_delete<<<resident_grid<k4_evict_delete>(256, 0, num_sms), 256, 0, st>>>(a);
+  launch_chained(k4_evict_delete, resident_grid<k4_evict_delete>(256, 0, num_sms), 256, 0, st, a);
   if (marks) cudaEventRecord(marks[0], st);
-  k4_evict_shift<<<resident_grid<k4_evict_shift>(256, 0, num_sms), 256, 0, st>>>(a);
+  launch_chained(k4_evict_shift, resident_grid<k4_evict_shift>(256, 0, num_sms), 256, 0, st, a);
   if (marks) cudaEventRecord(marks[1], st);
-}
-
-void launch_evict(const EvictArgs& a, int chunks_per_inst, int num_sms, cudaStream_t st) {
-  launch_evict_select(a, chunks_per_inst, num_sms, st, nullptr);
-  launch_evict_apply(a, num_sms, st, nullptr);
 }
 
 // Compaction of one instance table: delete entries with meta == 0 (marked) or

@@ -25,13 +25,14 @@ struct GIndex {
   unsigned long long* used;   // claimed slots
 };
 
-// Slot of `key`, or -1.  Only for phases without concurrent claims.  Adds buckets read.
+// Slot of `key`, or -1.  Only for phases without concurrent claims.  Adds buckets read.  (Through
+// L2: an earlier kernel of the same chain may have claimed the slots.)
 __device__ __forceinline__ int64_t gix_find(const GIndex& g, uint64_t key, uint32_t* reads) {
   const uint32_t mask = (1u << g.log2nb) - 1;
   uint32_t b = home_bucket(key, g.log2nb);
   for (uint32_t it = 0; it <= mask; ++it) {
     const ulonglong2* p = reinterpret_cast<const ulonglong2*>(g.keys + 4 * (size_t)b);
-    const ulonglong2 x = __ldg(p), y = __ldg(p + 1);
+    const ulonglong2 x = __ldcg(p), y = __ldcg(p + 1);
     *reads += 1;
     if (x.x == key) return 4 * (int64_t)b;
     if (x.y == key) return 4 * (int64_t)b + 1;

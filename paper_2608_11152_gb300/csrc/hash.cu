@@ -345,6 +345,7 @@ int32_t hash_long_blocks(int64_t n_tokens, int num_sms) {
 }
 
 __global__ void __launch_bounds__(32 * kHashWarps, kHashCtas) k1_block_hash(HashArgs a) {
+  chain_wait();
   if (*a.err) return;
   hash_batch(a);
 }
@@ -363,7 +364,7 @@ void launch_hash_lists(const HashArgs& a, cudaStream_t st) {
 void launch_block_hash(HashArgs a, int num_sms, cudaStream_t st) {
   const int res = resident_grid<k1_block_hash>(32 * kHashWarps, 0, num_sms);
   a.group = hash_group_size(a.n, res * kHashWarps);
-  k1_block_hash<<<a.n < res ? a.n : res, 32 * kHashWarps, 0, st>>>(a);
+  launch_chained(k1_block_hash, a.n < res ? a.n : res, 32 * kHashWarps, 0, st, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -396,6 +397,7 @@ namespace {
 // tiles took 18.8 us at 20,001 requests, a memory round trip and a block scan per tile.
 __global__ void __launch_bounds__(kHashTile) k1na_offsets(HashArgs a, unsigned long long* scratch) {
   __shared__ unsigned s_sum[kHashTile / 32];
+  chain_wait();
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   const int r = blockIdx.x * kHashTile + t;
   int64_t o0 = 0, o1 = 0;
@@ -426,6 +428,7 @@ __global__ void __launch_bounds__(kHashTile) k1na_offsets(HashArgs a, unsigned l
 // keys[s_tile[tile of r] + off[r] + j].
 __global__ void __launch_bounds__(32 * kHashWarps, kHashCtas) k1na_hash(HashArgs a, unsigned long long* scratch) {
   __shared__ uint32_t s_tile[65];  // blocks before each tile
+  chain_wait();
   if (scratch[0]) return;
   const int tiles = (a.n + kHashTile - 1) / kHashTile, t = threadIdx.x;
   if (t <= 64) {
@@ -502,7 +505,7 @@ extern "C" int misat_block_hash_noalloc(const int64_t* tok_off, const int32_t* t
   a.group = hash_group_size(n, res * kHashWarps);
   if (cudaMemsetAsync(scratch, 0, 8 * sizeof(*scratch), st) != cudaSuccess) return MISAT_ERR_CUDA;
   k1na_offsets<<<(n + kHashTile - 1) / kHashTile, kHashTile, 0, st>>>(a, scratch);
-  k1na_hash<<<n < res ? n : res, 32 * kHashWarps, 0, st>>>(a, scratch);
+  launch_chained(k1na_hash, n < res ? n : res, 32 * kHashWarps, 0, st, a, scratch);
   if (cudaGetLastError() != cudaSuccess) return MISAT_ERR_CUDA;
   unsigned long long err = 0;
   if (cudaMemcpyAsync(&err, scratch, sizeof(err), cudaMemcpyDeviceToHost, st) != cudaSuccess ||

@@ -150,12 +150,18 @@ struct CapsArgs {
   const int32_t* err;
 };
 void launch_caps(const CapsArgs& a, cudaStream_t st);  // caps and price orders
-// Writes the host's per-route class parameters (footprints, residencies, mixture) to the
-// device (kernel arguments are taken at launch, so the host array may change right after).
-struct RouteParams {
+// First kernel of a route: the host's class parameters (footprints, residencies, mixture; kernel
+// arguments are taken at launch, so the host's array may change right after) and cleared scratch.
+struct ClearArgs {
   int64_t v[9];
+  int64_t* params;            // [9]
+  unsigned long long* words[2];  // two runs of counters
+  int32_t n_words[2];
+  uint4* run[4];              // batch-sized tables, in 16-byte units
+  uint32_t n_run[4];
+  uint32_t fill[4];
 };
-void launch_route_params(const RouteParams& p, int64_t* dst, cudaStream_t st);
+void launch_clear(const ClearArgs& a, int num_sms, cudaStream_t st);
 
 // ---- serial selection (select.cu) ----
 // Grid of prompt lengths whose price orders are kept: exact below 16 tokens, then 16 steps per
@@ -181,6 +187,7 @@ struct SelectPrepArgs {
   int32_t W;
   ReqArrays rq;
   const uint16_t* H;           // [n*W], readable 16 bytes past its end
+  uint16_t* out_H;             // NULL, or the caller's copy of it
   const int64_t* backlog;      // [W] d_w
   const int64_t* tokcost;      // [W] 1/mu_w
   const int32_t* gh;           // [W] global headroom at batch start
@@ -190,7 +197,7 @@ struct SelectPrepArgs {
   int32_t* segcnt;             // [blocks] out: leaders per block
   const int32_t* err;
 };
-void launch_select_prep(const SelectPrepArgs& a, cudaStream_t st);
+void launch_select_prep(const SelectPrepArgs& a, int num_sms, cudaStream_t st);
 
 struct SelectArgs {
   int32_t n;
@@ -231,11 +238,17 @@ struct FinalizeArgs {
 void launch_finalize(const FinalizeArgs& a, cudaStream_t st);
 
 // ---- commit ----
+// Session table update of a commit (rq.leader == NULL: none, as for loaded chains).
+struct SessUpdateArgs {
+  ReqArrays rq;
+  SessTable st;
+  int32_t* prot;               // [W*3]
+};
 struct InsertArgs {
   const InstDesc* desc;
   int32_t n;
   int4* units;                 // work list: 32-byte unit records (2 int4), up to 128 blocks each
-  unsigned* n_units;           // units listed (zeroed by the launcher)
+  unsigned* n_units;           // units listed (zeroed first)
   int64_t units_cap;
   const int32_t* nb;
   const int64_t* kbase;
@@ -251,12 +264,14 @@ struct InsertArgs {
   int32_t* err;
   GIndex gix;                  // mirrored when gix.keys != NULL
   ulonglong2* gnew;            // keys new to an instance table, (key, instance), for the
-  unsigned* n_gnew;            //   global index pass (zeroed by the launcher)
+  unsigned* n_gnew;            //   global index pass (zeroed first)
   int64_t gnew_cap;
   const ulonglong2* grp;       // groups of the admitted requests (NULL: insert every block)
   uint32_t grp_log2;
   int32_t* skip;               // [n] leading blocks a later request of the group inserts
   unsigned long long* ops;     // blocks in the work list (NULL: not counted)
+  unsigned* n_act;             // commit: the eviction's list length, zeroed with the others
+  SessUpdateArgs sess;
 };
 void launch_insert(const InsertArgs& a, int num_sms, cudaStream_t st);  // tables, then global index
 void launch_insert_tables(const InsertArgs& a, int num_sms, cudaStream_t st);
@@ -272,15 +287,6 @@ struct EntryInsertArgs {
   GIndex gix;
 };
 void launch_insert_entries(const EntryInsertArgs& a, cudaStream_t st);
-
-struct SessUpdateArgs {
-  int32_t n;
-  ReqArrays rq;
-  SessTable st;
-  int32_t* prot;               // [W*3]
-  int32_t* err;
-};
-void launch_session_update(const SessUpdateArgs& a, cudaStream_t st);
 
 struct CompleteArgs {
   int32_t n;
@@ -313,10 +319,9 @@ struct EvictArgs {
   int32_t* err;
   GIndex gix;                  // deletions clear the instance's bit when gix.keys != NULL
   int32_t* act;                // [W] instances over capacity (listed by the estimate pass)
-  unsigned* n_act;             // entries in act (zeroed by the launcher)
+  unsigned* n_act;             // entries in act (zeroed by the caller)
 };
-void launch_evict(const EvictArgs& a, int chunks_per_inst, int num_sms, cudaStream_t st);
-// the two halves: select (estimate, collect, select; reads the tables only) and apply
+// the eviction's two halves: select (estimate, collect, select; reads the tables only) and apply
 // (delete, shift; also clears global-index bits)
 // marks (may be NULL): events recorded after each kernel (select: 3, apply: 2), for phase timing
 void launch_evict_select(const EvictArgs& a, int chunks_per_inst, int num_sms, cudaStream_t st,

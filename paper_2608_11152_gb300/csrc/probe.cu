@@ -59,6 +59,7 @@ __device__ __forceinline__ void block_add_stats(unsigned long long* stats, unsig
 // (c) k2_probe_first_gix on the batch-local index writes every request's H row, hbest and
 //     hit-list entries from its key's mask, as with the global index.
 __global__ void __launch_bounds__(256) k2_first_claim(ProbeArgs a) {
+  chain_wait();
   if (block_error(a.err)) return;
   const int lane = threadIdx.x & 31;
   const int stride = gridDim.x * blockDim.x;
@@ -89,6 +90,7 @@ constexpr int kDistIlp = 4;  // tables per lane with their home sectors in fligh
 __global__ void __launch_bounds__(256) k2_probe_distinct(ProbeArgs a) {
   __shared__ Bucket* s_tab[kMaxW];
   __shared__ uint32_t s_lg[kMaxW];
+  chain_wait();
   if (block_error(a.err)) return;
   for (int w = threadIdx.x; w < a.W; w += blockDim.x) {
     s_tab[w] = a.desc[w].tab;
@@ -158,6 +160,7 @@ __global__ void __launch_bounds__(256) k2_probe_distinct(ProbeArgs a) {
 constexpr int kSG = 16;
 
 __global__ void __launch_bounds__(256) k2_probe_search(ProbeArgs a) {
+  chain_wait();
   if (block_error(a.err)) return;
   const unsigned nh = *a.n_hits;
   const unsigned lim = (int64_t)nh < a.hits_cap ? nh : (unsigned)a.hits_cap;
@@ -215,6 +218,7 @@ __global__ void __launch_bounds__(256) k2_probe_search(ProbeArgs a) {
 // pair, at its request's base (one atomic per warp) plus the rank of the bit in the mask.
 __global__ void __launch_bounds__(256) k2_probe_first_gix(ProbeArgs a) {
   extern __shared__ unsigned long long s_gm[];  // [warps][32][mw] masks, then [warps][32] (nb, base)
+  chain_wait();
   if (block_error(a.err)) return;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int wpb = blockDim.x >> 5;
@@ -239,7 +243,7 @@ __global__ void __launch_bounds__(256) k2_probe_first_gix(ProbeArgs a) {
     }
     int bits = 0, wmin = INT32_MAX;
     for (uint32_t i = 0; i < mw; ++i) {
-      const unsigned long long m = slot >= 0 ? __ldg(a.gix.masks + (size_t)slot * mw + i) : 0ull;
+      const unsigned long long m = slot >= 0 ? __ldcg(a.gix.masks + (size_t)slot * mw + i) : 0ull;
       sm[lane * mw + i] = m;
       bits += __popcll(m);
       if (m && wmin == INT32_MAX) wmin = 64 * (int)i + __ffsll((long long)m) - 1;
@@ -353,21 +357,21 @@ void launch_probe_first(const ProbeArgs& a, int num_sms, cudaStream_t st) {
   const int gres = resident_grid<k2_probe_first_gix>(256, gsmem, num_sms);
   const int ggrid = gblocks < gres ? gblocks : gres;
   if (a.gix.keys) {
-    k2_probe_first_gix<<<ggrid, 256, 8 * 32 * (a.gix.mw * sizeof(unsigned long long) + sizeof(int2)), st>>>(a);
+    launch_chained(k2_probe_first_gix, ggrid, 256, gsmem, st, a);
     return;
   }
   // per-instance tables: the context allocates the batch-local index with the tables
-  k2_first_claim<<<ggrid, 256, 0, st>>>(a);
-  k2_probe_distinct<<<num_sms * 8, 256, 0, st>>>(a);  // two waves: measured faster than one for this pass
+  launch_chained(k2_first_claim, ggrid, 256, 0, st, a);
+  launch_chained(k2_probe_distinct, num_sms * 8, 256, 0, st, a);  // two waves: measured faster than one for this pass
   ProbeArgs e = a;
   e.gix = a.fb;
   e.stats = a.stats_fb;
-  k2_probe_first_gix<<<ggrid, 256, 8 * 32 * (a.fb.mw * sizeof(unsigned long long) + sizeof(int2)), st>>>(e);
+  launch_chained(k2_probe_first_gix, ggrid, 256, gsmem, st, e);
 }
 
 void launch_probe_search(const ProbeArgs& a, int num_sms, cudaStream_t st) {
   if ((int64_t)a.n * a.W <= 0) return;
-  k2_probe_search<<<resident_grid<k2_probe_search>(256, 0, num_sms), 256, 0, st>>>(a);
+  launch_chained(k2_probe_search, resident_grid<k2_probe_search>(256, 0, num_sms), 256, 0, st, a);
 }
 
 }  // namespace misat

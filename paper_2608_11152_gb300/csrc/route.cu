@@ -10,6 +10,7 @@ namespace misat {
 // device session table (state at batch start, Sec. 4.1: O_w u P_w merged) and
 // insert them into a batch-local map that keeps each session's first arrival.
 __global__ void __launch_bounds__(256) k0_prologue(PrologueArgs a) {
+  chain_wait();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   bool ok = r < a.n;
   uint8_t c = 0;
@@ -77,6 +78,7 @@ __global__ void __launch_bounds__(256) k0_prologue(PrologueArgs a) {
 // batch that are protected nowhere (Sec. 4.2: held and candidate sessions each count).
 __global__ void __launch_bounds__(256) k0_leaders(PrologueArgs a) {
   __shared__ unsigned long long s_cand[3];
+  chain_wait();
   if (block_error(a.err)) return;
   if (threadIdx.x < 3) s_cand[threadIdx.x] = 0;
   __syncthreads();
@@ -116,8 +118,8 @@ __global__ void __launch_bounds__(256) k0_leaders(PrologueArgs a) {
 void launch_prologue(const PrologueArgs& a, cudaStream_t st) {
   if (a.n <= 0) return;
   const int grid = (a.n + 255) / 256;
-  k0_prologue<<<grid, 256, 0, st>>>(a);
-  k0_leaders<<<grid, 256, 0, st>>>(a);
+  launch_chained(k0_prologue, grid, 256, 0, st, a);
+  launch_chained(k0_leaders, grid, 256, 0, st, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -216,6 +218,7 @@ int price_order_blocks(int W) {
 // K3a caps, one thread per instance (Sec. 4.1; Eqs. 9-10 MISA; Eqs. 11, 13 MISA-T) in the first
 // CTA; the other CTAs sort the selection's price orders.
 __global__ void __launch_bounds__(1024) k3_caps(CapsArgs a) {
+  chain_wait();
   if (block_error(a.err)) return;
   if (blockIdx.x > 0) {
     sort_price_orders(a.backlog, a.tokcost, a.W, blockIdx.x - 1, a.orders);
@@ -288,14 +291,31 @@ __global__ void __launch_bounds__(1024) k3_caps(CapsArgs a) {
 }
 
 void launch_caps(const CapsArgs& a, cudaStream_t st) {
-  k3_caps<<<1 + price_order_blocks(a.W), 1024, 0, st>>>(a);
+  launch_chained(k3_caps, 1 + price_order_blocks(a.W), 1024, 0, st, a);
 }
 
-__global__ void k_route_params(RouteParams p, int64_t* dst) {
-  if (threadIdx.x < 9) dst[threadIdx.x] = p.v[threadIdx.x];
+// Clears a route's scratch (one kernel where eight memsets took 1.5 us each).  Launched without
+// overlap: everything enqueued before, the caller's inputs among it, is complete before it begins.
+__global__ void __launch_bounds__(256) k0_clear(ClearArgs a) {
+  chain_wait();
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+  if (t < 9) a.params[t] = a.v[t];
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+    for (uint32_t i = t; i < (uint32_t)a.n_words[k]; i += stride) a.words[k][i] = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const uint4 v = make_uint4(a.fill[k], a.fill[k], a.fill[k], a.fill[k]);
+    for (uint32_t i = t; i < a.n_run[k]; i += stride) a.run[k][i] = v;
+  }
 }
 
-void launch_route_params(const RouteParams& p, int64_t* dst, cudaStream_t st) { k_route_params<<<1, 32, 0, st>>>(p, dst); }
+void launch_clear(const ClearArgs& a, int num_sms, cudaStream_t st) {
+  uint32_t most = (uint32_t)a.n_words[0];
+  for (uint32_t n : a.n_run) most = n > most ? n : most;
+  const int blocks = (int)((most + 255) / 256);
+  k0_clear<<<blocks < 1 ? 1 : (blocks < 4 * num_sms ? blocks : 4 * num_sms), 256, 0, st>>>(a);
+}
 
 // ---------------------------------------------------------------------------
 // Finalise: held leaders keep the reason the selection gave them, followers copy their
@@ -304,6 +324,7 @@ void launch_route_params(const RouteParams& p, int64_t* dst, cudaStream_t st) { 
 // [8..10] admitted by class, [11..13] held by class, [14] hit tokens, [15] query tokens.
 __global__ void __launch_bounds__(256) k4_finalize(FinalizeArgs a) {
   __shared__ unsigned long long s_st[16];
+  chain_wait();
   if (block_error(a.err)) return;
   if (threadIdx.x < 16) s_st[threadIdx.x] = 0;
   __syncthreads();
@@ -365,7 +386,7 @@ __global__ void __launch_bounds__(256) k4_finalize(FinalizeArgs a) {
 
 void launch_finalize(const FinalizeArgs& a, cudaStream_t st) {
   if (a.n <= 0) return;
-  k4_finalize<<<(a.n + 255) / 256, 256, 0, st>>>(a);
+  launch_chained(k4_finalize, (a.n + 255) / 256, 256, 0, st, a);
 }
 
 }  // namespace misat

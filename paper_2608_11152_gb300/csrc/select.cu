@@ -55,7 +55,23 @@ constexpr int kFixed = -3;           // the same, decided for good
 // a cached prefix (one entry at a time took 0.13 ms at 3,001 requests of 1,000 instances).
 __global__ void __launch_bounds__(256) k3_select_prep(SelectPrepArgs a) {
   __shared__ int s_wc[8];
+  chain_wait();
   if (block_error(a.err)) return;
+  const int leaders = (a.n + 255) / 256;
+  if ((int)blockIdx.x >= leaders) {  // the caller's copy of H, beside the records
+    const int64_t total = (int64_t)a.n * a.W, t = (int64_t)(blockIdx.x - leaders) * blockDim.x + threadIdx.x,
+                  stride = (int64_t)(gridDim.x - leaders) * blockDim.x;
+    int64_t done = 0;
+    if ((reinterpret_cast<uintptr_t>(a.out_H) & 15) == 0) {
+      const uint4* src = reinterpret_cast<const uint4*>(a.H);
+      uint4* dst = reinterpret_cast<uint4*>(a.out_H);
+#pragma unroll 4
+      for (int64_t i = t; i < total >> 3; i += stride) dst[i] = __ldcg(src + i);
+      done = total & ~(int64_t)7;
+    }
+    for (int64_t i = done + t; i < total; i += stride) a.out_H[i] = __ldcg(a.H + i);
+    return;
+  }
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const bool lead = r < a.n && a.rq.status[r] == kStUnresolved;
@@ -94,7 +110,7 @@ __global__ void __launch_bounds__(256) k3_select_prep(SelectPrepArgs a) {
     const uint4* p = reinterpret_cast<const uint4*>(row - lead_in);
     const int pieces = (lead_in + a.W + 7) >> 3;
     for (int q = 0; q < pieces; ++q) {
-      const uint4 v = __ldg(p + q);
+      const uint4 v = __ldcg(p + q);
       if ((v.x | v.y | v.z | v.w) == 0) continue;
       const uint32_t u[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -131,9 +147,14 @@ __global__ void __launch_bounds__(256) k3_select_prep(SelectPrepArgs a) {
   }
 }
 
-void launch_select_prep(const SelectPrepArgs& a, cudaStream_t st) {
+void launch_select_prep(const SelectPrepArgs& a, int num_sms, cudaStream_t st) {
   if (a.n <= 0) return;
-  k3_select_prep<<<(a.n + 255) / 256, 256, 0, st>>>(a);
+  int grid = (a.n + 255) / 256;
+  if (a.out_H) {
+    const int64_t copy = ((int64_t)a.n * a.W + 8191) / 8192;
+    grid += (int)(copy < 8 * num_sms ? copy : 8 * num_sms);
+  }
+  launch_chained(k3_select_prep, grid, 256, 0, st, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -321,7 +342,7 @@ __device__ __forceinline__ int sel_choose(const SelSmem& s, const SelectArgs& a,
       const uint4* p = reinterpret_cast<const uint4*>(row - lead_in);
       const int pieces = (lead_in + W + 7) >> 3;
       for (int q = 0; q < pieces; ++q) {
-        const uint4 v = __ldg(p + q);
+        const uint4 v = __ldcg(p + q);
         if ((v.x | v.y | v.z | v.w) == 0) continue;
         for (int e = 0; e < 8; ++e) {
           const uint32_t u = e < 2 ? v.x : (e < 4 ? v.y : (e < 6 ? v.z : v.w));
@@ -429,6 +450,7 @@ __global__ void __launch_bounds__(1024, 1) k4_select(SelectArgs a, int cs) {
   __shared__ int s_fixmin;
   __shared__ int s_tgmax;
   __shared__ unsigned long long s_tcmin;
+  chain_wait();
   if (block_error(a.err)) return;
   const int W = a.W;
   const int T = blockDim.x, NW = T >> 5;
@@ -471,7 +493,7 @@ __global__ void __launch_bounds__(1024, 1) k4_select(SelectArgs a, int cs) {
     const uint4* src = reinterpret_cast<const uint4*>(a.orders);
     const int pieces = kPriceCells * (price_order_stride(W) >> 3);
 #pragma unroll 4
-    for (int i = tid; i < pieces; i += T) s.ord[i] = __ldg(src + i);
+    for (int i = tid; i < pieces; i += T) s.ord[i] = __ldcg(src + i);
   }
   // leaders before each block of 256 requests (exclusive scan of the prep kernel's counts)
   {
@@ -863,17 +885,19 @@ void launch_select(const SelectArgs& a, int max_cluster, cudaStream_t st) {
   if (a.n <= 0) return;
   int cs, threads;
   select_shape(a.n, max_cluster, &cs, &threads);
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = cs;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchAttribute at[2] = {};
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3(cs);
   lc.blockDim = dim3(threads);
   lc.dynamicSmemBytes = sel_smem_layout(a.W, cs, threads / 32, (a.n + 255) / 256, nullptr, nullptr);
   lc.stream = st;
-  lc.attrs = &at;
-  lc.numAttrs = 1;
+  lc.attrs = at;
+  lc.numAttrs = 2;
   cudaLaunchKernelEx(&lc, k4_select, a, cs);
 }
 
