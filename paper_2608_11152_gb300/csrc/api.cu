@@ -97,6 +97,8 @@ struct misat_ctx {
   uint32_t** d_dslots = nullptr;
   unsigned* d_ncand = nullptr;
   unsigned* d_nd = nullptr;
+  unsigned* d_nholes = nullptr;
+  int2* d_scale = nullptr;
   unsigned long long* d_thr = nullptr;  // [2W] bracket lo | hi
   // per-instance inputs and state
   int64_t* d_backlog = nullptr;
@@ -556,6 +558,8 @@ EvictArgs evict_args(misat_ctx* c, unsigned long long* evicted_counter) {
   ev.dmask = c->d_dmask;
   ev.n_cand = c->d_ncand;
   ev.n_d = c->d_nd;
+  ev.n_holes = c->d_nholes;
+  ev.scale = c->d_scale;
   ev.thr_lo = c->d_thr;
   ev.thr_hi = c->d_thr + c->W;
   ev.theta = c->d_theta;
@@ -914,7 +918,7 @@ int misat_create(const misat_config* cfg, void* cuda_stream, misat_ctx** out) {
       (rc = dalloc_n(c, &c->d_desc, Ws)) || (rc = dalloc_n(c, &c->d_bitmap, Ws)) || (rc = dalloc_n(c, &c->d_ca, Ws)) ||
       (rc = dalloc_n(c, &c->d_cb, Ws)) || (rc = dalloc_n(c, &c->d_cc, Ws)) || (rc = dalloc_n(c, &c->d_slots, Ws)) ||
       (rc = dalloc_n(c, &c->d_dmask, Ws)) || (rc = dalloc_n(c, &c->d_ncand, Ws)) ||
-      (rc = dalloc_n(c, &c->d_dslots, Ws)) || (rc = dalloc_n(c, &c->d_nd, Ws)) ||
+      (rc = dalloc_n(c, &c->d_dslots, Ws)) || (rc = dalloc_n(c, &c->d_nd, Ws)) || (rc = dalloc_n(c, &c->d_nholes, Ws)) || (rc = dalloc_n(c, &c->d_scale, Ws)) ||
       (rc = dalloc_n(c, &c->d_thr, 2 * Ws)) ||
       (rc = dalloc_n(c, &c->d_stage_tok, (size_t)c->max_tokens + 8)) ||
       (rc = dalloc_n(c, &c->d_stage_off, NB + 1)) || (rc = dalloc_n(c, &c->d_stage_cls, NB)) ||

@@ -6,15 +6,17 @@
 // Admissions concentrate on few instances (every cold request of a round prefers the
 // same cheapest instance), so E ranges from 0 to a large part of an instance; the work
 // is spread over many CTAs per instance and the one serial step is kept small:
-//   k4_evict_estimate  (1 CTA / instance)  sorted sample of up to 4096 metas -> a meta
-//                      bracket [lo, hi] that contains the E-th smallest w.h.p.
+//   k4_evict_estimate  (1 CTA / instance)  histogram of the metas of up to 2048 buckets -> a meta
+//                      bracket [lo, hi] that contains the E-th smallest w.h.p. (for sure where
+//                      that is the whole table)
 //   k4_evict_collect   (many CTAs / instance, streaming)  fullness bitmap; entries with
 //                      meta < lo are certainly evicted (slot list D), entries with
 //                      lo <= meta <= hi go to a short list U with their values and slots
-//   k4_evict_select    (1 CTA / instance)  theta = the (E - |D|)-th smallest of U by
-//                      radix narrowing; if the bracket missed, the CTA re-collects the
-//                      whole instance and selects exactly anyway
-//   k4_evict_delete    deletes D and the entries of U at or below theta
+//   k4_evict_select    (1 CTA / instance)  theta = the (E - |D|)-th smallest of U: the bin of
+//                      a histogram that holds it, then by counting ranks; if the bracket
+//                      missed, the CTA re-collects the whole instance and selects exactly anyway
+//   k4_evict_delete    deletes D and the entries of U at or below theta; those that leave a hole
+//                      in a full bucket are listed
 //   k4_evict_shift     refills the holes of every run of full buckets that lost an entry
 //                      with backward shifts (no tombstones), one thread per run
 #include "common.cuh"
@@ -24,8 +26,11 @@ namespace misat {
 
 namespace {
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kSelThreads = 1024;
+constexpr int kEstThreads = 512;
 constexpr int kBins = 4096;
+constexpr int kEstBuckets = 2048;  // sampled per instance, four by each thread
+constexpr int kSelSmem = 1024;      // candidates kept in shared memory
+constexpr int kRankMax = 64;        // candidates that are ranked by counting
 
 __device__ __forceinline__ bool le128(uint64_t ma, uint64_t ka, uint64_t mb, uint64_t kb) {
   return ma < mb || (ma == mb && ka <= kb);
@@ -34,43 +39,42 @@ __device__ __forceinline__ bool le128(uint64_t ma, uint64_t ka, uint64_t mb, uin
 __device__ __forceinline__ uint64_t v_hi(const uint4& v) { return ((unsigned long long)v.y << 32) | v.x; }
 __device__ __forceinline__ uint64_t v_lo(const uint4& v) { return ((unsigned long long)v.w << 32) | v.z; }
 
-// Block-wide (1024 threads, 4096 bins): bin t with cum(<t) < E <= cum(<=t); cum(<t) in *below.
-__device__ int find_threshold_bin(uint32_t* hist, long long E, long long* below, long long* s_tmp) {
-  const int t = threadIdx.x;
-  long long local = (long long)hist[4 * t] + hist[4 * t + 1] + hist[4 * t + 2] + hist[4 * t + 3];
-  const int lane = t & 31, wid = t >> 5;
-  long long incl = local;
+// Block-wide (T threads): bin t with cum(<t) < E <= cum(<=t), 1 <= E <= all; cum(<t) in
+// *below.
+template <int T>
+__device__ int find_threshold_bin(const uint32_t* hist, uint32_t E, uint32_t* below) {
+  constexpr int kPer = kBins / T;
+  __shared__ uint32_t s_tmp[32];
+  __shared__ int s_bin;
+  __shared__ uint32_t s_below;
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  uint32_t h[kPer], local = 0;
+#pragma unroll
+  for (int i = 0; i < kPer; i += 4) {
+    const uint4 v = reinterpret_cast<const uint4*>(hist + kPer * t)[i / 4];
+    h[i] = v.x;
+    h[i + 1] = v.y;
+    h[i + 2] = v.z;
+    h[i + 3] = v.w;
+    local += v.x + v.y + v.z + v.w;
+  }
+  uint32_t incl = local;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const long long v = __shfl_up_sync(kFull, incl, o);
+    const uint32_t v = __shfl_up_sync(kFull, incl, o);
     if (lane >= o) incl += v;
   }
   if (lane == 31) s_tmp[wid] = incl;
-  __syncthreads();
-  if (wid == 0) {
-    long long v = s_tmp[lane];
-    long long sc = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const long long u = __shfl_up_sync(kFull, sc, o);
-      if (lane >= o) sc += u;
-    }
-    s_tmp[lane] = sc - v;
-  }
-  __syncthreads();
-  const long long excl = s_tmp[wid] + incl - local;
-  __shared__ int s_bin;
-  __shared__ long long s_below;
   if (t == 0) s_bin = -1;
   __syncthreads();
-  long long c = excl;
-  for (int i = 0; i < 4; ++i) {
-    const long long h = hist[4 * t + i];
-    if (c < E && E <= c + h) {
-      s_bin = 4 * t + i;
+  uint32_t c = incl - local + __reduce_add_sync(kFull, lane < wid ? s_tmp[lane] : 0u);
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    if (c < E && E <= c + h[i]) {
+      s_bin = kPer * t + i;
       s_below = c;
     }
-    c += h;
+    c += h[i];
   }
   __syncthreads();
   *below = s_below;
@@ -90,102 +94,130 @@ __device__ __forceinline__ uint32_t digit128(uint64_t hi, uint64_t lo, int shift
 }  // namespace
 
 
-__global__ void __launch_bounds__(kSelThreads) k4_evict_estimate(EvictArgs a) {
-  constexpr int kEst = 2048;  // 4 slots of up to 512 evenly spaced buckets
-  __shared__ unsigned long long s_smp[kEst];
-  __shared__ uint32_t hist[kBins];
-  __shared__ long long s_tmp[32];
-  __shared__ unsigned long long s_min, s_max;
-  __shared__ unsigned s_m;
+// Metas without the bits that no sample uses (a commit's ticks fill a small part of the span between
+// two sequence numbers): in this order the samples spread over the histogram's bins, while equal bins
+// of the metas themselves held a whole commit each.
+struct TickScale {
+  int ab, db;      // bits of the samples' largest arrival and depth
+  __device__ unsigned long long pack(unsigned long long m) const {
+    const unsigned long long low = (m & 0xffffu), base = 65536ull - (1ull << db);
+    const unsigned long long arr = (m >> 16) & 0xfffffu, top = (1ull << ab) - 1;
+    return ((((m >> 36) << ab) | (arr < top ? arr : top)) << db) | (low > base ? low - base : 0ull);
+  }
+  // the smallest meta that packs to x or more
+  __device__ unsigned long long unpack(unsigned long long x) const {
+    const unsigned long long low = x & ((1ull << db) - 1), arr = (x >> db) & ((1ull << ab) - 1), seq = x >> (db + ab);
+    if (seq >> 28) return ~0ull;
+    return (seq << 36) | (arr << 16) | (low ? low + 65536ull - (1ull << db) : 0ull);
+  }
+};
+
+// Bound by latency: one round of loads and a few block barriers.  The samples stay in registers,
+// and a bin is a shift (with 128-bit quotients of equal bins it took 16 us, on tables of any
+// size); 2,048 buckets instead of 512 make the bracket, and U with it, half as wide.
+__global__ void __launch_bounds__(kEstThreads) k4_evict_estimate(EvictArgs a) {
+  constexpr int kPer = kEstBuckets / kEstThreads;
+  __shared__ __align__(16) uint32_t hist[kBins];
+  struct Part {
+    unsigned long long mn, mx;
+    unsigned occ, arr, dep;
+  };
+  __shared__ Part s_part[kEstThreads / 32];
   chain_wait();
   const int w = a.only_w ? *a.only_w : blockIdx.x;
   if (block_error(a.err)) return;
   const long long size = a.size[w];
-  const long long E = size - a.desc[w].cap;
+  const InstDesc d = a.desc[w];
+  const long long E = size - d.cap;
   const int tid = threadIdx.x;
   if (tid == 0) {
     a.active[w] = E > 0 ? 1 : 0;
     a.n_d[w] = 0;
     a.n_cand[w] = 0;
+    a.n_holes[w] = 0;
     if (E > 0) a.act[atomicAdd(a.n_act, 1u)] = w;  // the streaming passes visit only these
   }
   if (E <= 0) return;
-  const InstDesc d = a.desc[w];
   const uint32_t NB = 1u << d.log2nb;
-  if (tid == 0) {
-    s_m = 0;
-    s_min = ~0ull;
-    s_max = 0;
+  const uint32_t nsb = NB < (uint32_t)kEstBuckets ? NB : (uint32_t)kEstBuckets;  // powers of two
+  unsigned long long m[4 * kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const uint32_t i = tid + k * kEstThreads;
+    ulonglong2 m01 = make_ulonglong2(0, 0), m23 = m01;
+    if (i < nsb) {
+      const ulonglong2* mp = reinterpret_cast<const ulonglong2*>(d.tab[i * (NB / nsb)].meta);
+      m01 = __ldcg(mp);
+      m23 = __ldcg(mp + 1);
+    }
+    m[4 * k] = m01.x;
+    m[4 * k + 1] = m01.y;
+    m[4 * k + 2] = m23.x;
+    m[4 * k + 3] = m23.y;
   }
-  for (int i = tid; i < kBins; i += kSelThreads) hist[i] = 0;
-  __syncthreads();
-  // samples: the metas of up to 512 evenly spaced buckets
+  for (int i = tid; i < kBins; i += kEstThreads) hist[i] = 0;
   unsigned long long mn = ~0ull, mx = 0;
-  {
-    const uint32_t nsb = NB < 512u ? NB : 512u;
-    unsigned occ = 0;
-    if ((uint32_t)tid < nsb) {
-      const uint32_t b = (uint32_t)(((uint64_t)tid * NB) / nsb);
-      const ulonglong2* mp = reinterpret_cast<const ulonglong2*>(d.tab[b].meta);
-      const ulonglong2 m01 = __ldcg(mp), m23 = __ldcg(mp + 1);
-      const unsigned long long m[4] = {m01.x, m01.y, m23.x, m23.y};
-      for (int s = 0; s < 4; ++s) {
-        s_smp[4 * tid + s] = m[s];
-        if (m[s]) {
-          ++occ;
-          mn = m[s] < mn ? m[s] : mn;
-          mx = m[s] > mx ? m[s] : mx;
-        }
-      }
-    } else if (tid < kEst / 4) {
-      for (int s = 0; s < 4; ++s) s_smp[4 * tid + s] = 0;
+  unsigned occ = 0, arr = 0, dep = 0;
+#pragma unroll
+  for (int k = 0; k < 4 * kPer; ++k)
+    if (m[k]) {
+      ++occ;
+      mn = m[k] < mn ? m[k] : mn;
+      mx = m[k] > mx ? m[k] : mx;
+      arr = max(arr, (unsigned)(m[k] >> 16) & 0xfffffu);
+      dep = max(dep, 0xffffu - ((unsigned)m[k] & 0xffffu));
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long a1 = __shfl_xor_sync(kFull, mn, o), a2 = __shfl_xor_sync(kFull, mx, o);
-      mn = a1 < mn ? a1 : mn;
-      mx = a2 > mx ? a2 : mx;
-      occ += __shfl_xor_sync(kFull, occ, o);
-    }
-    if ((tid & 31) == 0 && occ) {
-      atomicAdd(&s_m, occ);
-      atomicMin(&s_min, mn);
-      atomicMax(&s_max, mx);
-    }
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long a1 = __shfl_xor_sync(kFull, mn, o), a2 = __shfl_xor_sync(kFull, mx, o);
+    mn = a1 < mn ? a1 : mn;
+    mx = a2 > mx ? a2 : mx;
   }
+  occ = __reduce_add_sync(kFull, occ);
+  arr = __reduce_max_sync(kFull, arr);
+  dep = __reduce_max_sync(kFull, dep);
+  if ((tid & 31) == 0) s_part[tid >> 5] = Part{mn, mx, occ, arr, dep};
   __syncthreads();
-  const unsigned m = s_m;
+  Part all = s_part[0];
+#pragma unroll
+  for (int k = 1; k < kEstThreads / 32; ++k) {
+    const Part p = s_part[k];
+    all.mn = p.mn < all.mn ? p.mn : all.mn;
+    all.mx = p.mx > all.mx ? p.mx : all.mx;
+    all.occ += p.occ;
+    all.arr = max(all.arr, p.arr);
+    all.dep = max(all.dep, p.dep);
+  }
+  const unsigned n = all.occ;
+  const TickScale ts{32 - __clz(all.arr), 32 - __clz(all.dep)};
   unsigned long long lo = 0, hi = ~0ull;
-  if (m > 0 && size > 0) {
-    // histogram of the samples over [min, max], 4096 equal bins
-    const unsigned long long smin = s_min;
-    const unsigned __int128 range = (unsigned __int128)(s_max - s_min) + 1;
-    auto bin_of = [&](unsigned long long x) {
-      return (uint32_t)((((unsigned __int128)(x - smin)) << 12) / range);
-    };
-    for (int i = tid; i < kEst; i += kSelThreads) {
-      const unsigned long long x = s_smp[i];
-      if (x) atomicAdd(&hist[bin_of(x)], 1u);
-    }
+  if (n > 0) {
+    // histogram of the samples from their minimum on, bins of 2^shift
+    const unsigned long long smin = ts.pack(all.mn);
+    const int shift = max(0, 52 - __clzll((long long)(ts.pack(all.mx) - smin)));
+#pragma unroll
+    for (int k = 0; k < 4 * kPer; ++k)
+      if (m[k]) atomicAdd(&hist[(uint32_t)((ts.pack(m[k]) - smin) >> shift)], 1u);
     __syncthreads();
-    // the E-th smallest sits near sample rank p = E m / size; bracket it by ~3 standard
-    // deviations of the sample count plus a constant on both sides
-    const double p = (double)E * (double)m / (double)size;
-    const double margin = 3.0 * sqrt(p + 1.0) + 16.0;
-    const long long rl = (long long)(p - margin), rh = (long long)(p + margin) + 1;
-    long long below;
-    const int bl = rl >= 1 ? find_threshold_bin(hist, rl, &below, s_tmp) : -1;
-    const int bh = rh <= (long long)m ? find_threshold_bin(hist, rh, &below, s_tmp) : -1;
-    // bin edges: every sample of bin b lies in [edge(b), edge(b + 1) - 1]
-    auto edge = [&](int b) {
-      return smin + (unsigned long long)((range * (unsigned)b + 4095) >> 12);
-    };
-    if (bl >= 0) lo = edge(bl);
-    if (bh >= 0) hi = edge(bh + 1) - 1;
+    // the E-th smallest sits near sample rank p = E n / size (exactly there in a whole table);
+    // bracket it by ~3 standard deviations of the sample count plus a constant on both sides
+    // (in 32 bits: 64-bit floating point is slow here, and a miss costs time only)
+    const float p = (float)E * ((float)n / (float)size);
+    const float margin = 3.0f * sqrtf(p + 1.0f) + 16.0f;
+    const long long rl = nsb == NB ? E : (long long)(p - margin), rh = nsb == NB ? E : (long long)(p + margin) + 1;
+    uint32_t below;
+    const int bl = rl >= 1 && rl <= (long long)n ? find_threshold_bin<kEstThreads>(hist, (uint32_t)rl, &below) : -1;
+    const int bh = rh < 1 || rh > (long long)n ? -1
+                   : rh == rl                  ? bl
+                                               : find_threshold_bin<kEstThreads>(hist, (uint32_t)rh, &below);
+    // every sample of bin b packs to [smin + b 2^shift, smin + (b + 1) 2^shift - 1]
+    if (bl >= 0) lo = ts.unpack(smin + ((unsigned long long)bl << shift));
+    if (bh >= 0) hi = ts.unpack(smin + ((unsigned long long)(bh + 1) << shift)) - 1;
   }
   if (tid == 0) {
     a.thr_lo[w] = lo;
     a.thr_hi[w] = hi;
+    a.scale[w] = make_int2(ts.ab, ts.db);
   }
 }
 
@@ -301,29 +333,33 @@ __global__ void __launch_bounds__(256) k4_evict_collect(EvictArgs a, uint32_t ch
   for (uint32_t it = blockIdx.x; it < items; it += gridDim.x) collect_chunk(a, a.act[it / chunks], it % chunks, chunks);
 }
 
-__global__ void __launch_bounds__(kSelThreads) k4_evict_select(EvictArgs a) {
-  __shared__ uint32_t hist[kBins];
-  __shared__ long long s_tmp[32];
+// T: 1,024 threads while there is an SM per instance; where there are more instances (their tables
+// are small then) 256, so that eight or more of them share an SM.
+template <int T>
+__global__ void __launch_bounds__(T) k4_evict_select(EvictArgs a) {
+  __shared__ __align__(16) uint32_t hist[kBins];
+  __shared__ uint4 s_v[kSelSmem], s_r[kRankMax];
   __shared__ unsigned s_cnt;
-  __shared__ unsigned long long s_or_hi, s_or_lo, s_v0_hi, s_v0_lo;
+  __shared__ unsigned long long s_or_hi, s_or_lo;
   chain_wait();
   const int w = a.only_w ? *a.only_w : blockIdx.x;
   if (block_error(a.err)) return;
   if (a.active[w] != 1) return;
-  const long long E = a.size[w] - a.desc[w].cap;
-  const int tid = threadIdx.x;
   const InstDesc d = a.desc[w];
+  const long long E = a.size[w] - d.cap;
+  const int tid = threadIdx.x;
   const uint32_t NB = 1u << d.log2nb;
   uint4* c0 = a.cand_a[w];
   unsigned cnt = a.n_cand[w];
   const unsigned nd = a.n_d[w];
   long long Erem = E - (long long)nd;
-  if (Erem <= 0 || Erem > (long long)cnt) {
+  const bool bracketed = Erem > 0 && Erem <= (long long)cnt, open = a.thr_hi[w] == ~0ull;
+  if (!bracketed) {
     // the bracket missed the E-th smallest: collect every entry of the instance here
     if (tid == 0) s_cnt = 0;
     __syncthreads();
     uint32_t* usl = a.slots[w];
-    for (uint32_t b = tid; b < NB; b += kSelThreads) {
+    for (uint32_t b = tid; b < NB; b += T) {
       for (int s = 0; s < 4; ++s) {
         const unsigned long long m = __ldcg(&d.tab[b].meta[s]);
         if (!m) continue;
@@ -341,58 +377,75 @@ __global__ void __launch_bounds__(kSelThreads) k4_evict_select(EvictArgs a) {
       a.n_d[w] = 0;
     }
   }
-  // radix narrowing over the candidates: each pass takes the 12 bits below the highest
-  // bit in which the remaining candidates differ and keeps the bin holding the target
-  uint4* cur = c0;
-  uint4* nxt = a.cand_b[w];
-  uint4* spare = a.cand_c[w];
-  for (int iter = 0; iter < 16 && cnt > 1; ++iter) {
+  // radix narrowing while there are many candidates, keeping the bin that holds the target, in
+  // shared memory as soon as it fits (the collected list, with its slots, is kept for the delete
+  // pass).  The first pass spreads the bracket over the bins in the samples' scale, which leaves a
+  // few entries; the others, hardly ever needed, take the 12 bits below the highest bit in which
+  // the entries differ.
+  const int2 sc = a.scale[w];
+  const TickScale ts{sc.x, sc.y};
+  const unsigned long long plo = ts.pack(a.thr_lo[w]);
+  const int tick_shift = max(0, 52 - __clzll((long long)(ts.pack(a.thr_hi[w]) - plo)));
+  const uint4* cur = c0;
+  for (int iter = 0; iter < 16 && cnt > (unsigned)kRankMax; ++iter) {
+    const bool tick = iter == 0 && bracketed && !open;
+    int shift = 0;
     if (tid == 0) {
-      s_v0_hi = v_hi(cur[0]);
-      s_v0_lo = v_lo(cur[0]);
       s_or_hi = 0;
       s_or_lo = 0;
+      s_cnt = 0;
     }
-    for (int i = tid; i < kBins; i += kSelThreads) hist[i] = 0;
+    for (int i = tid; i < kBins; i += T) hist[i] = 0;
     __syncthreads();
-    unsigned long long oh = 0, ol = 0;
-    for (unsigned i = tid; i < cnt; i += kSelThreads) {
-      const uint4 v = cur[i];
-      oh |= v_hi(v) ^ s_v0_hi;
-      ol |= v_lo(v) ^ s_v0_lo;
-    }
+    if (!tick) {
+      const uint4 v0 = cur[0];
+      unsigned long long oh = 0, ol = 0;
+#pragma unroll 4
+      for (unsigned i = tid; i < cnt; i += T) {
+        const uint4 v = cur[i];
+        oh |= v_hi(v) ^ v_hi(v0);
+        ol |= v_lo(v) ^ v_lo(v0);
+      }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      oh |= __shfl_xor_sync(kFull, oh, o);
-      ol |= __shfl_xor_sync(kFull, ol, o);
+      for (int o = 16; o > 0; o >>= 1) {
+        oh |= __shfl_xor_sync(kFull, oh, o);
+        ol |= __shfl_xor_sync(kFull, ol, o);
+      }
+      if ((tid & 31) == 0) {
+        if (oh) atomicOr(&s_or_hi, oh);
+        if (ol) atomicOr(&s_or_lo, ol);
+      }
+      __syncthreads();
+      const unsigned long long dh = s_or_hi, dl = s_or_lo;
+      if (dh == 0 && dl == 0) break;  // all equal (cannot happen for distinct keys)
+      const int top = dh ? 64 + 63 - __clzll((long long)dh) : 63 - __clzll((long long)dl);
+      shift = top >= 11 ? top - 11 : 0;
     }
-    if ((tid & 31) == 0) {
-      if (oh) atomicOr(&s_or_hi, oh);
-      if (ol) atomicOr(&s_or_lo, ol);
-    }
-    __syncthreads();
-    const unsigned long long dh = s_or_hi, dl = s_or_lo;
-    if (dh == 0 && dl == 0) break;  // all equal (cannot happen for distinct keys)
-    const int top = dh ? 64 + 63 - __clzll((long long)dh) : 63 - __clzll((long long)dl);
-    const int shift = top >= 11 ? top - 11 : 0;
-    for (unsigned i = tid; i < cnt; i += kSelThreads) {
+    auto bin_of = [&](const uint4& v) {
+      return tick ? (uint32_t)((ts.pack(v_hi(v)) - plo) >> tick_shift) : digit128(v_hi(v), v_lo(v), shift);
+    };
+#pragma unroll 4
+    for (unsigned i = tid; i < cnt; i += T) {
       const uint4 v = cur[i];
-      atomicAdd(&hist[digit128(v_hi(v), v_lo(v), shift)], 1u);
+      atomicAdd(&hist[bin_of(v)], 1u);
     }
     __syncthreads();
-    long long bl;
-    const int t = find_threshold_bin(hist, Erem, &bl, s_tmp);
+    uint32_t bl;
+    const int bin = find_threshold_bin<T>(hist, (uint32_t)Erem, &bl);
     Erem -= bl;
-    if (tid == 0) s_cnt = 0;
-    __syncthreads();
-    for (unsigned i0 = 0; i0 < cnt; i0 += kSelThreads) {
+    const unsigned kept = hist[bin];
+    uint4* nxt = kept <= (unsigned)kRankMax                 ? s_r
+                 : kept <= (unsigned)kSelSmem && cur != s_v ? s_v
+                                                            : (cur == a.cand_b[w] ? a.cand_c[w] : a.cand_b[w]);
+#pragma unroll 4
+    for (unsigned i0 = 0; i0 < cnt; i0 += T) {
       // keep the target bin: one shared add per warp, positions by ballot rank
       const unsigned i = i0 + tid;
       uint4 v = make_uint4(0, 0, 0, 0);
       bool keep = false;
       if (i < cnt) {
         v = cur[i];
-        keep = digit128(v_hi(v), v_lo(v), shift) == (uint32_t)t;
+        keep = bin_of(v) == (uint32_t)bin;
       }
       const unsigned bal = __ballot_sync(kFull, keep);
       unsigned base = 0;
@@ -401,30 +454,42 @@ __global__ void __launch_bounds__(kSelThreads) k4_evict_select(EvictArgs a) {
       if (keep) nxt[base + __popc(bal & lanemask_lt())] = v;
     }
     __syncthreads();
-    cnt = s_cnt;
-    uint4* done = cur;  // the collected list (with its slots) is kept for the delete pass
+    cnt = kept;
     cur = nxt;
-    nxt = (done == c0) ? spare : done;
-    __syncthreads();
   }
-  if (tid == 0) {
-    if (cnt < 1) set_error(a.err, MISAT_ERR_TABLE_FULL);
-    const uint4 v = cur[0];
-    a.theta[2 * w] = v_hi(v);
-    a.theta[2 * w + 1] = v_lo(v);
+  if (cnt > (unsigned)kRankMax || cnt < 1) {  // no instance holds two equal entries
+    if (tid == 0) set_error(a.err, MISAT_ERR_TABLE_FULL);
+    return;
+  }
+  if (cur != s_r)
+    for (unsigned i = tid; i < cnt; i += T) s_r[i] = cur[i];
+  __syncthreads();
+  // the target has Erem - 1 entries below it
+  if (tid < (int)cnt) {
+    const uint64_t mh = v_hi(s_r[tid]), ml = v_lo(s_r[tid]);
+    int rank = 0;
+#pragma unroll 4
+    for (unsigned j = 0; j < cnt; ++j) {
+      const uint64_t oh = v_hi(s_r[j]), ol = v_lo(s_r[j]);
+      rank += oh < mh || (oh == mh && ol < ml);
+    }
+    if (rank == (int)(Erem - 1)) {
+      a.theta[2 * w] = mh;
+      a.theta[2 * w + 1] = ml;
+    }
   }
 }
 
 namespace {
 // The apply passes take the entries of all instances over capacity as one index space, so
 // that every thread gets about the same number whatever the instances' shares: entry g
-// belongs to the k-th active instance with s_pre[k] <= g < s_pre[k + 1] (its D list first,
-// then its candidates).  Built by each CTA in shared memory; returns the total.
-__device__ unsigned long long list_prefix(const EvictArgs& a, unsigned long long* s_pre, int nact) {
+// belongs to the k-th active instance with s_pre[k] <= g < s_pre[k + 1].  Built by each CTA in
+// shared memory from the instances' list lengths; returns the total.
+template <class F>
+__device__ unsigned long long list_prefix(const EvictArgs& a, unsigned long long* s_pre, int nact, F&& len) {
   // the lengths are loaded in parallel, then warp 0 scans them 32 at a time
   for (int k = threadIdx.x; k < nact; k += blockDim.x) {
-    const int w = a.act[k];
-    s_pre[k + 1] = (unsigned long long)a.n_d[w] + a.n_cand[w];
+    s_pre[k + 1] = len(a.act[k]);
   }
   __syncthreads();
   if (threadIdx.x < 32) {
@@ -459,81 +524,119 @@ __device__ __forceinline__ int list_owner(const unsigned long long* s_pre, int n
   return lo;
 }
 
-// Delete slot sl of instance w's table; the global index (if any) loses bit w of its key.
-__device__ __forceinline__ void delete_slot(const GIndex& g, int w, Bucket* tab, uint32_t* dmask, uint32_t sl,
-                                            int32_t* err) {
-  const uint32_t b = sl >> 2, s = sl & 3;
-  if (g.keys && gix_clear(g, tab[b].key[s], w) < 0) set_error(err, MISAT_ERR_INTERNAL);
-  tab[b].key[s] = kEmpty;
-  tab[b].meta[s] = 0;
-  atomicOr(&dmask[b >> 3], 1u << ((b & 7) * 4 + s));
-}
 }  // namespace
 
-// Delete D and the candidates at or below theta; record them in the deleted-slot masks.
-// Deletions are counted per instance in shared memory and added to the sizes once per CTA.
+// Delete D and the candidates at or below theta; record them in the deleted-slot masks, and those in
+// full buckets in the list of holes to refill (a fifth of them).  A CTA takes pieces of 1,024
+// entries of one instance's lists (D first), four a thread with their loads in flight together:
+// what bounds it is the chain slot -> bitmap, slot -> key -> global index of scattered accesses.
+// The counters get one atomic per piece (with one per warp the pass waited for them: 95 us for
+// 1.5 million deletions).
+constexpr int kDelPer = 4;
+constexpr int kDelPiece = 256 * kDelPer;
 __global__ void __launch_bounds__(256) k4_evict_delete(EvictArgs a) {
   __shared__ unsigned long long s_pre[kMaxW + 1];
-  __shared__ unsigned s_del[kMaxW];
+  __shared__ unsigned s_cnt[2], s_base;
   chain_wait();
   if (block_error(a.err)) return;
   const int nact = (int)*(volatile const unsigned*)a.n_act;
-  for (int k = threadIdx.x; k < nact; k += blockDim.x) s_del[k] = 0;
-  const unsigned long long total = list_prefix(a, s_pre, nact);
-  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-  for (unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += stride) {
-    const int k = list_owner(s_pre, nact, g);
-    const int w = a.act[k];
-    const unsigned i = (unsigned)(g - s_pre[k]), nd = a.n_d[w];
-    uint32_t sl;
-    if (i < nd) {
-      sl = a.dslots[w][i];
-    } else {
-      const uint4 v = a.cand_a[w][i - nd];
-      if (!le128(v_hi(v), v_lo(v), a.theta[2 * w], a.theta[2 * w + 1])) continue;
-      sl = a.slots[w][i - nd];
-    }
-    delete_slot(a.gix, w, a.desc[w].tab, a.dmask[w], sl, a.err);
-    atomicAdd(&s_del[k], 1u);
-  }
-  __syncthreads();
+  auto len = [&](int w) { return (unsigned long long)a.n_d[w] + a.n_cand[w]; };
+  const unsigned long long total =
+      list_prefix(a, s_pre, nact, [&](int w) { return (len(w) + kDelPiece - 1) / kDelPiece; });
+  const int lane = threadIdx.x & 31;
   unsigned long long mine = 0;
-  for (int k = threadIdx.x; k < nact; k += blockDim.x) {
-    const unsigned d = s_del[k];
-    if (d) {
-      atomic_add_i64(&a.size[a.act[k]], -(long long)d);
-      mine += d;
+  for (unsigned long long it = blockIdx.x; it < total; it += gridDim.x) {
+    const int k = list_owner(s_pre, nact, it);
+    const int w = a.act[k];
+    const unsigned nd = a.n_d[w], n = nd + a.n_cand[w];
+    const unsigned i0 = (unsigned)(it - s_pre[k]) * kDelPiece + threadIdx.x;
+    const unsigned long long tm = a.theta[2 * w], tk = a.theta[2 * w + 1];
+    const uint32_t* bitmap = a.bitmaps[w];
+    Bucket* tab = a.desc[w].tab;
+    uint32_t* dmask = a.dmask[w];
+    if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
+    __syncthreads();
+    uint32_t sl[kDelPer];
+    bool del[kDelPer], hole[kDelPer];
+#pragma unroll
+    for (int j = 0; j < kDelPer; ++j) {
+      const unsigned i = i0 + 256 * j;
+      del[j] = i < n;
+      sl[j] = 0;
+      if (del[j]) {
+        sl[j] = i < nd ? a.dslots[w][i] : a.slots[w][i - nd];
+        if (i >= nd) {
+          const uint4 v = a.cand_a[w][i - nd];
+          del[j] = le128(v_hi(v), v_lo(v), tm, tk);
+        }
+      }
     }
+    // a hole in a bucket that was not full, the last of its run, needs no refill
+#pragma unroll
+    for (int j = 0; j < kDelPer; ++j) hole[j] = del[j] && ((bitmap[sl[j] >> 7] >> ((sl[j] >> 2) & 31)) & 1u);
+    unsigned at[kDelPer];
+#pragma unroll
+    for (int j = 0; j < kDelPer; ++j) {
+      const unsigned md = __ballot_sync(kFull, del[j]), mh = __ballot_sync(kFull, hole[j]);
+      unsigned base = 0;
+      if (lane == 0) {
+        if (md) atomicAdd(&s_cnt[0], (unsigned)__popc(md));
+        if (mh) base = atomicAdd(&s_cnt[1], (unsigned)__popc(mh));
+      }
+      at[j] = __shfl_sync(kFull, base, 0) + __popc(mh & lanemask_lt());
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      if (s_cnt[0]) atomic_add_i64(&a.size[w], -(long long)s_cnt[0]);
+      mine += s_cnt[0];
+      s_base = s_cnt[1] ? atomicAdd(&a.n_holes[w], s_cnt[1]) : 0;
+    }
+    if (a.gix.keys) {
+      unsigned long long key[kDelPer];
+#pragma unroll
+      for (int j = 0; j < kDelPer; ++j) key[j] = del[j] ? tab[sl[j] >> 2].key[sl[j] & 3] : 0;
+#pragma unroll
+      for (int j = 0; j < kDelPer; ++j)
+        if (del[j] && gix_clear(a.gix, key[j], w) < 0) set_error(a.err, MISAT_ERR_INTERNAL);
+    }
+#pragma unroll
+    for (int j = 0; j < kDelPer; ++j)
+      if (del[j]) {
+        const uint32_t b = sl[j] >> 2, s = sl[j] & 3;
+        tab[b].key[s] = kEmpty;
+        tab[b].meta[s] = 0;
+        atomicOr(&dmask[b >> 3], 1u << ((b & 7) * 4 + s));
+      }
+    __syncthreads();
+    uint32_t* list = reinterpret_cast<uint32_t*>(a.cand_b[w]) + s_base;
+#pragma unroll
+    for (int j = 0; j < kDelPer; ++j)
+      if (hole[j]) list[at[j]] = sl[j];
   }
-  const long long tot = block_sum((long long)mine);
-  if (threadIdx.x == 0 && tot) atomicAdd(a.evicted, (unsigned long long)tot);
+  if (threadIdx.x == 0 && mine) atomicAdd(a.evicted, mine);
 }
 
 // Refill the holes of every run of full buckets that lost an entry.  The thread of the
-// run's first deleted slot (lowest bucket, then lowest slot) owns the run.
+// run's first deleted slot (lowest bucket, then lowest slot) owns the run.  Bound by the latency of
+// its owner's dependent reads, five to ten for most runs, and lanes of a warp that walk different
+// runs take turns: only holes that may need a refill are listed (with all deletions and
+// candidates, ten a thread, it took 148 us in a batch of 65,536 requests), and neighbours in
+// the list go to different warps, so that a warp has more than one only when all have.
 __global__ void __launch_bounds__(256) k4_evict_shift(EvictArgs a) {
   __shared__ unsigned long long s_pre[kMaxW + 1];
   chain_wait();
   if (block_error(a.err)) return;
   const int nact = (int)*(volatile const unsigned*)a.n_act;
-  const unsigned long long total = list_prefix(a, s_pre, nact);
-  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-  for (unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += stride) {
+  const unsigned long long total = list_prefix(a, s_pre, nact, [&](int w) { return (unsigned long long)a.n_holes[w]; });
+  const unsigned warps = gridDim.x * (blockDim.x >> 5), warp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  for (unsigned long long g = (unsigned long long)(threadIdx.x & 31) * warps + warp; g < total; g += 32ull * warps) {
     const int k = list_owner(s_pre, nact, g);
     const int w = a.act[k];
-    const unsigned i = (unsigned)(g - s_pre[k]), nd = a.n_d[w];
+    const uint32_t sl = reinterpret_cast<const uint32_t*>(a.cand_b[w])[g - s_pre[k]];
     const uint32_t* full = a.bitmaps[w];
     const uint32_t* dmask = a.dmask[w];
     const InstDesc d = a.desc[w];
     const uint32_t NB = 1u << d.log2nb, mask = NB - 1;
-    uint32_t sl;
-    if (i < nd) {
-      sl = a.dslots[w][i];
-    } else {
-      const uint4 v = a.cand_a[w][i - nd];
-      if (!le128(v_hi(v), v_lo(v), a.theta[2 * w], a.theta[2 * w + 1])) continue;
-      sl = a.slots[w][i - nd];
-    }
     // the bitmap and deleted-mask words last read (runs are short: mostly one word each)
     uint32_t fw_i = 0xffffffffu, fw = 0, dw_i = 0xffffffffu, dw = 0;
     auto is_full = [&](uint32_t b) {
@@ -551,8 +654,6 @@ __global__ void __launch_bounds__(256) k4_evict_shift(EvictArgs a) {
       return (dw >> ((b & 7) * 4)) & 0xFu;
     };
     const uint32_t x = sl >> 2, sx = sl & 3;
-    // a hole in the last (not full) bucket of a run needs no refill
-    if (!is_full(x)) continue;
     // my deletion must be the lowest deleted slot of bucket x (the masks are not modified
     // by this kernel, unlike the buckets)
     if ((uint32_t)(__ffs(dmask_at(x)) - 1) != sx) continue;
@@ -629,12 +730,13 @@ int stream_grid(const EvictArgs& a, int chunks_per_inst, int resident) {
 void launch_evict_select(const EvictArgs& a, int chunks_per_inst, int num_sms, cudaStream_t st,
                          const cudaEvent_t* marks) {
   const int W = a.only_w ? 1 : a.W;
-  launch_chained(k4_evict_estimate, W, kSelThreads, 0, st, a);
+  launch_chained(k4_evict_estimate, W, kEstThreads, 0, st, a);
   if (marks) cudaEventRecord(marks[0], st);
   launch_chained(k4_evict_collect, stream_grid(a, chunks_per_inst, resident_grid<k4_evict_collect>(256, 0, num_sms)), 256,
                  0, st, a, (uint32_t)chunks_per_inst);
   if (marks) cudaEventRecord(marks[1], st);
-  launch_chained(k4_evict_select, W, kSelThreads, 0, st, a);
+  if (W <= num_sms) launch_chained(k4_evict_select<1024>, W, 1024, 0, st, a);
+  else launch_chained(k4_evict_select<256>, W, 256, 0, st, a);
   if (marks) cudaEventRecord(marks[2], st);
 }
 

@@ -449,10 +449,10 @@ __global__ void __launch_bounds__(32 * kHashWarps, kHashCtas) k1na_hash(HashArgs
 
 std::mutex g_noalloc_mu;
 unsigned long long* g_noalloc_ptr[256];  // device address of the scratch array, per device
-int g_noalloc_sms[256];
+int g_noalloc_sms[256], g_noalloc_ctas[256];  // SMs, resident CTAs of the hash
 
 // Per device, once, with that device current: the device address of the scratch array.
-int noalloc_setup(unsigned long long** scratch, int* sms) {
+int noalloc_setup(unsigned long long** scratch, int* sms, int* ctas) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 256) return MISAT_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_noalloc_mu);
@@ -465,10 +465,15 @@ int noalloc_setup(unsigned long long** scratch, int* sms) {
     int s = 0;
     if (cudaDeviceGetAttribute(&s, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return MISAT_ERR_CUDA;
     g_noalloc_sms[dev] = s;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k1na_hash, 32 * kHashWarps, 0) != cudaSuccess)
+      return MISAT_ERR_CUDA;
+    g_noalloc_ctas[dev] = s * (per_sm < 1 ? 1 : per_sm);
     g_noalloc_ptr[dev] = reinterpret_cast<unsigned long long*>(p);
   }
   *scratch = g_noalloc_ptr[dev];
   *sms = g_noalloc_sms[dev];
+  *ctas = g_noalloc_ctas[dev];
   return MISAT_OK;
 }
 
@@ -484,8 +489,8 @@ extern "C" int misat_block_hash_noalloc(const int64_t* tok_off, const int32_t* t
   if (!tok_off || (keys_cap > 0 && !keys_out)) return MISAT_ERR_INVALID_ARG;
   if (n_tokens > 0 && (!tokens || ((uintptr_t)tokens & 15) != 0)) return MISAT_ERR_INVALID_ARG;
   unsigned long long* scratch = nullptr;
-  int sms = 1;
-  int rc = noalloc_setup(&scratch, &sms);
+  int sms = 1, res = 1;
+  int rc = noalloc_setup(&scratch, &sms, &res);
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   HashArgs a{};
@@ -501,7 +506,6 @@ extern "C" int misat_block_hash_noalloc(const int64_t* tok_off, const int32_t* t
   a.off = reinterpret_cast<uint32_t*>(scratch + kNoAllocHead);
   a.list = reinterpret_cast<int32_t*>(scratch + kNoAllocHead) + n;
   a.long_blocks = hash_long_blocks(n_tokens, sms);
-  const int res = resident_grid<k1na_hash>(32 * kHashWarps, 0, sms);
   a.group = hash_group_size(n, res * kHashWarps);
   if (cudaMemsetAsync(scratch, 0, 8 * sizeof(*scratch), st) != cudaSuccess) return MISAT_ERR_CUDA;
   k1na_offsets<<<(n + kHashTile - 1) / kHashTile, kHashTile, 0, st>>>(a, scratch);

@@ -304,15 +304,17 @@ struct EvictArgs {
   long long* size;             // [W]
   uint32_t* const* bitmaps;    // [W] per instance fullness bitmap (NB/32 words)
   uint4* const* cand_a;        // [W] candidate lists (meta, key) as uint4: the collected list
-  uint4* const* cand_b;        //     and two work lists of the radix narrowing
+  uint4* const* cand_b;        //     and two work lists of the radix narrowing (b then holds the holes)
   uint4* const* cand_c;
   uint32_t* const* slots;      // [W] slot (bucket*4+s) of each entry of cand_a
   uint32_t* const* dslots;     // [W] slots certainly evicted (meta below the bracket)
   uint32_t* const* dmask;      // [W] deleted-slot mask, 4 bits per bucket (NB/8 words)
   unsigned* n_cand;            // [W] entries in cand_a
   unsigned* n_d;               // [W] entries in dslots
+  unsigned* n_holes;           // [W] deleted slots of full buckets, listed in cand_b
   unsigned long long* thr_lo;  // [W] meta bracket of the E-th smallest
   unsigned long long* thr_hi;  // [W]
+  int2* scale;                 // [W] bits of the sampled arrivals and depths
   unsigned long long* theta;   // [W*2] (meta, key)
   int32_t* active;             // [W] 1: delete entries <= theta, 2: marked entries only
   unsigned long long* evicted;
