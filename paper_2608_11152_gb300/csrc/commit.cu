@@ -17,17 +17,16 @@ namespace misat {
 namespace {
 constexpr unsigned kFull = 0xffffffffu;
 
-// Find-or-claim `key` in an instance table and merge `meta`, starting at bucket `b` whose
-// four keys the caller has already read into k[] (possibly stale: keys are only ever
-// added while inserts run, so a stale read can only miss a claim, which the CAS catches).
-// Returns 1 if the key was new, 0 if it existed, -1 if no free slot was found.
-__device__ __forceinline__ int table_insert_at(const InstDesc& d, uint64_t key, uint64_t meta, uint32_t b,
-                                               unsigned long long k[4]) {
+// Find-or-claim `key` in an instance table and merge `meta`.  Returns 1 if the key was new, 0 if it
+// existed, -1 if no free slot was found.
+__device__ __forceinline__ int table_insert(const InstDesc& d, uint64_t key, uint64_t meta) {
   const uint32_t mask = (1u << d.log2nb) - 1;
+  uint32_t b = home_bucket(key, d.log2nb);
   for (uint32_t it = 0; it <= mask; ++it) {
     Bucket* B = d.tab + b;
     for (int tries = 0; tries < 2 * kSlots; ++tries) {
-      if (it | tries) ld_bucket_keys_cg(B, k);
+      unsigned long long k[4];
+      ld_bucket_keys_cg(B, k);
       int s = -1;
 #pragma unroll
       for (int i = 0; i < 4; ++i)
@@ -53,13 +52,6 @@ __device__ __forceinline__ int table_insert_at(const InstDesc& d, uint64_t key, 
   return -1;
 }
 
-__device__ __forceinline__ int table_insert(const InstDesc& d, uint64_t key, uint64_t meta) {
-  const uint32_t b = home_bucket(key, d.log2nb);
-  unsigned long long k[4];
-  ld_bucket_keys_cg(d.tab + b, k);
-  return table_insert_at(d, key, meta, b, k);
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -69,10 +61,14 @@ __device__ __forceinline__ int table_insert(const InstDesc& d, uint64_t key, uin
 // (pointer to its first key, the instance table, the tick of its request, first depth,
 // instance, table size, block count), so a warp reaches its keys in one dependent load
 // instead of walking request -> instance -> table descriptor.  A warp then inserts one unit:
-// lane l takes blocks l, l+32, l+64, l+96 of it and issues all four home-bucket reads
-// before the first atomic; a key already present costs one fire-and-forget atomicMax on
-// its meta, a new one a CAS.  While those are in flight the warp already loads its next
-// unit's record and keys (software pipelining over the warp's units).  The order of the
+// lane l takes blocks l, l+32, l+64, l+96 of it side by side: four bucket reads in flight, then
+// four claims, then for whatever is left the next buckets.  A key already present costs one
+// fire-and-forget atomicMax on its meta, a new one a CAS.  While the first reads are in flight
+// the warp already loads its next unit's record and keys (software pipelining over the
+// warp's units).  One key after the other, a lane waited for each claim, and for each second
+// bucket of the seventh of the keys whose home bucket is full (us before and now: 4,096 requests
+// 27/22, 16,384 31/28, 9,216 with long prompts 67/60, 65,536 130/124, where the scattered accesses
+// themselves bound it).  Units of up to 32 blocks skip the other three keys.  The order of the
 // units is free: the final key set and metas do not depend on it.
 constexpr int kIns = 4;
 constexpr int kUnitBlocks = 32 * kIns;
@@ -104,6 +100,62 @@ __device__ __forceinline__ UnitRec load_unit(const int4* units, int64_t u) {
 __device__ __forceinline__ void load_unit_keys(const UnitRec& u, int lane, uint64_t key[kIns]) {
 #pragma unroll
   for (int k = 0; k < kIns; ++k) key[k] = lane + 32 * k < u.cnt ? __ldg(u.keys + lane + 32 * k) : 0;
+}
+
+// Places the lane's first N keys of a unit whose home buckets (hb) have been read into kk, side by
+// side; returns the mask of those that were new.  (A bucket seen full is passed for good and a lost
+// claim fills a slot, so at most kSlots turns a bucket; what is read may be stale, but keys are only
+// ever added while inserts run, so it can only miss a claim, which the CAS catches.)
+template <int N>
+__device__ __forceinline__ unsigned place_keys(const UnitRec& u, const uint64_t* key, uint32_t* hb,
+                                               unsigned long long (*kk)[4], int lane, int32_t* err) {
+  const uint32_t mask = (1u << u.log2nb) - 1;
+  unsigned pend = 0, isnew = 0;
+#pragma unroll
+  for (int k = 0; k < N; ++k) pend |= lane + 32 * k < u.cnt ? 1u << k : 0u;
+  for (uint32_t turn = 0; pend; ++turn) {
+    if (turn > (uint32_t)kSlots * mask + 2 * kSlots) {
+      set_error(err, MISAT_ERR_TABLE_FULL);
+      break;
+    }
+    int e[N];
+    unsigned long long old[N];
+    if (turn) {
+#pragma unroll
+      for (int k = 0; k < N; ++k)
+        if ((pend >> k) & 1u) ld_bucket_keys_cg(u.tab + hb[k], kk[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      e[k] = -1;
+      old[k] = 0;
+      if (!((pend >> k) & 1u)) continue;
+      Bucket* B = u.tab + hb[k];
+      int s = -1;
+#pragma unroll
+      for (int i = 3; i >= 0; --i) {
+        if (kk[k][i] == key[k]) s = i;
+        if (kk[k][i] == kEmpty) e[k] = i;
+      }
+      if (s >= 0) {
+        atomicMax(&B->meta[s], (unsigned long long)(u.mhi - (uint64_t)(u.j0 + lane + 32 * k)));
+        pend &= ~(1u << k);
+        e[k] = -1;
+      } else if (e[k] >= 0) {
+        old[k] = atomicCAS(&B->key[e[k]], kEmpty, (unsigned long long)key[k]);
+      } else {
+        hb[k] = (hb[k] + 1) & mask;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      if (e[k] < 0 || !(old[k] == kEmpty || old[k] == key[k])) continue;
+      atomicMax(&u.tab[hb[k]].meta[e[k]], (unsigned long long)(u.mhi - (uint64_t)(u.j0 + lane + 32 * k)));
+      isnew |= old[k] == kEmpty ? 1u << k : 0u;
+      pend &= ~(1u << k);
+    }
+  }
+  return isnew;
 }
 
 // Session table update at commit (Sec. 4.1: an admitted new session becomes pending /
@@ -285,22 +337,11 @@ __global__ void __launch_bounds__(kInsThreads, 3) k4_insert(InsertArgs a) {
       nxt = load_unit(units, u + warps);
       load_unit_keys(nxt, lane, nkey);
     }
-    const InstDesc d{cur.tab, cur.log2nb, 0, 0};
+    const unsigned isnew = cur.cnt > 32 ? place_keys<kIns>(cur, key, hb, kk, lane, a.err) : place_keys<1>(cur, key, hb, kk, lane, a.err);
+    __syncwarp();
     unsigned cnt = 0;
-    int isnew[kIns];
 #pragma unroll
-    for (int k = 0; k < kIns; ++k) {
-      const int j = lane + 32 * k;
-      isnew[k] = 0;
-      if (j < cur.cnt) {
-        const int res = table_insert_at(d, key[k], cur.mhi - (uint64_t)(cur.j0 + j), hb[k], kk[k]);
-        if (res < 0)
-          set_error(a.err, MISAT_ERR_TABLE_FULL);
-        else
-          isnew[k] = res;
-      }
-      cnt += __popc(__ballot_sync(kFull, isnew[k]));
-    }
+    for (int k = 0; k < kIns; ++k) cnt += __popc(__ballot_sync(kFull, (isnew >> k) & 1u));
     if (a.gix.keys && cnt) {
       // keys new to instance w are listed for the global-index pass (one slot range per warp)
       unsigned base = 0;
@@ -308,8 +349,9 @@ __global__ void __launch_bounds__(kInsThreads, 3) k4_insert(InsertArgs a) {
       base = __shfl_sync(kFull, base, 0);
 #pragma unroll
       for (int k = 0; k < kIns; ++k) {
-        const unsigned bal = __ballot_sync(kFull, isnew[k]);
-        if (isnew[k]) {
+        const bool mine = (isnew >> k) & 1u;
+        const unsigned bal = __ballot_sync(kFull, mine);
+        if (mine) {
           const unsigned pos = base + __popc(bal & lanemask_lt());
           if ((int64_t)pos < a.gnew_cap)
             a.gnew[pos] = make_ulonglong2((unsigned long long)key[k], (unsigned long long)cur.w);

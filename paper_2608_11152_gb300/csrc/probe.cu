@@ -85,8 +85,11 @@ __global__ void __launch_bounds__(256) k2_first_claim(ProbeArgs a) {
   }
 }
 
-constexpr int kDistIlp = 4;  // tables per lane with their home sectors in flight together
-
+// kDistIlp: tables per lane that are looked up side by side (1, 2 or 4, as many as the instances
+// need).  One after the other, a lane waited for the next bucket of each of the seventh of its
+// tables whose home bucket is full (108/100 us at 27,000 keys x 128 instances, 95/85 at 53,000 x
+// 64: what is left is the rate of scattered 64-byte reads).
+template <int kDistIlp>
 __global__ void __launch_bounds__(256) k2_probe_distinct(ProbeArgs a) {
   __shared__ Bucket* s_tab[kMaxW];
   __shared__ uint32_t s_lg[kMaxW];
@@ -101,43 +104,55 @@ __global__ void __launch_bounds__(256) k2_probe_distinct(ProbeArgs a) {
   const int nd = (int)*a.fb_count;
   const uint32_t mw = a.fb.mw;
   unsigned long long probes = 0, reads = 0;
-  for (int d = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; d < nd; d += (gridDim.x * blockDim.x) >> 5) {
-    const int64_t slot = a.fb_list[d];
-    const uint64_t key = a.fb.keys[slot];
+  const int warps = (gridDim.x * blockDim.x) >> 5;
+  int d = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  // the next key is on its way while this one is looked up
+  int64_t slot = d < nd ? a.fb_list[d] : 0;
+  uint64_t key = d < nd ? a.fb.keys[slot] : 0;
+  int64_t slot_n = d + warps < nd ? a.fb_list[d + warps] : 0;
+  for (; d < nd; d += warps) {
+    const uint64_t key_n = d + warps < nd ? a.fb.keys[slot_n] : 0;
+    const int64_t slot_nn = d + 2 * warps < nd ? a.fb_list[d + 2 * warps] : 0;
     for (int w0 = 0; w0 < a.W; w0 += 32 * kDistIlp) {
-      // the home-bucket sectors of the lane's kDistIlp tables are requested before any is
-      // examined; a full home bucket without the key continues its probe sequence after
-      ulonglong2 k01[kDistIlp], k23[kDistIlp];
+      // the lane's kDistIlp tables side by side: their home-bucket sectors, then the next
+      // buckets of those whose bucket is full without the key
+      uint32_t b[kDistIlp];
+      unsigned pend = 0, hit = 0;
 #pragma unroll
       for (int i = 0; i < kDistIlp; ++i) {
         const int w = w0 + 32 * i + lane;
-        k01[i] = make_ulonglong2(kEmpty, kEmpty);
-        k23[i] = k01[i];
         if (w < a.W) {
-          const ulonglong2* p = reinterpret_cast<const ulonglong2*>(s_tab[w][home_bucket(key, s_lg[w])].key);
-          k01[i] = __ldg(p);
-          k23[i] = __ldg(p + 1);
+          pend |= 1u << i;
+          b[i] = home_bucket(key, s_lg[w]);
+          probes += 1;
         }
       }
+      for (uint32_t turn = 0; pend; ++turn) {
+        ulonglong2 k01[kDistIlp], k23[kDistIlp];
 #pragma unroll
-      for (int i = 0; i < kDistIlp; ++i) {
-        const int w = w0 + 32 * i + lane;
-        int h = 0;
-        if (w < a.W) {
-          h = (k01[i].x == key) | (k01[i].y == key) | (k23[i].x == key) | (k23[i].y == key);
+        for (int i = 0; i < kDistIlp; ++i)
+          if ((pend >> i) & 1u) {
+            const ulonglong2* p = reinterpret_cast<const ulonglong2*>(s_tab[w0 + 32 * i + lane][b[i]].key);
+            k01[i] = __ldg(p);
+            k23[i] = __ldg(p + 1);
+          }
+#pragma unroll
+        for (int i = 0; i < kDistIlp; ++i) {
+          if (!((pend >> i) & 1u)) continue;
+          const uint32_t mask = (1u << s_lg[w0 + 32 * i + lane]) - 1;
+          const bool h = (k01[i].x == key) | (k01[i].y == key) | (k23[i].x == key) | (k23[i].y == key);
           const bool open =
               (k01[i].x == kEmpty) | (k01[i].y == kEmpty) | (k23[i].x == kEmpty) | (k23[i].y == kEmpty);
-          uint32_t rd = 1;
-          if (!h && !open) {
-            InstDesc dd;
-            dd.tab = s_tab[w];
-            dd.log2nb = s_lg[w];
-            h = table_contains_from(dd, key, (home_bucket(key, dd.log2nb) + 1) & ((1u << dd.log2nb) - 1), &rd);
-          }
-          probes += 1;
-          reads += rd;
+          reads += 1;
+          hit |= h ? 1u << i : 0u;
+          if (h || open || turn >= mask) pend &= ~(1u << i);
+          b[i] = (b[i] + 1) & mask;
         }
-        const unsigned m = __ballot_sync(0xffffffffu, h);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < kDistIlp; ++i) {
+        const unsigned m = __ballot_sync(0xffffffffu, (hit >> i) & 1u);
         if (lane == 0) {
           const int wb = w0 + 32 * i;
           if (wb < a.W) {
@@ -147,6 +162,9 @@ __global__ void __launch_bounds__(256) k2_probe_distinct(ProbeArgs a) {
         }
       }
     }
+    slot = slot_n;
+    key = key_n;
+    slot_n = slot_nn;
   }
   block_add_stats(a.stats, probes, reads);
 }
@@ -362,7 +380,8 @@ void launch_probe_first(const ProbeArgs& a, int num_sms, cudaStream_t st) {
   }
   // per-instance tables: the context allocates the batch-local index with the tables
   launch_chained(k2_first_claim, ggrid, 256, 0, st, a);
-  launch_chained(k2_probe_distinct, num_sms * 8, 256, 0, st, a);  // two waves: measured faster than one for this pass
+  const auto distinct = a.W <= 32 ? k2_probe_distinct<1> : (a.W <= 64 ? k2_probe_distinct<2> : k2_probe_distinct<4>);
+  launch_chained(distinct, num_sms * 8, 256, 0, st, a);  // two waves: measured faster than one for this pass
   ProbeArgs e = a;
   e.gix = a.fb;
   e.stats = a.stats_fb;
