@@ -572,13 +572,24 @@ EvictArgs evict_args(misat_ctx* c, unsigned long long* evicted_counter) {
   return ev;
 }
 
+uint32_t max_log2nb(const misat_ctx* c) {
+  uint32_t m = 1;
+  for (const auto& d : c->h_desc) m = std::max(m, d.log2nb);
+  return m;
+}
+
 // Eviction of every instance above capacity (d_nact zeroed before); `join` (may be NULL) is waited
 // for between the read-only half and the deletions.
 int evict_all(misat_ctx* c, unsigned long long* evicted_counter, cudaEvent_t join = nullptr) {
   const EvictArgs ev = evict_args(c, evicted_counter);
+  const uint32_t maxlg = max_log2nb(c);
+  if (evict_is_small(maxlg)) {
+    if (join) CK(cudaStreamWaitEvent(c->stream, join, 0));
+    launch_evict_small(ev, c->stream);
+    for (int i = 12; i < 17; ++i) c->mark(i);
+    return cudaGetLastError() == cudaSuccess ? MISAT_OK : MISAT_ERR_CUDA;
+  }
   // streaming CTAs per instance: about 4 buckets per thread, at most 256 CTAs of 256
-  uint32_t maxlg = 1;
-  for (auto& d : c->h_desc) maxlg = std::max(maxlg, d.log2nb);
   const int chunks = (int)std::min<uint64_t>(256, std::max<uint64_t>(1, ((uint64_t)1 << maxlg) / (4 * 256)));
   // with phase timing there is an event after each kernel
   const cudaEvent_t* marks = c->timing ? c->ev + 12 : nullptr;
@@ -1292,7 +1303,7 @@ int misat_commit(misat_ctx* c) {
     c->mark(9);
     cudaEvent_t join = nullptr;
     if (ia.gix.keys) {
-      if (c->side_stream && !c->timing) {
+      if (c->side_stream && !c->timing && !evict_is_small(max_log2nb(c))) {
         CK(cudaEventRecord(c->ev_fork, st));
         CK(cudaStreamWaitEvent(c->side_stream, c->ev_fork, 0));
         launch_insert_gix(ia, c->num_sms * 4, c->side_stream);

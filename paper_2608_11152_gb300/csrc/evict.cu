@@ -112,17 +112,75 @@ struct TickScale {
   }
 };
 
+struct EstPart {
+  unsigned long long mn, mx;   // smallest and largest sampled meta
+  unsigned occ, arr, dep;      // samples, their largest arrival and depth
+};
+constexpr int kEstMetas = 4 * kEstBuckets / kEstThreads;  // per thread
+
+// The thread's metas of nsb of the table's NB buckets (powers of two), evenly spaced: slot s of
+// sampled bucket threadIdx.x + k kEstThreads is m[4k + s].
+__device__ __forceinline__ void load_metas(const InstDesc& d, uint32_t NB, uint32_t nsb, unsigned long long* m) {
+#pragma unroll
+  for (int k = 0; k < kEstMetas / 4; ++k) {
+    const uint32_t i = threadIdx.x + k * kEstThreads;
+    ulonglong2 m01 = make_ulonglong2(0, 0), m23 = m01;
+    if (i < nsb) {
+      const ulonglong2* mp = reinterpret_cast<const ulonglong2*>(d.tab[i * (NB / nsb)].meta);
+      m01 = __ldcg(mp);
+      m23 = __ldcg(mp + 1);
+    }
+    m[4 * k] = m01.x;
+    m[4 * k + 1] = m01.y;
+    m[4 * k + 2] = m23.x;
+    m[4 * k + 3] = m23.y;
+  }
+}
+
+// Range of the block's metas (one block barrier).
+__device__ __forceinline__ EstPart sample_range(const unsigned long long* m, EstPart* s_part) {
+  unsigned long long mn = ~0ull, mx = 0;
+  unsigned occ = 0, arr = 0, dep = 0;
+#pragma unroll
+  for (int k = 0; k < kEstMetas; ++k)
+    if (m[k]) {
+      ++occ;
+      mn = m[k] < mn ? m[k] : mn;
+      mx = m[k] > mx ? m[k] : mx;
+      arr = max(arr, (unsigned)(m[k] >> 16) & 0xfffffu);
+      dep = max(dep, 0xffffu - ((unsigned)m[k] & 0xffffu));
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long a1 = __shfl_xor_sync(kFull, mn, o), a2 = __shfl_xor_sync(kFull, mx, o);
+    mn = a1 < mn ? a1 : mn;
+    mx = a2 > mx ? a2 : mx;
+  }
+  occ = __reduce_add_sync(kFull, occ);
+  arr = __reduce_max_sync(kFull, arr);
+  dep = __reduce_max_sync(kFull, dep);
+  if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = EstPart{mn, mx, occ, arr, dep};
+  __syncthreads();
+  EstPart all = s_part[0];
+#pragma unroll
+  for (int k = 1; k < kEstThreads / 32; ++k) {
+    const EstPart p = s_part[k];
+    all.mn = p.mn < all.mn ? p.mn : all.mn;
+    all.mx = p.mx > all.mx ? p.mx : all.mx;
+    all.occ += p.occ;
+    all.arr = max(all.arr, p.arr);
+    all.dep = max(all.dep, p.dep);
+  }
+  return all;
+}
+
 // Bound by latency: one round of loads and a few block barriers.  The samples stay in registers,
 // and a bin is a shift (with 128-bit quotients of equal bins it took 16 us, on tables of any
 // size); 2,048 buckets instead of 512 make the bracket, and U with it, half as wide.
 __global__ void __launch_bounds__(kEstThreads) k4_evict_estimate(EvictArgs a) {
   constexpr int kPer = kEstBuckets / kEstThreads;
   __shared__ __align__(16) uint32_t hist[kBins];
-  struct Part {
-    unsigned long long mn, mx;
-    unsigned occ, arr, dep;
-  };
-  __shared__ Part s_part[kEstThreads / 32];
+  __shared__ EstPart s_part[kEstThreads / 32];
   chain_wait();
   const int w = a.only_w ? *a.only_w : blockIdx.x;
   if (block_error(a.err)) return;
@@ -141,53 +199,9 @@ __global__ void __launch_bounds__(kEstThreads) k4_evict_estimate(EvictArgs a) {
   const uint32_t NB = 1u << d.log2nb;
   const uint32_t nsb = NB < (uint32_t)kEstBuckets ? NB : (uint32_t)kEstBuckets;  // powers of two
   unsigned long long m[4 * kPer];
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    const uint32_t i = tid + k * kEstThreads;
-    ulonglong2 m01 = make_ulonglong2(0, 0), m23 = m01;
-    if (i < nsb) {
-      const ulonglong2* mp = reinterpret_cast<const ulonglong2*>(d.tab[i * (NB / nsb)].meta);
-      m01 = __ldcg(mp);
-      m23 = __ldcg(mp + 1);
-    }
-    m[4 * k] = m01.x;
-    m[4 * k + 1] = m01.y;
-    m[4 * k + 2] = m23.x;
-    m[4 * k + 3] = m23.y;
-  }
+  load_metas(d, NB, nsb, m);
   for (int i = tid; i < kBins; i += kEstThreads) hist[i] = 0;
-  unsigned long long mn = ~0ull, mx = 0;
-  unsigned occ = 0, arr = 0, dep = 0;
-#pragma unroll
-  for (int k = 0; k < 4 * kPer; ++k)
-    if (m[k]) {
-      ++occ;
-      mn = m[k] < mn ? m[k] : mn;
-      mx = m[k] > mx ? m[k] : mx;
-      arr = max(arr, (unsigned)(m[k] >> 16) & 0xfffffu);
-      dep = max(dep, 0xffffu - ((unsigned)m[k] & 0xffffu));
-    }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long a1 = __shfl_xor_sync(kFull, mn, o), a2 = __shfl_xor_sync(kFull, mx, o);
-    mn = a1 < mn ? a1 : mn;
-    mx = a2 > mx ? a2 : mx;
-  }
-  occ = __reduce_add_sync(kFull, occ);
-  arr = __reduce_max_sync(kFull, arr);
-  dep = __reduce_max_sync(kFull, dep);
-  if ((tid & 31) == 0) s_part[tid >> 5] = Part{mn, mx, occ, arr, dep};
-  __syncthreads();
-  Part all = s_part[0];
-#pragma unroll
-  for (int k = 1; k < kEstThreads / 32; ++k) {
-    const Part p = s_part[k];
-    all.mn = p.mn < all.mn ? p.mn : all.mn;
-    all.mx = p.mx > all.mx ? p.mx : all.mx;
-    all.occ += p.occ;
-    all.arr = max(all.arr, p.arr);
-    all.dep = max(all.dep, p.dep);
-  }
+  const EstPart all = sample_range(m, s_part);
   const unsigned n = all.occ;
   const TickScale ts{32 - __clz(all.arr), 32 - __clz(all.dep)};
   unsigned long long lo = 0, hi = ~0ull;
@@ -616,6 +630,93 @@ __global__ void __launch_bounds__(256) k4_evict_delete(EvictArgs a) {
   if (threadIdx.x == 0 && mine) atomicAdd(a.evicted, mine);
 }
 
+namespace {
+// Refills the holes of the run of full buckets that deleted slot sl of a full bucket belongs to, if
+// that is the run's first deleted slot (lowest bucket, then lowest slot).  full, dmask: the
+// table's fullness bits and deleted slots (four bits a bucket) before any refill.
+__device__ __forceinline__ void refill_run(const InstDesc d, const uint32_t* full, const uint32_t* dmask, uint32_t sl) {
+  const uint32_t NB = 1u << d.log2nb, mask = NB - 1;
+      // the bitmap and deleted-mask words last read (runs are short: mostly one word each)
+      uint32_t fw_i = 0xffffffffu, fw = 0, dw_i = 0xffffffffu, dw = 0;
+      auto is_full = [&](uint32_t b) {
+        if ((b >> 5) != fw_i) {
+          fw_i = b >> 5;
+          fw = full[fw_i];
+        }
+        return (fw >> (b & 31)) & 1u;
+      };
+      auto dmask_at = [&](uint32_t b) {
+        if ((b >> 3) != dw_i) {
+          dw_i = b >> 3;
+          dw = dmask[dw_i];
+        }
+        return (dw >> ((b & 7) * 4)) & 0xFu;
+      };
+      const uint32_t x = sl >> 2, sx = sl & 3;
+      // my deletion must be the lowest deleted slot of bucket x (the masks are not modified
+      // by this kernel, unlike the buckets)
+      if ((uint32_t)(__ffs(dmask_at(x)) - 1) != sx) return;
+      // run start: walk back over full buckets; no earlier bucket of the run may hold a deletion
+      uint32_t s0 = x, len = 0;
+      bool lead = true;
+      while (is_full((s0 - 1) & mask) && len < NB) {
+        s0 = (s0 - 1) & mask;
+        ++len;
+        if (dmask_at(s0)) {
+          lead = false;
+          break;
+        }
+      }
+      if (!lead) return;
+      // run end: the first bucket after x that was not full
+      uint32_t e = x, rl = 0;
+      while (is_full(e) && rl < NB) {
+        e = (e + 1) & mask;
+        ++rl;
+      }
+      const uint32_t runlen = ((e - s0) & mask);  // buckets s0 .. e-1 are full, e ends the run
+      for (uint32_t ii = 0; ii < runlen; ++ii) {
+        Bucket* X = d.tab + ((s0 + ii) & mask);
+        unsigned long long xk[4];
+        {
+          const ulonglong2* p = reinterpret_cast<const ulonglong2*>(X->key);
+          const ulonglong2 u0 = p[0], u1 = p[1];
+          xk[0] = u0.x;
+          xk[1] = u0.y;
+          xk[2] = u1.x;
+          xk[3] = u1.y;
+        }
+        bool stop = false;
+  #pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          if (stop || xk[s] != kEmpty) continue;
+          bool moved = false;
+          for (uint32_t j = ii + 1; j <= runlen && !moved; ++j) {
+            Bucket* Y = d.tab + ((s0 + j) & mask);
+            const ulonglong2* p = reinterpret_cast<const ulonglong2*>(Y->key);
+            const ulonglong2 u0 = p[0], u1 = p[1];
+            const unsigned long long yk[4] = {u0.x, u0.y, u1.x, u1.y};
+  #pragma unroll
+            for (int t = 0; t < 4; ++t) {
+              const unsigned long long k = yk[t];
+              if (moved || k == kEmpty) continue;
+              const uint32_t rel = (home_bucket(k, d.log2nb) - s0) & mask;
+              if (rel <= ii) {
+                X->key[s] = k;
+                X->meta[s] = Y->meta[t];
+                Y->key[t] = kEmpty;
+                Y->meta[t] = 0;
+                xk[s] = k;
+                moved = true;
+              }
+            }
+          }
+          if (!moved) stop = true;  // no later entry of the run can move into this bucket
+        }
+      }
+}
+}  // namespace
+
 // Refill the holes of every run of full buckets that lost an entry.  The thread of the
 // run's first deleted slot (lowest bucket, then lowest slot) owns the run.  Bound by the latency of
 // its owner's dependent reads, five to ten for most runs, and lanes of a warp that walk different
@@ -633,91 +734,139 @@ __global__ void __launch_bounds__(256) k4_evict_shift(EvictArgs a) {
     const int k = list_owner(s_pre, nact, g);
     const int w = a.act[k];
     const uint32_t sl = reinterpret_cast<const uint32_t*>(a.cand_b[w])[g - s_pre[k]];
-    const uint32_t* full = a.bitmaps[w];
-    const uint32_t* dmask = a.dmask[w];
-    const InstDesc d = a.desc[w];
-    const uint32_t NB = 1u << d.log2nb, mask = NB - 1;
-    // the bitmap and deleted-mask words last read (runs are short: mostly one word each)
-    uint32_t fw_i = 0xffffffffu, fw = 0, dw_i = 0xffffffffu, dw = 0;
-    auto is_full = [&](uint32_t b) {
-      if ((b >> 5) != fw_i) {
-        fw_i = b >> 5;
-        fw = full[fw_i];
-      }
-      return (fw >> (b & 31)) & 1u;
-    };
-    auto dmask_at = [&](uint32_t b) {
-      if ((b >> 3) != dw_i) {
-        dw_i = b >> 3;
-        dw = dmask[dw_i];
-      }
-      return (dw >> ((b & 7) * 4)) & 0xFu;
-    };
-    const uint32_t x = sl >> 2, sx = sl & 3;
-    // my deletion must be the lowest deleted slot of bucket x (the masks are not modified
-    // by this kernel, unlike the buckets)
-    if ((uint32_t)(__ffs(dmask_at(x)) - 1) != sx) continue;
-    // run start: walk back over full buckets; no earlier bucket of the run may hold a deletion
-    uint32_t s0 = x, len = 0;
-    bool lead = true;
-    while (is_full((s0 - 1) & mask) && len < NB) {
-      s0 = (s0 - 1) & mask;
-      ++len;
-      if (dmask_at(s0)) {
-        lead = false;
-        break;
-      }
-    }
-    if (!lead) continue;
-    // run end: the first bucket after x that was not full
-    uint32_t e = x, rl = 0;
-    while (is_full(e) && rl < NB) {
-      e = (e + 1) & mask;
-      ++rl;
-    }
-    const uint32_t runlen = ((e - s0) & mask);  // buckets s0 .. e-1 are full, e ends the run
-    for (uint32_t ii = 0; ii < runlen; ++ii) {
-      Bucket* X = d.tab + ((s0 + ii) & mask);
-      unsigned long long xk[4];
-      {
-        const ulonglong2* p = reinterpret_cast<const ulonglong2*>(X->key);
-        const ulonglong2 u0 = p[0], u1 = p[1];
-        xk[0] = u0.x;
-        xk[1] = u0.y;
-        xk[2] = u1.x;
-        xk[3] = u1.y;
-      }
-      bool stop = false;
-#pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        if (stop || xk[s] != kEmpty) continue;
-        bool moved = false;
-        for (uint32_t j = ii + 1; j <= runlen && !moved; ++j) {
-          Bucket* Y = d.tab + ((s0 + j) & mask);
-          const ulonglong2* p = reinterpret_cast<const ulonglong2*>(Y->key);
-          const ulonglong2 u0 = p[0], u1 = p[1];
-          const unsigned long long yk[4] = {u0.x, u0.y, u1.x, u1.y};
-#pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const unsigned long long k = yk[t];
-            if (moved || k == kEmpty) continue;
-            const uint32_t rel = (home_bucket(k, d.log2nb) - s0) & mask;
-            if (rel <= ii) {
-              X->key[s] = k;
-              X->meta[s] = Y->meta[t];
-              Y->key[t] = kEmpty;
-              Y->meta[t] = 0;
-              xk[s] = k;
-              moved = true;
-            }
-          }
-        }
-        if (!moved) stop = true;  // no later entry of the run can move into this bucket
-      }
-    }
+    const InstDesc d = a.desc[w];  // (a copy: the refill writes memory that may be anything)
+    refill_run(d, a.bitmaps[w], a.dmask[w], sl);
   }
 }
 
+// The whole eviction of an instance whose table the sample covers (up to kEstBuckets buckets), by one
+// CTA: the metas stay in registers from the first histogram to the choice of what goes, which is then
+// listed in shared memory and spread over the threads.  In place of five kernels (8 + 6 + 5 + 8 + 13
+// us, each little more than its latency, for 4 instances of 1,024 buckets; 21 us this one).
+__global__ void __launch_bounds__(kEstThreads) k4_evict_small(EvictArgs a) {
+  constexpr int kPer = kEstBuckets / kEstThreads;
+  __shared__ __align__(16) uint32_t hist[kBins];
+  __shared__ EstPart s_part[kEstThreads / 32];
+  __shared__ uint4 s_v[kRankMax];
+  __shared__ uint32_t s_full[kEstBuckets / 32], s_dmask[kEstBuckets / 8];
+  __shared__ uint16_t s_del[4 * kEstBuckets], s_hole[kEstBuckets];
+  __shared__ unsigned s_cnt, s_ndel, s_nholes;
+  __shared__ unsigned long long s_theta[2];
+  chain_wait();
+  if (block_error(a.err)) return;
+  const int w = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  const long long size = a.size[w];
+  const InstDesc d = a.desc[w];
+  const long long E = size - d.cap;
+  if (E <= 0) return;
+  const uint32_t NB = 1u << d.log2nb;
+  unsigned long long m[4 * kPer];
+  load_metas(d, NB, NB, m);
+  for (int i = tid; i < kEstBuckets / 8; i += kEstThreads) s_dmask[i] = 0;
+  if (tid == 0) s_cnt = s_ndel = s_nholes = 0;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const unsigned bits = __ballot_sync(kFull, m[4 * k] && m[4 * k + 1] && m[4 * k + 2] && m[4 * k + 3]);
+    if (lane == 0) s_full[(tid + k * kEstThreads) >> 5] = bits;
+  }
+  const EstPart all = sample_range(m, s_part);
+  const TickScale ts{32 - __clz(all.arr), 32 - __clz(all.dep)};
+  // the bin of the E-th smallest, then that bin's values over the bins, until it holds a few
+  unsigned long long lo = ts.pack(all.mn);
+  int shift = max(0, 52 - __clzll((long long)(ts.pack(all.mx) - lo)));
+  uint32_t rest = (uint32_t)E, cnt = 0;
+  while (true) {
+    for (int i = tid; i < kBins; i += kEstThreads) hist[i] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 4 * kPer; ++k) {
+      const unsigned long long x = ts.pack(m[k]);
+      if (m[k] && x >= lo && ((x - lo) >> shift) < (unsigned)kBins) atomicAdd(&hist[(uint32_t)((x - lo) >> shift)], 1u);
+    }
+    __syncthreads();
+    uint32_t below;
+    const int bin = find_threshold_bin<kEstThreads>(hist, rest, &below);
+    rest -= below;
+    cnt = hist[bin];
+    lo += (unsigned long long)bin << shift;
+    if (cnt <= (unsigned)kRankMax || shift == 0) break;
+    // (values behind the bin that fall into the next pass's bins come after the target)
+    shift = max(0, shift - 12);
+    __syncthreads();  // hist is cleared again
+  }
+  const unsigned long long hi = lo + (1ull << shift) - 1;
+  // its entries in order of (meta, key): the threshold has rest - 1 of them below it.  (Only
+  // equal ticks, which a commit never writes, can be more than kRankMax; they are ranked from the
+  // work list.)
+  uint4* list = cnt <= (unsigned)kRankMax ? s_v : a.cand_a[w];
+#pragma unroll
+  for (int k = 0; k < 4 * kPer; ++k) {
+    const unsigned long long x = ts.pack(m[k]);
+    if (!m[k] || x < lo || x > hi) continue;
+    const unsigned long long key = d.tab[tid + (k / 4) * kEstThreads].key[k & 3];
+    list[atomicAdd(&s_cnt, 1u)] = make_uint4((uint32_t)m[k], (uint32_t)(m[k] >> 32), (uint32_t)key, (uint32_t)(key >> 32));
+  }
+  __syncthreads();
+  for (unsigned i = tid; i < cnt; i += kEstThreads) {
+    const uint64_t mh = v_hi(list[i]), ml = v_lo(list[i]);
+    uint32_t rank = 0;
+    for (unsigned j = 0; j < cnt; ++j) {
+      const uint64_t oh = v_hi(list[j]), ol = v_lo(list[j]);
+      rank += oh < mh || (oh == mh && ol < ml);
+    }
+    if (rank == rest - 1) {
+      s_theta[0] = mh;
+      s_theta[1] = ml;
+    }
+  }
+  __syncthreads();
+  const unsigned long long tm = s_theta[0], tk = s_theta[1];
+  // deletions: listed by the buckets' owners, then a thread each (an owner's would be a chain of up
+  // to sixteen key reads and global-index lookups)
+  unsigned del = 0;  // bit k: entry m[k]
+#pragma unroll
+  for (int k = 0; k < 4 * kPer; ++k) {
+    if (!m[k] || m[k] > tm) continue;
+    if (m[k] == tm && d.tab[tid + (k / 4) * kEstThreads].key[k & 3] > tk) continue;
+    del |= 1u << k;
+  }
+  const unsigned mine = __popc(del);
+  unsigned incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned v = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += v;
+  }
+  unsigned at = 0;
+  if (lane == 31) at = atomicAdd(&s_ndel, incl);
+  at = __shfl_sync(kFull, at, 31) + incl - mine;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const uint32_t b = tid + k * kEstThreads;
+    const unsigned four = (del >> (4 * k)) & 0xfu;
+    if (!four) continue;
+    atomicOr(&s_dmask[b >> 3], four << (4 * (b & 7)));
+    if ((s_full[b >> 5] >> (b & 31)) & 1u) s_hole[atomicAdd(&s_nholes, 1u)] = (uint16_t)(4 * b + __ffs(four) - 1);
+    for (unsigned left = four; left; left &= left - 1) s_del[at++] = (uint16_t)(4 * b + __ffs(left) - 1);
+  }
+  __syncthreads();
+  const unsigned ndel = s_ndel, nholes = s_nholes;
+  for (unsigned i = tid; i < ndel; i += kEstThreads) {
+    const uint32_t sl = s_del[i];
+    Bucket* B = d.tab + (sl >> 2);
+    if (a.gix.keys && gix_clear(a.gix, B->key[sl & 3], w) < 0) set_error(a.err, MISAT_ERR_INTERNAL);
+    B->key[sl & 3] = kEmpty;
+    B->meta[sl & 3] = 0;
+  }
+  if (tid == 0) {
+    a.size[w] = size - (long long)ndel;
+    atomicAdd(a.evicted, (unsigned long long)ndel);
+  }
+  __syncthreads();
+  // neighbours in the list go to different warps (lanes that walk different runs take turns)
+  for (unsigned i = (tid >> 5) + (kEstThreads / 32) * lane; i < nholes; i += kEstThreads)
+    refill_run(d, s_full, s_dmask, s_hole[i]);
+}
 
 namespace {
 int stream_grid(const EvictArgs& a, int chunks_per_inst, int resident) {
@@ -738,6 +887,12 @@ void launch_evict_select(const EvictArgs& a, int chunks_per_inst, int num_sms, c
   if (W <= num_sms) launch_chained(k4_evict_select<1024>, W, 1024, 0, st, a);
   else launch_chained(k4_evict_select<256>, W, 256, 0, st, a);
   if (marks) cudaEventRecord(marks[2], st);
+}
+
+bool evict_is_small(uint32_t max_log2nb) { return ((uint64_t)1 << max_log2nb) <= (uint64_t)kEstBuckets; }
+
+void launch_evict_small(const EvictArgs& a, cudaStream_t st) {
+  launch_chained(k4_evict_small, a.W, kEstThreads, 0, st, a);
 }
 
 void launch_evict_apply(const EvictArgs& a, int num_sms, cudaStream_t st, const cudaEvent_t* marks) {

@@ -323,7 +323,10 @@ struct EvictArgs {
   int32_t* act;                // [W] instances over capacity (listed by the estimate pass)
   unsigned* n_act;             // entries in act (zeroed by the caller)
 };
-// the eviction's two halves: select (estimate, collect, select; reads the tables only) and apply
+// the whole eviction where no table has more buckets than evict_is_small allows, ...
+bool evict_is_small(uint32_t max_log2nb);
+void launch_evict_small(const EvictArgs& a, cudaStream_t st);
+// ... and its two halves otherwise: select (estimate, collect, select; reads the tables only) and apply
 // (delete, shift; also clears global-index bits)
 // marks (may be NULL): events recorded after each kernel (select: 3, apply: 2), for phase timing
 void launch_evict_select(const EvictArgs& a, int chunks_per_inst, int num_sms, cudaStream_t st,
