@@ -53,14 +53,15 @@ CLOCK_QUERY = ("timestamp,index,clocks.sm,clocks.max.sm,power.draw,clocks_event_
                "clocks_event_reasons.sw_thermal_slowdown,clocks_event_reasons.sw_power_cap")
 
 
-def kernels_per_step(global_index):
-    """Kernels one route+commit launches.  Route: class parameters, prologue, leaders, hash,
-    caps, the block-0 probe (one kernel with the global index; with per-instance tables three:
+def kernels_per_step(global_index, small_tables=False):
+    """Kernels one route+commit launches.  Route: clearing and class parameters, prologue, leaders,
+    hash, caps, the block-0 probe (one kernel with the global index; with per-instance tables three:
     claim of the distinct block-0 keys, their probes, the per-request expansion), probe search,
     the two of the selection (records, deferred acceptance), finalize.
-    Commit: insert dedup, insert work list, insert, the global-index pass (global layout only),
-    sessions, and the five eviction kernels (estimate, collect, select, delete, shift)."""
-    return (10 + 9 + 1) if global_index else (12 + 9)
+    Commit: insert dedup, insert work list and sessions, insert, the global-index pass (global
+    layout only), and the eviction: one kernel where every table is small, else five (estimate,
+    collect, select, delete, shift)."""
+    return (10 if global_index else 12) + 3 + (1 if global_index else 0) + (1 if small_tables else 5)
 
 
 def max_over_ranks(ms, dist, device):
@@ -660,6 +661,8 @@ def run_gb300(args):
     for w in range(sc.W):
         if r.index_size(w) >= int(sc.cap_blocks[w]):
             evict_buckets += r.table_buckets(w)
+    # tables that one kernel evicts (up to 2,048 buckets each)
+    small_tables = max(r.table_buckets(w) for w in range(sc.W)) <= 2048
     ab = algorithmic_bytes(sc, st, mask_words=gidx["mask_words"] if gidx else None,
                            admitted_blocks=admitted_blocks, evict_buckets=evict_buckets,
                            insert_ops=int(st.insert_ops))
@@ -734,7 +737,7 @@ def run_gb300(args):
                 "sequential_h2d_bytes_per_step": h2d_full,
                 "sequential_api": ("misat_route_host + misat_commit on the measured batch from the same state "
                                    "(copy, route, read-back; CUDA events)")},
-        "gpu_launches": kernels_per_step(pidx == misat.PREFIX_GLOBAL) * K,
+        "gpu_launches": kernels_per_step(pidx == misat.PREFIX_GLOBAL, small_tables) * K,
         "roofline": dom_roof,
         "kernels": kernels,
         "prefix_index": args.prefix_index,
