@@ -96,6 +96,7 @@ struct ProbeArgs {
   unsigned long long* stats;         // phase 1: [0] probes, [1] bucket reads
   unsigned long long* stats_search;  // phase 2: [0] probes, [1] bucket reads
   int32_t* err;
+  int32_t rows;                      // requests per warp of the row expansion (set by the launcher)
   GIndex gix;                        // phase 1 reads the global index when gix.keys != NULL
   // per-instance layout: a batch-local index of the distinct block-0 keys (GIndex layout,
   // keys cleared per batch), the list of its claimed slots, the list's length (also the

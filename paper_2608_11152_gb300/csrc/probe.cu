@@ -228,11 +228,11 @@ __global__ void __launch_bounds__(256) k2_probe_search(ProbeArgs a) {
   block_add_stats(a.stats_search, probes, reads);
 }
 
-// Phase 1 through the global index: a warp takes 32 requests, each lane looks up the
-// block-0 key of one of them (one lookup answers every instance) and the masks go to shared
-// memory.  The warp's 32 H rows are one contiguous run of 32W u16 (64W bytes, 16-byte
-// aligned), written as 16-byte stores of eight entries (H = 1 where the bit is set) spread
-// over the lanes; each set bit of a request with at least two blocks also becomes a hit
+// Phase 1 through the global index: a warp takes G = 32 requests (8 where that leaves SMs
+// without a warp), a lane looks up the block-0 key of one of them (one lookup answers every
+// instance) and the masks go to shared memory.  The warp's G H rows are one contiguous run of G W u16
+// (16-byte aligned for both G), written as 16-byte stores of eight entries (H = 1 where the bit is
+// set) spread over the lanes; each set bit of a request with at least two blocks also becomes a hit
 // pair, at its request's base (one atomic per warp) plus the rank of the bit in the mask.
 __global__ void __launch_bounds__(256) k2_probe_first_gix(ProbeArgs a) {
   extern __shared__ unsigned long long s_gm[];  // [warps][32][mw] masks, then [warps][32] (nb, base)
@@ -244,10 +244,11 @@ __global__ void __launch_bounds__(256) k2_probe_first_gix(ProbeArgs a) {
   unsigned long long* sm = s_gm + (size_t)wid * 32 * mw;
   int2* s_nbb = reinterpret_cast<int2*>(s_gm + (size_t)wpb * 32 * mw) + wid * 32;
   unsigned long long probes = 0, reads = 0;
-  const int groups = (a.n + 31) >> 5;
+  const int G = a.rows;
+  const int groups = (a.n + G - 1) / G;
   const int W = a.W;
-  for (int grp = blockIdx.x * wpb + wid; grp < groups; grp += gridDim.x * wpb) {
-    const int r = grp * 32 + lane;
+  for (int grp = wid * gridDim.x + blockIdx.x; grp < groups; grp += gridDim.x * wpb) {
+    const int r = lane < G ? grp * G + lane : a.n;
     int nb = 0;
     int64_t slot = -1;
     if (r < a.n) {
@@ -282,9 +283,9 @@ __global__ void __launch_bounds__(256) k2_probe_first_gix(ProbeArgs a) {
     s_nbb[lane] = make_int2(nb, (int)base);
     __syncwarp();
     // the group's rows: elements e = i*W + w of a run of cnt*W entries
-    const int cnt = min(32, a.n - grp * 32);
+    const int cnt = min(G, a.n - grp * G);
     const int64_t run = (int64_t)cnt * W;
-    uint16_t* rows = a.H + (int64_t)grp * 32 * W;
+    uint16_t* rows = a.H + (int64_t)grp * G * W;
     const int64_t n8 = (run + 7) >> 3;
     if ((W & 7) == 0) {
       // eight entries of one row per chunk: one mask byte gives them all
@@ -312,7 +313,7 @@ __global__ void __launch_bounds__(256) k2_probe_first_gix(ProbeArgs a) {
               rest &= rest - 1;
               const unsigned p = (unsigned)q.y + rank++;
               if ((int64_t)p < a.hits_cap)
-                a.hits[p] = make_int2(grp * 32 + i, w0 + bit);
+                a.hits[p] = make_int2(grp * G + i, w0 + bit);
               else
                 set_error(a.err, MISAT_ERR_TABLE_FULL);
             }
@@ -343,7 +344,7 @@ __global__ void __launch_bounds__(256) k2_probe_first_gix(ProbeArgs a) {
             for (uint32_t j = 0; j < wd; ++j) rank += (unsigned)__popcll(mi[j]);
             const unsigned p = (unsigned)q.y + rank;
             if ((int64_t)p < a.hits_cap)
-              a.hits[p] = make_int2(grp * 32 + i, w);
+              a.hits[p] = make_int2(grp * G + i, w);
             else
               set_error(a.err, MISAT_ERR_TABLE_FULL);
           }
@@ -369,20 +370,24 @@ __global__ void __launch_bounds__(256) k2_probe_first_gix(ProbeArgs a) {
 void launch_probe_first(const ProbeArgs& a, int num_sms, cudaStream_t st) {
   const int64_t total = (int64_t)a.n * a.W;
   if (total <= 0) return;
-  const int groups = (a.n + 31) / 32;
+  ProbeArgs e = a;
+  // rows per warp: 32 once they give every SM eight warps (3,001 requests x 1,000 instances: 94 warps
+  // took 32 us, 376 take 15; 4,096 x 128: 10.5 and 8.1)
+  e.rows = a.n >= 32 * 8 * num_sms ? 32 : 8;
+  const int groups = (a.n + e.rows - 1) / e.rows;
   const int gblocks = (groups + 7) / 8;
   const size_t gsmem = 8 * 32 * ((a.gix.keys ? a.gix.mw : a.fb.mw) * sizeof(unsigned long long) + sizeof(int2));
   const int gres = resident_grid<k2_probe_first_gix>(256, gsmem, num_sms);
   const int ggrid = gblocks < gres ? gblocks : gres;
   if (a.gix.keys) {
-    launch_chained(k2_probe_first_gix, ggrid, 256, gsmem, st, a);
+    launch_chained(k2_probe_first_gix, ggrid, 256, gsmem, st, e);
     return;
   }
   // per-instance tables: the context allocates the batch-local index with the tables
-  launch_chained(k2_first_claim, ggrid, 256, 0, st, a);
+  const int cblocks = (a.n + 255) / 256;
+  launch_chained(k2_first_claim, cblocks < gres ? cblocks : gres, 256, 0, st, a);
   const auto distinct = a.W <= 32 ? k2_probe_distinct<1> : (a.W <= 64 ? k2_probe_distinct<2> : k2_probe_distinct<4>);
   launch_chained(distinct, num_sms * 8, 256, 0, st, a);  // two waves: measured faster than one for this pass
-  ProbeArgs e = a;
   e.gix = a.fb;
   e.stats = a.stats_fb;
   launch_chained(k2_probe_first_gix, ggrid, 256, gsmem, st, e);

@@ -163,3 +163,27 @@ def test_global_index_rebuilds_when_claimed_slots_accumulate():
     assert any(b < a for a, b in zip(claimed_seen, claimed_seen[1:])), \
         f"no rebuild happened (claimed slots {claimed_seen}, {slots} slots)"
     r.close()
+
+
+@pytest.mark.parametrize("n,W", [(7, 5), (9, 65), (38911, 3), (38912, 3), (38915, 9)])
+def test_rows_at_the_edges_of_the_warps_share(n, W):
+    """H rows and hit pairs where a warp's share of the requests changes from 8 to 32 (38,912 requests on
+    152 SMs) and at ragged ends, for both index layouts."""
+    from tests.test_gpu_selection import _batch, _scenario
+
+    rng = np.random.default_rng(n)
+    batches = []
+    for k in range(2):  # the second batch finds the first one's blocks on some instances
+        lens = rng.integers(0, 70, n)
+        batches.append(_batch(rng, rng.integers(0, 3, n), np.arange(1, n + 1) + k * n, lens, shared=40))
+    sc = _scenario(W, [4 * n // W + 64] * W, 3, rng.integers(0, 5, W), rng.integers(1, 4, W), [0] * W, batches)
+    for index in (0, 1):
+        r, o = make_router(sc, max_sessions=4 * n, prefix_index=index), make_oracle(sc)
+        try:
+            for b in batches:
+                route_both(r, o, b, W)
+                for x in (r, o):
+                    x.commit()
+                    x.set_instance_state(np.arange(W, dtype=np.int64)[::-1] * 100, None, None)
+        finally:
+            r.close()
