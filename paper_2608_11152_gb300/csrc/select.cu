@@ -52,7 +52,9 @@ constexpr int kFixed = -3;           // the same, decided for good
 //   [2], [3] = the kTop cheapest of those, (w << 16 | H), by (cost, w)
 // theta is Eq. (7)'s bound: the released leader waits for a full w_hit when the chosen
 // instance's d_w is above theta.  H rows are read 16 bytes at a time, and only of leaders with
-// a cached prefix (one entry at a time took 0.13 ms at 3,001 requests of 1,000 instances).
+// a cached prefix, Ahead pieces in flight (3,001 requests of 1,000 instances: one entry at a time
+// 130 us, one piece 31, four 20; with 64 or 128 instances four are 1 us slower than one).
+template <int Ahead>
 __global__ void __launch_bounds__(256) k3_select_prep(SelectPrepArgs a) {
   __shared__ int s_wc[8];
   chain_wait();
@@ -109,31 +111,40 @@ __global__ void __launch_bounds__(256) k3_select_prep(SelectPrepArgs a) {
     const int lead_in = (int)((reinterpret_cast<uintptr_t>(row) & 15) >> 1);
     const uint4* p = reinterpret_cast<const uint4*>(row - lead_in);
     const int pieces = (lead_in + a.W + 7) >> 3;
-    for (int q = 0; q < pieces; ++q) {
-      const uint4 v = __ldcg(p + q);
-      if ((v.x | v.y | v.z | v.w) == 0) continue;
-      const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+    for (int q0 = 0; q0 < pieces; q0 += Ahead) {
+      uint4 ahead[Ahead];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const uint32_t h = (u[e >> 1] >> (16 * (e & 1))) & 0xffffu;
-        const int w = 8 * q + e - lead_in;
-        if (!h || w < 0 || w >= a.W) continue;
-        if (w != pw && (a.gh[w] <= 0 || a.ch[w * 3 + b] <= 0)) continue;
-        ++nh;
-        const int64_t c = a.backlog[w] + (x - 16 * (int64_t)h) * a.tokcost[w];
-        if (c < cost[kTop - 1]) {  // instances come in index order: equal costs keep it
-          cost[kTop - 1] = c;
-          ent[kTop - 1] = ((uint32_t)w << 16) | h;
+      for (int k = 0; k < Ahead; ++k) ahead[k] = q0 + k < pieces ? __ldcg(p + q0 + k) : make_uint4(0, 0, 0, 0);
+#pragma unroll 1
+      for (int k = 0; k < Ahead; ++k) {
+        const uint4 v = ahead[0];
 #pragma unroll
-          for (int i = kTop - 1; i > 0; --i)
-            if (cost[i] < cost[i - 1]) {
-              const int64_t tcost = cost[i];
-              cost[i] = cost[i - 1];
-              cost[i - 1] = tcost;
-              const uint32_t te = ent[i];
-              ent[i] = ent[i - 1];
-              ent[i - 1] = te;
-            }
+        for (int i = 0; i + 1 < Ahead; ++i) ahead[i] = ahead[i + 1];
+        const int q = q0 + k;
+        if ((v.x | v.y | v.z | v.w) == 0) continue;
+        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const uint32_t h = (u[e >> 1] >> (16 * (e & 1))) & 0xffffu;
+          const int w = 8 * q + e - lead_in;
+          if (!h || w < 0 || w >= a.W) continue;
+          if (w != pw && (a.gh[w] <= 0 || a.ch[w * 3 + b] <= 0)) continue;
+          ++nh;
+          const int64_t c = a.backlog[w] + (x - 16 * (int64_t)h) * a.tokcost[w];
+          if (c < cost[kTop - 1]) {  // instances come in index order: equal costs keep it
+            cost[kTop - 1] = c;
+            ent[kTop - 1] = ((uint32_t)w << 16) | h;
+#pragma unroll
+            for (int i = kTop - 1; i > 0; --i)
+              if (cost[i] < cost[i - 1]) {
+                const int64_t tcost = cost[i];
+                cost[i] = cost[i - 1];
+                cost[i - 1] = tcost;
+                const uint32_t te = ent[i];
+                ent[i] = ent[i - 1];
+                ent[i - 1] = te;
+              }
+          }
         }
       }
     }
@@ -154,7 +165,7 @@ void launch_select_prep(const SelectPrepArgs& a, int num_sms, cudaStream_t st) {
     const int64_t copy = ((int64_t)a.n * a.W + 8191) / 8192;
     grid += (int)(copy < 8 * num_sms ? copy : 8 * num_sms);
   }
-  launch_chained(k3_select_prep, grid, 256, 0, st, a);
+  launch_chained(a.W > 256 ? k3_select_prep<4> : k3_select_prep<1>, grid, 256, 0, st, a);
 }
 
 // ---------------------------------------------------------------------------
