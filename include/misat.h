@@ -364,8 +364,8 @@ int misat_checkpoint_free(misat_checkpoint* ckpt);
 
 /* ---- per-phase device time (measurement; the paper has no counterpart) ----
  * With timing enabled, the route and commit kernels are launched directly (no graph
- * replay, the global-index pass on the context's stream instead of beside the session
- * update) with CUDA events on the context's stream between them.  misat_phase_times waits
+ * replay, the global-index pass on the context's stream instead of beside the eviction's
+ * read-only half) with CUDA events on the context's stream between them.  misat_phase_times waits
  * and writes the durations (ms) of the last route / commit, indexed by MISAT_PHASE_*
  * (MISAT_N_PHASES values). */
 #define MISAT_PHASE_PROLOGUE 0      /* validation, session snapshot, leaders */
@@ -375,9 +375,9 @@ int misat_checkpoint_free(misat_checkpoint* ckpt);
 #define MISAT_PHASE_PROBE_SEARCH 4  /* K2 binary search of the hit pairs */
 #define MISAT_PHASE_SELECT 5        /* K3b placement + K4a admission: the serial selection */
 #define MISAT_PHASE_FINALIZE 6      /* holds, followers, outputs */
-#define MISAT_PHASE_INSERT 7        /* K4b index insert (work list + table inserts) */
-#define MISAT_PHASE_SESSIONS 8      /* session table update */
-#define MISAT_PHASE_EVICT 9         /* K4c eviction, all five kernels */
+#define MISAT_PHASE_INSERT 7        /* K4b index insert (work list, session table update, table inserts) */
+#define MISAT_PHASE_SESSIONS 8      /* nothing of its own: the session update is timed with the insert */
+#define MISAT_PHASE_EVICT 9         /* K4c eviction, all its kernels */
 #define MISAT_PHASE_GIX_INSERT 10   /* global prefix index bits of the new keys (inline while timing) */
 #define MISAT_PHASE_EVICT_ESTIMATE 11
 #define MISAT_PHASE_EVICT_COLLECT 12

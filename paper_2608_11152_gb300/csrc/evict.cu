@@ -786,6 +786,10 @@ __global__ void __launch_bounds__(kEstThreads) k4_evict_small(EvictArgs a) {
     __syncthreads();
     uint32_t below;
     const int bin = find_threshold_bin<kEstThreads>(hist, rest, &below);
+    if (bin < 0) {  // the table holds fewer entries than its size says
+      if (tid == 0) set_error(a.err, MISAT_ERR_INTERNAL);
+      return;
+    }
     rest -= below;
     cnt = hist[bin];
     lo += (unsigned long long)bin << shift;
