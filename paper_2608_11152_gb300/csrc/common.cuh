@@ -166,15 +166,6 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return m;
 }
 
-// Streaming 16-byte read-only load (read once: no L1 allocation, 256-byte L2 prefetch).
-__device__ __forceinline__ int4 ld_stream_v4(const int4* p) {
-  int4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v4.s32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p));
-  return v;
-}
-
 // Read the four keys of a bucket (one 32-byte sector) through the read-only path.
 __device__ __forceinline__ void ld_bucket_keys(const Bucket* b, unsigned long long k[4]) {
   const ulonglong2* p = reinterpret_cast<const ulonglong2*>(b->key);
