@@ -20,7 +20,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmisat.so")
 SOURCES = ["api.cu", "hash.cu", "probe.cu", "route.cu", "select.cu", "commit.cu", "evict.cu", "gindex.cu",
            "overload.cu", "stage.cu"]
-HEADERS = ["common.cuh", "gindex.cuh", "kernels.h"]
+HEADERS = ["common.cuh", "gindex.cuh", "kernels.h", "tick_scale.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

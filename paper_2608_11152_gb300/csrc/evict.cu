@@ -21,13 +21,14 @@
 //                      with backward shifts (no tombstones), one thread per run
 #include "common.cuh"
 #include "kernels.h"
+#include "tick_scale.h"
 
 namespace misat {
 
 namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kEstThreads = 512;
-constexpr int kBins = 4096;
+constexpr int kBins = kTickBins;
 constexpr int kEstBuckets = 2048;  // sampled per instance, four by each thread
 constexpr int kSelSmem = 1024;      // candidates kept in shared memory
 constexpr int kRankMax = 64;        // candidates that are ranked by counting
@@ -92,25 +93,6 @@ __device__ __forceinline__ uint32_t digit128(uint64_t hi, uint64_t lo, int shift
 }
 
 }  // namespace
-
-
-// Metas without the bits that no sample uses (a commit's ticks fill a small part of the span between
-// two sequence numbers): in this order the samples spread over the histogram's bins, while equal bins
-// of the metas themselves held a whole commit each.
-struct TickScale {
-  int ab, db;      // bits of the samples' largest arrival and depth
-  __device__ unsigned long long pack(unsigned long long m) const {
-    const unsigned long long low = (m & 0xffffu), base = 65536ull - (1ull << db);
-    const unsigned long long arr = (m >> 16) & 0xfffffu, top = (1ull << ab) - 1;
-    return ((((m >> 36) << ab) | (arr < top ? arr : top)) << db) | (low > base ? low - base : 0ull);
-  }
-  // the smallest meta that packs to x or more
-  __device__ unsigned long long unpack(unsigned long long x) const {
-    const unsigned long long low = x & ((1ull << db) - 1), arr = (x >> db) & ((1ull << ab) - 1), seq = x >> (db + ab);
-    if (seq >> 28) return ~0ull;
-    return (seq << 36) | (arr << 16) | (low ? low + 65536ull - (1ull << db) : 0ull);
-  }
-};
 
 struct EstPart {
   unsigned long long mn, mx;   // smallest and largest sampled meta
@@ -208,7 +190,7 @@ __global__ void __launch_bounds__(kEstThreads) k4_evict_estimate(EvictArgs a) {
   if (n > 0) {
     // histogram of the samples from their minimum on, bins of 2^shift
     const unsigned long long smin = ts.pack(all.mn);
-    const int shift = max(0, 52 - __clzll((long long)(ts.pack(all.mx) - smin)));
+    const int shift = bin_shift(ts.pack(all.mx) - smin);
 #pragma unroll
     for (int k = 0; k < 4 * kPer; ++k)
       if (m[k]) atomicAdd(&hist[(uint32_t)((ts.pack(m[k]) - smin) >> shift)], 1u);
@@ -399,7 +381,7 @@ __global__ void __launch_bounds__(T) k4_evict_select(EvictArgs a) {
   const int2 sc = a.scale[w];
   const TickScale ts{sc.x, sc.y};
   const unsigned long long plo = ts.pack(a.thr_lo[w]);
-  const int tick_shift = max(0, 52 - __clzll((long long)(ts.pack(a.thr_hi[w]) - plo)));
+  const int tick_shift = bin_shift(ts.pack(a.thr_hi[w]) - plo);
   const uint4* cur = c0;
   for (int iter = 0; iter < 16 && cnt > (unsigned)kRankMax; ++iter) {
     const bool tick = iter == 0 && bracketed && !open;
@@ -446,6 +428,10 @@ __global__ void __launch_bounds__(T) k4_evict_select(EvictArgs a) {
     __syncthreads();
     uint32_t bl;
     const int bin = find_threshold_bin<T>(hist, (uint32_t)Erem, &bl);
+    if (bin < 0) {  // the table holds fewer entries than its size says
+      if (tid == 0) set_error(a.err, MISAT_ERR_INTERNAL);
+      return;
+    }
     Erem -= bl;
     const unsigned kept = hist[bin];
     uint4* nxt = kept <= (unsigned)kRankMax                 ? s_r
@@ -773,7 +759,7 @@ __global__ void __launch_bounds__(kEstThreads) k4_evict_small(EvictArgs a) {
   const TickScale ts{32 - __clz(all.arr), 32 - __clz(all.dep)};
   // the bin of the E-th smallest, then that bin's values over the bins, until it holds a few
   unsigned long long lo = ts.pack(all.mn);
-  int shift = max(0, 52 - __clzll((long long)(ts.pack(all.mx) - lo)));
+  int shift = bin_shift(ts.pack(all.mx) - lo);
   uint32_t rest = (uint32_t)E, cnt = 0;
   while (true) {
     for (int i = tid; i < kBins; i += kEstThreads) hist[i] = 0;

@@ -1,6 +1,7 @@
 """Eviction at the shapes where its selection changes (exact, against the oracle): whole and sampled
 tables, more instances than SMs, a table that stays sparse after it was far over capacity, long prompts
-in one tick, equal ticks that only the key decides, holes in runs of full buckets."""
+in one tick, equal ticks that only the key decides, holes in runs of full buckets, ticks beyond those
+that the sample of a table meets."""
 
 import numpy as np
 import pytest
@@ -68,3 +69,85 @@ def test_equal_ticks_go_by_the_key(n, cap):
             assert np.array_equal(gk, ok_) and np.array_equal(gm, om)
         finally:
             r.close()
+
+
+GOLD = 0x9E3779B97F4A7C15
+BUCKETS_LOG2 = 12  # an instance of 4,097 to 8,192 blocks; its even buckets are the sample
+
+
+def _keys_at_home(rng, odd, taken):
+    """One key per entry of `odd`, home in an odd or an even bucket of the table as it says, at most four
+    to a bucket (so that every entry stays in its home bucket)."""
+    out = np.zeros(len(odd), np.uint64)
+    left = {0: list(np.flatnonzero(~odd)), 1: list(np.flatnonzero(odd))}
+    while left[0] or left[1]:
+        for k in np.unique(rng.integers(2, 1 << 63, size=20000, dtype=np.uint64)).tolist():
+            home = ((k * GOLD) & (2**64 - 1)) >> (64 - BUCKETS_LOG2)
+            todo = left[home & 1]
+            if todo and taken.get(home, 0) < 4:
+                taken[home] = taken.get(home, 0) + 1
+                out[todo.pop()] = k
+    return out
+
+
+def _load_and_compare(keys, metas, cap, index):
+    b = _batch(np.random.default_rng(0), [0], [1], [16])
+    sc = _scenario(1, [cap], 3, [0], [1], [0], [b])
+    r, o = make_router(sc, prefix_index=index), make_oracle(sc)
+    try:
+        assert r.table_buckets(0) == 1 << BUCKETS_LOG2
+        for x in (r, o):
+            x.load_entries(0, keys, metas)
+        gk, gm = r.dump_index(0)
+        ok_, om = o.dump_index(0)
+        assert len(gk) == cap
+        assert np.array_equal(gk, ok_) and np.array_equal(gm, om)
+        assert r.table_buckets(0) == 1 << BUCKETS_LOG2
+    finally:
+        r.close()
+
+
+@pytest.mark.parametrize("index", [0, 1])
+@pytest.mark.parametrize("seed,n", [(0, 16), (1, 32), (2, 32)])
+def test_an_arrival_beyond_the_sampled_ones(seed, n, index):
+    """Eight commits of n requests (a power of two); the second has one more, whose few blocks, the only ones
+    with so large an arrival, all lie in buckets that are not sampled.  The last entry to leave
+    goes over that commit's end, through the larger arrival, and into the next commit."""
+    rng = np.random.default_rng(seed)
+    metas, late = [], []
+    for seq in range(1, 9):
+        for a in range(n + (seq == 2)):
+            depths = int(rng.integers(1, 2 * 1100 // n)) if a < n - 1 else int(rng.integers(20, 40))
+            metas += [(seq << 36) | (a << 16) | (65535 - d) for d in range(depths)]
+            late += [a >= n] * depths
+    metas, late = np.array(metas, np.uint64), np.array(late)
+    keys = _keys_at_home(rng, np.where(late, True, rng.random(len(metas)) < 0.5), {})
+    order = np.sort(metas)
+    first, last = np.searchsorted(order, [(2 << 36) | (n << 16), 3 << 36])  # the larger arrival's entries
+    for E in sorted({first - 60, first - 9, first - 1, first, first + 1, first + 8, last - 1, last, last + 1, last + 30}):
+        _load_and_compare(keys, metas, len(metas) - int(E), index)
+
+
+@pytest.mark.parametrize("index", [0, 1])
+def test_batches_of_changing_size(index):
+    """A commit has a few more requests than a power of two, the ones before and behind it fewer."""
+    rng = np.random.default_rng(5 + index)
+    sizes = [31, 33, 32, 65, 64, 17, 129, 16, 33, 30, 35, 31]
+    W, cap, ses, batches = 2, 4200, iter(range(1, 1 << 20)), []
+    for n in sizes:
+        lens = rng.integers(0, 2 * 6000 * 16 // n, n)
+        lens[-2:] = rng.integers(16, 600, 2)  # few blocks at the largest arrivals
+        batches.append(_batch(rng, rng.integers(0, 3, n), [next(ses) for _ in range(n)], lens))
+    sc = _scenario(W, [cap, cap + 100], 3, np.zeros(W), np.ones(W), np.zeros(W), batches)
+    r, o = make_router(sc, max_sessions=2000, prefix_index=index), make_oracle(sc)
+    try:
+        for k, b in enumerate(batches):
+            back = np.array([0, 40_000]) if k % 2 else np.array([40_000, 0])
+            for x in (r, o):
+                x.set_instance_state(back, None, None)
+            route_both(r, o, b, W, check_H=False, check_keys=False)
+            r.commit()
+            o.commit()
+            compare_state(r, o, W)
+    finally:
+        r.close()
