@@ -367,6 +367,7 @@ __global__ void __launch_bounds__(T) k4_evict_select(EvictArgs a) {
     }
     __syncthreads();
     cnt = s_cnt;
+    __syncthreads();  // the counter is cleared again below
     Erem = E;
     if (tid == 0) {
       a.n_cand[w] = cnt;

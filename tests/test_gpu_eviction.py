@@ -128,6 +128,20 @@ def test_an_arrival_beyond_the_sampled_ones(seed, n, index):
         _load_and_compare(keys, metas, len(metas) - int(E), index)
 
 
+@pytest.mark.parametrize("n", [(6000, 500), (500, 6000)])
+def test_a_sample_that_does_not_represent_the_table(n):
+    """The sampled buckets hold the recent entries and the others the old ones (or few recent ones among
+    many old), so that the bracket misses and the whole table is collected: equal and distinct
+    ticks, thresholds in both parts."""
+    rng = np.random.default_rng(n[0])
+    seq = np.repeat([1, 9], n).astype(np.uint64)
+    metas = (seq << np.uint64(36)) | (rng.integers(0, 50, sum(n)).astype(np.uint64) << np.uint64(16))
+    metas |= np.uint64(65535) - rng.integers(0, 40, sum(n)).astype(np.uint64)
+    keys = _keys_at_home(rng, seq == 1, {})
+    for E in (1, 40, 499, 500, 501, 1000, 1600):
+        _load_and_compare(keys, metas, sum(n) - E, 1)
+
+
 @pytest.mark.parametrize("index", [0, 1])
 def test_batches_of_changing_size(index):
     """A commit has a few more requests than a power of two, the ones before and behind it fewer."""
