@@ -408,11 +408,12 @@ __device__ __forceinline__ int sel_choose(const SelSmem& s, const SelectArgs& a,
     const int64_t cg = y.x + xg * y.y;
     const int64_t bound = cg + slack;  // of this and every later entry
     if (bound > best_c) break;
-    // equal bound: this entry may still win by its index; one behind it could only tie with it by
-    // having the same cost at x_g, and then it has the larger index.  A fast entry is
-    // cheaper than all behind it over the whole cell.
-    const bool last = bound == best_c || (ent & kPriceFast);
     consider(w, cg + dx * y.y);
+    // Entries behind this one that cost as little as the bound have the same cost at x_g, and so a
+    // larger index: at an equal bound they can win only while this one's is below the best's (the
+    // best may be a cached instance with any index).  A fast entry is cheaper than all behind it over
+    // the whole cell.
+    const bool last = (bound == best_c && w >= best_w) || (ent & kPriceFast);
     if (last) break;
   }
   if (best_w >= 0 && ((lx >> 22) & 1u)) {

@@ -1,7 +1,9 @@
 """The selection kernel at the sizes where its shape changes, against the CPU oracle (exact:
 decisions, reasons, caps and protected counts): one CTA and clusters, batches just above a
-shape's limit, several windows, instance counts whose price orders do not fit shared memory, and
-an Eq. (7) leader that has to give a proposal back."""
+shape's limit, several windows, instance counts whose price orders do not fit shared memory, an
+Eq. (7) leader that has to give a proposal back, and ties between a cached instance and others."""
+
+import itertools
 
 import numpy as np
 import pytest
@@ -106,5 +108,66 @@ def test_a_leader_that_must_wait_gives_its_proposal_back(tail):
         for x in (r, o):
             x.commit()
         compare_state(r, o, W)
+    finally:
+        r.close()
+
+
+def _load(x, prompts, inst):
+    """Makes the full blocks of prompts[i] resident on instance inst[i]."""
+    off = np.concatenate([[0], np.cumsum([len(p) for p in prompts])]).astype(np.int64)
+    n = len(prompts)
+    x.load_chains(off, np.concatenate(prompts).astype(np.int32), np.asarray(inst, np.int32), np.zeros(n, np.uint64),
+                  np.arange(n, dtype=np.uint32), np.full(n, 1 << 16, np.int32))
+
+
+@pytest.mark.parametrize("slow,cheap,cached", list(itertools.permutations(range(3))))
+def test_a_tie_with_a_cached_instance_goes_to_the_lower_index(slow, cheap, cached):
+    """At the start of its price cell (992 tokens) `slow` and `cheap` cost the same; 8 tokens on, `cheap`
+    costs what `cached` does with its 400 tokens, and `slow` 16 more."""
+    rng = np.random.default_rng(1)
+    back, cost = np.zeros(3, np.int64), np.zeros(3, np.int64)
+    back[slow], cost[slow] = 3016, 7
+    back[cheap], cost[cheap] = 5000, 5
+    back[cached], cost[cached] = 6400, 6
+    b = _batch(rng, [0], [1], [1000])
+    sc = _scenario(3, [1000] * 3, 3, back, cost, [0] * 3, [b])
+    r, o = make_router(sc), make_oracle(sc)
+    try:
+        for x in (r, o):
+            _load(x, [b.tokens[:400]], [cached])
+        out = route_both(r, o, b, 3)
+        assert int(out["inst"][0]) == min(cheap, cached)
+    finally:
+        r.close()
+
+
+def _tie_costs(rng, W, length, hits):
+    """(d_w, 1/mu_w): most instances without a cached prefix cost the same at the start of the prompt's
+    price cell, and the cheapest a token of them what one or two cached ones do with their prefix."""
+    start = length >> (length.bit_length() - 5) << (length.bit_length() - 5)
+    cost = rng.integers(2, 7, W)
+    back = np.where(hits > 0, 40 * length - (length - 16 * hits) * cost,
+                    40 * length - (length - start) * cost.min() - start * cost)
+    return back + np.where(rng.random(W) < np.where(hits > 0, 1 - 2 / W, 0.2), rng.integers(1, 20, W), 0), cost
+
+
+@pytest.mark.parametrize("W,mode,length", [(6, 3, 47), (20, 3, 70), (20, 0, 1000), (200, 2, 1000), (1000, 3, 5003)])
+def test_ties_between_cached_and_other_instances(W, mode, length):
+    rng = np.random.default_rng(W + length)
+    n = 300 if mode == 3 else 30 * W  # more than the instances take
+    b = _batch(rng, rng.integers(0, 3, n), np.arange(1, n + 1), np.full(n, length), shared=length)
+    hits = np.where(rng.random(W) < 0.4, rng.integers(1, length // 16 + 1, W), 0)
+    sc = _scenario(W, [1000 if mode == 3 else 100] * W, mode, np.zeros(W), np.ones(W), rng.integers(0, 2, W), [b])
+    r, o = make_router(sc), make_oracle(sc)
+    try:
+        on = np.flatnonzero(hits)
+        for x in (r, o):
+            for at in np.array_split(on, -(-len(on) // 100)):
+                _load(x, [b.tokens[:16 * h] for h in hits[at]], at)
+        for _ in range(12):
+            back, cost = _tie_costs(rng, W, length, hits)
+            for x in (r, o):
+                x.set_instance_state(back, cost, None)
+            route_both(r, o, b, W)
     finally:
         r.close()
