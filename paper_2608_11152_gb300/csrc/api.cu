@@ -724,12 +724,17 @@ void enqueue_route(misat_ctx* c, const misat_batch* b, misat_decisions* out, cud
   launch_probe_search(pr, c->num_sms, st);
   c->mark(5, st);
 
+  // the caller's H is written beside the records; a buffer at an odd address, where two-byte stores
+  // would fault, by a copy
+  const bool odd_H = (reinterpret_cast<uintptr_t>(b->out_H) & 1) != 0;
+  if (odd_H) cudaMemcpyAsync(b->out_H, c->d_H, (size_t)n * c->W * sizeof(uint16_t), cudaMemcpyDeviceToDevice, st);
+
   SelectPrepArgs sp{};
   sp.n = n;
   sp.W = c->W;
   sp.rq = c->rq;
   sp.H = c->d_H;
-  sp.out_H = reinterpret_cast<uint16_t*>(b->out_H);
+  sp.out_H = odd_H ? nullptr : b->out_H;
   sp.backlog = c->d_backlog;
   sp.tokcost = c->d_tokcost;
   sp.gh = c->ia.gh;

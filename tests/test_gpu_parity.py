@@ -522,6 +522,33 @@ def test_all_four_modes_on_config1():
         r.close()
 
 
+@pytest.mark.parametrize("offset", [0, 1, 2, 3, 15, 16])
+def test_H_is_written_at_any_address(offset):
+    """The caller's H buffer at every alignment, odd addresses among them, launched and replayed; the
+    bytes around it stay as they are."""
+    sc = wl.config1()
+    r, o = make_router(sc), make_oracle(sc)
+    try:
+        for b, _ in sc.warm:
+            route_both(r, o, b, sc.W)
+            r.commit()
+            o.commit()
+        b, W = sc.batch, sc.W
+        db, out = r.device_batch(b), r.alloc_decisions(b.n)
+        size = 2 * b.n * W
+        o.route(b.cls, b.session, b.tok_off, b.tokens)
+        assert o.H().any()
+        buf = torch.empty(size + 64, dtype=torch.uint8, device="cuda")
+        for _ in range(4):
+            buf.fill_(0xA5)
+            r.route(db, out=out, out_H=buf[offset:])
+            got = buf.cpu().numpy()
+            assert np.array_equal(got[offset:offset + size].copy().view(np.uint16).reshape(b.n, W), o.H())
+            assert (got[:offset] == 0xA5).all() and (got[offset + size:] == 0xA5).all()
+    finally:
+        r.close()
+
+
 @pytest.mark.parametrize("seed,W", [(0, 64), (1, 300), (2, 37), (3, 5)])
 def test_serial_selection_many_windows_and_fills(seed, W):
     """Batches of a few thousand leaders (several selection windows) against small caps, so
