@@ -529,11 +529,10 @@ def test_H_is_written_at_any_address(offset):
     sc = wl.config1()
     r, o = make_router(sc), make_oracle(sc)
     try:
-        for b, _ in sc.warm:
-            route_both(r, o, b, sc.W)
-            r.commit()
-            o.commit()
         b, W = sc.batch, sc.W
+        route_both(r, o, b, W)  # its admitted prompts are resident from here on
+        r.commit()
+        o.commit()
         db, out = r.device_batch(b), r.alloc_decisions(b.n)
         size = 2 * b.n * W
         o.route(b.cls, b.session, b.tok_off, b.tokens)
