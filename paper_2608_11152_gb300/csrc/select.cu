@@ -850,17 +850,16 @@ __global__ void __launch_bounds__(1024, 1) k4_select(SelectArgs a, int cs) {
 
 namespace {
 
-// CTAs and threads of the selection cluster for a batch of n requests: one CTA while the
-// leaders fit it (its barriers are block barriers), then as many CTAs as a cluster takes with
-// as few threads as hold the batch (a round's choices share an SM's issue slots), then windows
-// of 16 x 1024.
-void select_shape(int n, int max_cs, int* cs, int* threads) {
-  *cs = 1;
-  if (n <= 1024) {
-    *threads = n <= 256 ? 256 : (n <= 512 ? 512 : 1024);
-    return;
-  }
-  *cs = max_cs;
+// CTAs and threads of the selection cluster for a batch of n requests and W instances.  One CTA, with
+// block barriers, for small batches of few instances; else the whole cluster, whose warps share the
+// instances' thresholds, with as few threads as hold the batch (a round's choices share an SM's
+// issue slots), then windows of 16 x 1024.  A route in us by one CTA and by 16 of 256 threads:
+// 4 instances 76/84 at 256 requests, 16 instances 121/133 at 512 and 133/123 at 1,000; 32
+// instances 197/173 at 256; 64 332/269 at 1,000; 512 563/244 at 256; 1,000 981/465 at 512.
+// (Windows of 16 x 512 suit batches without cached prefixes, 16,384 requests of 64 instances
+// 391/355, but not the steady loop: 65,536 of 128 instances 992/1,099.)
+void select_shape(int n, int W, int max_cs, int* cs, int* threads) {
+  *cs = n <= 512 && W < 32 ? 1 : max_cs;
   *threads = 256;
   while (*threads < 1024 && *cs * *threads < n) *threads <<= 1;
 }
@@ -896,7 +895,7 @@ cudaError_t select_configure(int* max_cluster) {
 void launch_select(const SelectArgs& a, int max_cluster, cudaStream_t st) {
   if (a.n <= 0) return;
   int cs, threads;
-  select_shape(a.n, max_cluster, &cs, &threads);
+  select_shape(a.n, a.W, max_cluster, &cs, &threads);
   cudaLaunchAttribute at[2] = {};
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = cs;

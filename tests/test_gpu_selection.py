@@ -45,7 +45,8 @@ def _scenario(W, cap, mode, backlog, tokcost, contraction, batches, hold=0):
 
 
 @pytest.mark.parametrize("n,W,mode", [
-    (256, 40, 0), (257, 40, 1), (1024, 7, 2), (1025, 33, 0),   # one CTA; the smallest cluster
+    (256, 7, 0), (257, 7, 1), (512, 31, 0),                    # one CTA of 256 and 512 threads
+    (513, 31, 1), (33, 32, 2), (1, 40, 0), (256, 40, 0), (257, 40, 1), (1024, 7, 2), (1025, 33, 0),  # clusters
     (4096, 100, 2), (4097, 100, 0), (8193, 64, 1),             # 256, 512 and 1024 threads a CTA
     (16500, 12, 0), (40000, 24, 2),                            # two and three windows
     (3000, 1000, 0), (9000, 513, 2),                           # price orders read from global memory
