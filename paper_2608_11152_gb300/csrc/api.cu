@@ -1026,7 +1026,9 @@ int misat_route(misat_ctx* c, const misat_batch* b, misat_decisions* out) {
   CK(cudaGetLastError());
   if (n == 0) {
     // the caps of an empty batch are still defined (no candidate sessions)
-    launch_caps(caps_args(c), st);
+    CapsArgs ca = caps_args(c);
+    ca.orders = nullptr;
+    launch_caps(ca, st);
     CK(cudaGetLastError());
     CK(enqueue_meta(c));
     c->routed = true;

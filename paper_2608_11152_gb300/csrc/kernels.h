@@ -147,7 +147,7 @@ struct CapsArgs {
   InstArrays ia;
   const int64_t* backlog;      // [W] d_w
   const int64_t* tokcost;      // [W] 1/mu_w
-  uint16_t* orders;            // [kPriceCells][stride] out: price orders of the selection
+  uint16_t* orders;            // [kPriceCells][stride] out: price orders of the selection (NULL: none)
   const int32_t* err;
 };
 void launch_caps(const CapsArgs& a, cudaStream_t st);  // caps and price orders

@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(1024) k3_caps(CapsArgs a) {
 }
 
 void launch_caps(const CapsArgs& a, cudaStream_t st) {
-  launch_chained(k3_caps, 1 + price_order_blocks(a.W), 1024, 0, st, a);
+  launch_chained(k3_caps, 1 + (a.orders ? price_order_blocks(a.W) : 0), 1024, 0, st, a);
 }
 
 // Clears a route's scratch (one kernel where eight memsets took 1.5 us each).  Launched without
