@@ -762,7 +762,7 @@ def run_gb300(args):
                   "query_tokens": st.query_tokens, "dtv_ppm": st.dtv_ppm,
                   "admitted_blocks": admitted_blocks, "insert_key_ops": int(st.insert_ops),
                   "first_block_keys": int(st.first_block_keys),
-                  "selection_path": "joint" if int(st.joint_selection) else "per-class"},
+                  "global_headroom_ran_out": bool(st.joint_selection)},
     }
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         base = setup_oracle(sc)

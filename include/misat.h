@@ -149,8 +149,7 @@ typedef struct misat_batch_stats {
                                     admitted requests, less the leading blocks that a later request
                                     of the same instance inserts with the same keys */
   int64_t joint_selection;       /* 1 if some instance ran out of global headroom during the last
-                                    route, so its leaders were decided by the joint chain over all
-                                    classes; 0 if the per-class chains decided them */
+                                    route, so that its leaders' classes met in one quota; else 0 */
   int64_t first_block_keys;      /* per-instance layout: distinct block-0 keys of the last route
                                     (each probed once per instance); 0 with the global index */
   int64_t first_block_lookups;   /* per-instance layout: lookups of the requests' block-0 keys in
@@ -395,8 +394,8 @@ int misat_phase_times(misat_ctx* ctx, float* ms_out);
  * memory-accounting scope where device allocations are not allowed.  It writes the same
  * chained 16-token block keys as misat_route, in request order (request 0's full blocks,
  * then request 1's, ... -- the layout of misat_dump_keys), and allocates nothing: its
- * scratch (per-request key offsets, a work counter, an error word) is a fixed array of
- * about 513 KiB inside this library, held by every GPU that loads it until exit.
+ * scratch (key offsets, the list of longer prompts, counters, an error word) is a fixed array
+ * of about 512 KiB inside this library, held by every GPU that loads it until exit.
  *   tok_off   device [n+1], as in misat_batch
  *   tokens    device [n_tokens], 16-byte aligned, readable to the next 16-byte boundary
  *   keys_out  device [keys_cap] u64
@@ -463,7 +462,7 @@ int misat_recheck_delays(int32_t n, const uint64_t* group, const uint8_t* held, 
 /* Wait for the stream and return the sticky device error (0 if none), then clear it and
  * drop any pending route.  A batch rejected on the device changes no persistent state;
  * after TABLE_FULL during a commit the index of the affected instance may hold part of
- * that commit's blocks.  [sync] */
+ * that commit's blocks, and the sessions that it admits may be protected already.  [sync] */
 int misat_sync(misat_ctx* ctx);
 
 /* Static description of an error code. */

@@ -1,14 +1,13 @@
-// Commit kernels (K4b, K4c): index insert, session table update, completions,
-// eviction down to capacity, table growth.
+// Commit kernels (K4b): index insert, session table update, completions, removals
+// announced by the engine, table growth, and the copies of a checkpoint restore.
 //
 // Index tables are bucketed linear-probing hash sets (4 keys per 32-byte sector).
 // Insert claims only empty slots with a CAS, so two threads inserting the same new
 // key always meet in the same slot (no duplicates) and an existing key is found by
 // every later inserter; the tick is merged with atomicMax (Sec. 4.4 reading: LRU).
-// Eviction never leaves tombstones: the exact eviction threshold theta (the E-th
-// smallest (meta, key)) is found by a per-instance radix select, then every run of
-// full buckets is compacted by one thread with backward shifts, so lookups keep
-// stopping at the first bucket with a free slot.
+// Eviction (evict.cu) never leaves tombstones: the holes that it makes in runs of full
+// buckets are refilled by backward shifts, so lookups keep stopping at the first bucket
+// with a free slot.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -534,7 +533,6 @@ void launch_mark_evict(const MarkArgs& a, int32_t w, const EvictArgs& ev, cudaSt
   launch_compact_marked(ev, st);
 }
 
-// Growth: re-insert every entry of `from` into the empty, larger table `to`.
 // Copy list: CTAs take spans of kSpan units of the flattened list; the item holding a span's
 // first unit is found by a (uniform) binary search, later items by stepping forward.
 __global__ void __launch_bounds__(256) k_copy_list(const __grid_constant__ CopyList L) {
@@ -577,6 +575,7 @@ void launch_copy_list(const CopyList& l, int num_sms, cudaStream_t st) {
   k_copy_list<<<grid, 256, 0, st>>>(l);
 }
 
+// Growth: re-insert every entry of `from` into the empty, larger table `to`.
 __global__ void __launch_bounds__(256) k_rehash(RehashArgs a) {
   const uint32_t NB = 1u << a.from.log2nb;
   for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < NB; b += gridDim.x * blockDim.x) {

@@ -25,8 +25,9 @@ struct GIndex {
   unsigned long long* used;   // claimed slots
 };
 
-// Slot of `key`, or -1.  Only for phases without concurrent claims.  Adds buckets read.  (Through
-// L2: an earlier kernel of the same chain may have claimed the slots.)
+// Slot of `key`, or -1.  Adds buckets read.  Reads through L2: an earlier kernel of the same chain, or
+// other threads of this one, may have claimed slots.  Claims only fill slots, so a key that was there
+// before the kernel is found whatever they do; one that is claimed meanwhile may be missed.
 __device__ __forceinline__ int64_t gix_find(const GIndex& g, uint64_t key, uint32_t* reads) {
   const uint32_t mask = (1u << g.log2nb) - 1;
   uint32_t b = home_bucket(key, g.log2nb);
@@ -34,23 +35,6 @@ __device__ __forceinline__ int64_t gix_find(const GIndex& g, uint64_t key, uint3
     const ulonglong2* p = reinterpret_cast<const ulonglong2*>(g.keys + 4 * (size_t)b);
     const ulonglong2 x = __ldcg(p), y = __ldcg(p + 1);
     *reads += 1;
-    if (x.x == key) return 4 * (int64_t)b;
-    if (x.y == key) return 4 * (int64_t)b + 1;
-    if (y.x == key) return 4 * (int64_t)b + 2;
-    if (y.y == key) return 4 * (int64_t)b + 3;
-    if (x.x == kEmpty || x.y == kEmpty || y.x == kEmpty || y.y == kEmpty) return -1;
-    b = (b + 1) & mask;
-  }
-  return -1;
-}
-
-// Slot of `key` while other threads may claim slots (their claims are only additions).
-__device__ __forceinline__ int64_t gix_find_cg(const GIndex& g, uint64_t key) {
-  const uint32_t mask = (1u << g.log2nb) - 1;
-  uint32_t b = home_bucket(key, g.log2nb);
-  for (uint32_t it = 0; it <= mask; ++it) {
-    const ulonglong2* p = reinterpret_cast<const ulonglong2*>(g.keys + 4 * (size_t)b);
-    const ulonglong2 x = __ldcg(p), y = __ldcg(p + 1);
     if (x.x == key) return 4 * (int64_t)b;
     if (x.y == key) return 4 * (int64_t)b + 1;
     if (y.x == key) return 4 * (int64_t)b + 2;
@@ -129,7 +113,8 @@ __device__ __forceinline__ int64_t gix_claim(const GIndex& g, uint64_t key, bool
 // Clear bit w of `key`.  Returns 0, or -1 if the key is not in the index (an index that
 // no longer mirrors the tables).
 __device__ __forceinline__ int gix_clear(const GIndex& g, uint64_t key, int w) {
-  const int64_t s = gix_find_cg(g, key);
+  uint32_t reads = 0;
+  const int64_t s = gix_find(g, key, &reads);
   if (s < 0) return -1;
   atomicAnd(g.masks + (size_t)s * g.mw + (w >> 6), ~(1ull << (w & 63)));
   return 0;

@@ -375,10 +375,10 @@ void launch_block_hash(HashArgs a, int num_sms, cudaStream_t st) {
 // fail, or fragment and shrink that pool), or a hook that runs inside another
 // framework's allocator or memory-accounting scope, where new device allocations are
 // not allowed.  misat_block_hash_noalloc serves them: it computes the same chained
-// block keys as the routing path and allocates nothing.  Its only scratch -- the
-// per-request key offsets, a work counter and an error word -- lives in the
+// block keys as the routing path and allocates nothing.  Its only scratch -- key
+// offsets, the list of longer prompts, counters and an error word -- lives in the
 // file-scope array below, which every GPU that loads this library holds
-// (about 513 KiB) until the process exits.
+// (about 512 KiB) until the process exits.
 
 // scratch layout in 8-byte words: [0] error word | [1..3] counters of the hash | [8..39] blocks
 // per tile of requests (32-bit) | [40 ..] key offsets within the tile, then the list of longer

@@ -19,7 +19,7 @@
 // thresholds only fall, so a choice stays right until its threshold passes it.  After r
 // rounds the r earliest events (an instance running out) are exact, so there are at most
 // 4 W + 1 rounds, and a round takes in every event whose proposers are already settled: 15
-// to 70 rounds for batches in which the serial chain has 100 to 500 events.
+// to 70 rounds a window for batches in which the serial chain has 100 to 500 events.
 //
 // Eq. (7) breaks the scheme in one way: a released continuation that proposes to w while
 // its cached instance w_hit has headroom may have to wait instead once w_hit is full, which
@@ -181,8 +181,9 @@ void launch_select_prep(const SelectPrepArgs& a, int num_sms, cudaStream_t st) {
 //      one over the words of the CTA it ends in give the new threshold, which is written into
 //      every CTA;                                                           cluster barrier
 //   3. leaders whose proposal lies behind its threshold are refused.
-// What bounds it: the instruction latency of one warp through steps 1 and 2 (about 1,000 and
-// 1,500 cycles) and the barriers (500 to 700 cycles each); the SMs are mostly idle.
+// What bounds it: latency.  A round of 16 CTAs at 128 instances takes 9,000 to 10,000 cycles: 2,000 to
+// 2,700 for the choices and about 2,000 for the thresholds of an ordinary CTA, and after each 2,000 to
+// 4,000 until the slowest CTA has reached the barrier.  The SMs are mostly idle.
 namespace {
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }

@@ -551,9 +551,8 @@ def test_H_is_written_at_any_address(offset):
 @pytest.mark.parametrize("seed,W", [(0, 64), (1, 300), (2, 37), (3, 5)])
 def test_serial_selection_many_windows_and_fills(seed, W):
     """Batches of a few thousand leaders (several selection windows) against small caps, so
-    that instances run out of global and class headroom inside windows and envelopes lose
-    many lines; released sessions make Eq. (7) leaders.  Decisions, caps and committed state
-    equal the oracle's after every batch."""
+    that instances run out of global and class headroom inside windows; released sessions make
+    Eq. (7) leaders.  Decisions, caps and committed state equal the oracle's after every batch."""
     sc = wl.small_random(9100 + seed, W=W, cap=200, n=3000, mode=seed % 2, n_warm=3)
     r, o = make_router(sc), make_oracle(sc)
     rng = np.random.default_rng(seed)
@@ -581,10 +580,10 @@ def test_serial_selection_many_windows_and_fills(seed, W):
 
 
 def test_per_class_and_joint_selection_paths_match_the_oracle():
-    """While no instance runs out of global headroom, the per-class chains decide a batch;
-    otherwise the joint chain over all classes decides it again.  Across these scenarios both
-    paths decide some batches (session admission, which has no class caps, makes the global cap
-    bind), and every batch equals the oracle's decisions and committed state."""
+    """Batches in which no instance runs out of global headroom, so that only the class quotas bind, and
+    batches in which one does (session admission, which has no class caps, makes the global cap
+    bind): the statistics tell them apart, both occur across these scenarios, and every batch equals
+    the oracle's decisions and committed state."""
     seen = {0: 0, 1: 0}
     for seed in range(12):
         rng = np.random.default_rng(300 + seed)
