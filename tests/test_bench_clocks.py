@@ -60,16 +60,20 @@ def test_profiled_figures_are_read_only_while_the_sources_match(tmp_path):
     assert bench.profiled_fields(str(summ), (str(src),)) == {}
 
 
-def test_selection_traffic_is_reported_for_the_captured_workload_only():
-    """The per-class selection's DRAM bytes were captured on the stress batch (65,536 requests,
-    128 instances): another workload gets no figure."""
-    import os
-
-    f = bench.profiled_fields(bench.SELECT_PROFILE, bench.SELECT_SOURCES)
-    if not f:  # the kernel changed since the capture: nothing is reported at all
-        assert bench.profiled_select_traffic(65536, 128) is None
-        return
-    assert bench.profiled_select_traffic(65536, 128) == int(f["traffic_bytes_per_launch"])
+def test_selection_traffic_is_reported_for_the_captured_workload_only(tmp_path, monkeypatch):
+    """The selection's DRAM bytes belong to the captured batch and instance count, and to the sources they
+    were captured with: anything else gets no figure."""
+    src = tmp_path / "k.cu"
+    src.write_text("__global__ void k() {}\n")
+    summ = tmp_path / "k.md"
+    summ.write_text("# ncu\n\n- `traffic_bytes_per_launch`: `3450000`\n- `batch_requests`: `65536`\n- `instances`: `128`\n"
+                    f"- `sources_sha256`: `{bench.hash_sources_sha256((str(src),))}`\n")
+    monkeypatch.setattr(bench, "SELECT_SOURCES", (str(src),))
+    monkeypatch.setattr(bench, "SELECT_PROFILE", str(summ))
+    assert bench.profiled_select_traffic(65536, 128) == 3450000
     assert bench.profiled_select_traffic(4096, 128) is None
     assert bench.profiled_select_traffic(65536, 64) is None
-    assert os.path.exists(bench.SELECT_PROFILE)
+    src.write_text("__global__ void k(int) {}\n")
+    assert bench.profiled_select_traffic(65536, 128) is None
+    monkeypatch.setattr(bench, "SELECT_PROFILE", str(tmp_path / "absent.md"))
+    assert bench.profiled_select_traffic(65536, 128) is None
