@@ -785,7 +785,6 @@ __global__ void __launch_bounds__(kEstThreads) k4_evict_small(EvictArgs a) {
     shift = max(0, shift - 12);
     __syncthreads();  // hist is cleared again
   }
-  const unsigned long long hi = lo + (1ull << shift) - 1;
   // its entries in order of (meta, key): the threshold has rest - 1 of them below it.  (Only
   // equal ticks, which a commit never writes, can be more than kRankMax; they are ranked from the
   // work list.)
@@ -793,7 +792,7 @@ __global__ void __launch_bounds__(kEstThreads) k4_evict_small(EvictArgs a) {
 #pragma unroll
   for (int k = 0; k < 4 * kPer; ++k) {
     const unsigned long long x = ts.pack(m[k]);
-    if (!m[k] || x < lo || x > hi) continue;
+    if (!m[k] || x < lo || (x - lo) >> shift) continue;  // (the bin may end beyond 64 bits)
     const unsigned long long key = d.tab[tid + (k / 4) * kEstThreads].key[k & 3];
     list[atomicAdd(&s_cnt, 1u)] = make_uint4((uint32_t)m[k], (uint32_t)(m[k] >> 32), (uint32_t)key, (uint32_t)(key >> 32));
   }

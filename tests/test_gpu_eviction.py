@@ -71,6 +71,30 @@ def test_equal_ticks_go_by_the_key(n, cap):
             r.close()
 
 
+@pytest.mark.parametrize("n,cap", [(9, 5), (600, 64), (600, 599), (3000, 2100), (7000, 4200)])
+def test_the_largest_ticks(n, cap):
+    """Sequence numbers, arrivals and depths up to the limits of their fields, in whole and in sampled
+    tables, with the last entry to leave among the smallest, the middle and the largest."""
+    rng = np.random.default_rng(n + cap)
+    keys = np.unique(rng.integers(2, 1 << 63, size=n, dtype=np.uint64))
+    b = _batch(rng, [0], [1], [16])
+    sc = _scenario(1, [cap], 3, [0], [1], [0], [b])
+    for old in (0.05, 0.5, 0.95):  # share of small sequence numbers
+        seq = np.where(rng.random(len(keys)) < old, rng.integers(0, 3, len(keys)), (1 << 28) - 1 - rng.integers(0, 3, len(keys)))
+        arr = rng.choice([0, 1, 77, 1 << 19, (1 << 20) - 1], len(keys))
+        metas = seq.astype(np.uint64) << np.uint64(36) | arr.astype(np.uint64) << np.uint64(16)
+        metas |= np.uint64(65535) - rng.choice([0, 1, 300, 65534], len(keys)).astype(np.uint64)
+        r, o = make_router(sc), make_oracle(sc)
+        try:
+            for x in (r, o):
+                x.load_entries(0, keys, metas)
+            gk, gm = r.dump_index(0)
+            ok_, om = o.dump_index(0)
+            assert np.array_equal(gk, ok_) and np.array_equal(gm, om)
+        finally:
+            r.close()
+
+
 GOLD = 0x9E3779B97F4A7C15
 BUCKETS_LOG2 = 12  # an instance of 4,097 to 8,192 blocks; its even buckets are the sample
 
